@@ -93,6 +93,38 @@ int device_sms() {
   return cached;
 }
 
+// The fixed-point constants of exp_fix, in integer arithmetic (the same on
+// every host).  The exponent v = R2 c, c = log2(e) inv8 2^-2k, of squares R2
+// up to the cutoff's (or 746 / (inv8 2^-2k), beyond which exp underflows) gets
+// eib integer bits (2^(eib - 1) > v) and 64 - eib fraction bits; the square is
+// shifted left to full 64 bits, so v = hi64((R2 << eq) ec).
+void exp_constants(Dev& d) {
+  constexpr unsigned long long kLog2e = 0xB8AA3B295C17F0BCull;  // log2(e) 2^63
+  const double a = d.inv8 * d.scale * d.scale;
+  const unsigned long long S2 = (unsigned long long)d.S * (unsigned long long)d.S;
+  const double lim = 746.0 / a;
+  const unsigned long long R = lim < (double)S2 ? (unsigned long long)lim : S2;
+  d.emax = R;
+  d.ec = 0;
+  d.eq = 0;
+  d.eib = 1;
+  if (R == 0) return;  // only coincident pairs have a weight: 1
+  while ((R >> (63 - d.eq)) == 0) ++d.eq;
+  const double vmax = (double)R * a * 1.4426950408889634 * (1.0 + 1e-9);
+  while (std::ldexp(1.0, d.eib - 1) <= vmax) ++d.eib;
+  int e = 0;
+  const unsigned long long mant = (unsigned long long)std::ldexp(std::frexp(d.inv8, &e), 53);
+  // ec = mant 2^(e - 53 - 2k) kLog2e 2^-63 2^(128 - eib - eq)
+  const unsigned __int128 P = (unsigned __int128)mant * kLog2e;
+  int se = 0;
+  std::frexp(d.scale, &se);  // scale = 2^(se - 1)
+  const int sh = e - 53 + 2 * (se - 1) - 63 + 128 - d.eib - d.eq;
+  if (sh >= 0)
+    d.ec = (unsigned long long)(P << sh);
+  else if (sh > -128)
+    d.ec = (unsigned long long)((P + ((unsigned __int128)1 << (-sh - 1))) >> -sh);
+}
+
 int ceil_log2(long long v) {  // smallest c with 2^c >= v (v >= 1)
   int c = 0;
   while (c < 62 && (1LL << c) < v) ++c;
@@ -830,7 +862,7 @@ mt_status mt_batch_create(const mt_params* p, const mt_batch* b, void* workspace
   d.inv8 = 1.0 / (8.0 * D.p.D_mt * D.p.dt);
   d.scale = std::ldexp(1.0, -D.p.frac_bits);
   d.inv8f = (float)(d.inv8 * d.scale * d.scale);
-  d.inv8s = std::ldexp(d.inv8, -2 * D.p.frac_bits);
+  exp_constants(d);
   d.key0 = (unsigned int)(D.p.seed & 0xffffffffu);
   d.key1 = (unsigned int)(D.p.seed >> 32);
   d.real = (unsigned int)D.p.realisation;

@@ -180,11 +180,16 @@ struct StepState {
   int xc, mc, sc;             // current X / id, mass and segment buffers
   unsigned long long step;    // steps completed
   const float* noise;         // injected normals or null
+  const unsigned long long* tab;  // the CTA's copy of the binary64 weights' table
 };
 
-__device__ __forceinline__ StepState step_state(const Dev& d) {
+// Called by every thread of a kernel of NT threads; s_tab is visible after
+// the kernel's first barrier.
+template <int PR, int NT>
+__device__ __forceinline__ StepState step_state(const Dev& d, unsigned long long* s_tab) {
   const Ctrl* c = d.ctrl;
-  return {c->xcur, c->mcur, c->scur, c->step, c->noise};
+  if (!mixw(PR)) exp_table<NT>(s_tab);
+  return {c->xcur, c->mcur, c->scur, c->step, c->noise, s_tab};
 }
 
 // The next segment's staged slots [a0, a0 + L) (positions, ids, both mass
@@ -385,7 +390,7 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
   for (int q = tid; q < np; q += NT) {
     const int jj = own[q];
     const int j = olo + jj, k = j + 1 + (q - pfx[jj]);
-    sw[q] = W::near(d, sx[k] - sx[j]);
+    sw[q] = W::near(d, sx[k] - sx[j], st.tab);
   }
   __syncthreads();
   // Pair u of slot j (u < c): u < L is the left pair (j - u - 1, j), else
@@ -862,8 +867,8 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         }
         // at most kWalk neighbours a side (or the dense list is full)
         T r = T(1);
-        for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) r += W::near(d, x - sx[q]);
-        for (int q = j + 1; q < m && sx[q] - x <= S; ++q) r += W::near(d, sx[q] - x);
+        for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) r += W::near(d, x - sx[q], st.tab);
+        for (int q = j + 1; q < m && sx[q] - x <= S; ++q) r += W::near(d, sx[q] - x, st.tab);
         sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
       }
     }
@@ -882,7 +887,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
         T* wrow = kCache ? reinterpret_cast<T*>(d.wc) + (size_t)j * m : nullptr;
         auto nu = [&](int qq) {
-          const T w = W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x);
+          const T w = W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
           if (kCache && cw) wrow[qq] = w;
           return w;
         };
@@ -947,12 +952,12 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         MV A = MS::load(sA, j), B = MS::load(sB, j);
         typename MS::Acc dA{}, dB{};
         for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) {
-          const T P = normalised<T>(d.norm, W::near(d, x - sx[q]), ip, sr[q]);
+          const T P = normalised<T>(d.norm, W::near(d, x - sx[q], st.tab), ip, sr[q]);
           MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
           MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
         }
         for (int q = j + 1; q < m && sx[q] - x <= S; ++q) {
-          const T P = normalised<T>(d.norm, W::near(d, sx[q] - x), ip, sr[q]);
+          const T P = normalised<T>(d.norm, W::near(d, sx[q] - x, st.tab), ip, sr[q]);
           MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
           MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
         }
@@ -989,7 +994,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         auto pair = [&](int qq, int ch) {
           if (qq == j) return;
           const T w =
-              from_c ? __ldcg(&wrow[qq]) : W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x);
+              from_c ? __ldcg(&wrow[qq]) : W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
           const T P = normalised<T>(d.norm, w, ip, sr[qq]);
           MS::acc(cA[ch], P, MS::diff(MS::load(sA, qq), A));
           MS::acc(cB[ch], P, MS::diff(MS::load(sB, qq), B));
@@ -1127,8 +1132,9 @@ __global__ void __launch_bounds__(Fast::kT, PR == MT_FP64 ? 3 : kFusedCtasPerSm)
     k_step1d(Dev d, cudaGraphConditionalHandle cond, int use_cond) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ bool s_last;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
   Ctrl* c = d.ctrl;
-  const StepState st = step_state(d);
+  const StepState st = step_state<PR, Fast::kT>(d, s_tab);
   const int sc = st.sc;
   const long long Dc = (c->dmax >> d.cshift) + 2;
   const unsigned char* pcur = d.pred[sc];
@@ -1210,8 +1216,9 @@ __global__ void __launch_bounds__(Big::kT, 1)
   __shared__ int s_warp[Big::kT / 32];
   __shared__ int s_list[Big::kT];
   __shared__ int s_nlist;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
   Ctrl* c = d.ctrl;
-  const StepState st = step_state(d);
+  const StepState st = step_state<PR, Big::kT>(d, s_tab);
   const int sc = st.sc;
   const long long Dc = (c->dmax >> d.cshift) + 2;
   const int rank = blockIdx.x % CL;
@@ -1281,7 +1288,8 @@ __global__ void __launch_bounds__(Big::kT, 1)
   __shared__ bool s_last;
   Ctrl* c = d.ctrl;
   const int nov = c->nov;
-  const StepState st = step_state(d);
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  const StepState st = step_state<PR, Big::kT>(d, s_tab);
   const int sc = st.sc;
   const long long Dc = (c->dmax >> d.cshift) + 2;
   const int rank = blockIdx.x % CL, cid = blockIdx.x / CL;

@@ -140,7 +140,9 @@ struct Dev {
   float inv8f;              // 1 / (8 D_mt dt) 2^-2k, float
   double inv8;              // 1 / (8 D_mt dt), double
   double scale;             // 2^-k
-  double inv8s;             // inv8 scale^2 (exact): the weights' exponent from D^2 in ticks
+  unsigned long long ec;    // binary64 weights: log2(e) inv8 2^-2k in fixed point (exp_fix),
+  unsigned long long emax;  // ... the largest squared separation that does not underflow,
+  int eq, eib;              // ... left shift of the square, integer bits of the exponent
   unsigned int key0, key1;  // Philox key (seed)
   unsigned int real;        // realisation counter word
   int nbig_cap;

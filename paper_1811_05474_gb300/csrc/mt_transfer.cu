@@ -19,25 +19,6 @@
 
 namespace mt {
 
-// ------------------------------------------- step epilogue (last CTA) --
-// The last CTA of a step's final pass advances the step counter and flips
-// the buffer selectors.  Called by every thread.
-__device__ void finish_step(const Dev& d, int flip_x, int flip_m) {
-  __shared__ bool s_last;
-  Ctrl* c = d.ctrl;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(&c->done, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
-  __threadfence();
-  c->step += 1;
-  c->xcur ^= flip_x;
-  c->mcur ^= flip_m;
-  c->done = 0;
-}
-
 // ------------------------------------------------------------ observables --
 // After every step (every path): sum A, sum B, sum (A - B) and mean A of each
 // realisation, one ring row per step (sum A and sum B are conserved by the
@@ -183,6 +164,9 @@ template <int PR>
 __global__ void __launch_bounds__(kThreads) k_rowsum_walk(Dev d) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -193,12 +177,12 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_walk(Dev d) {
     for (long long q = p - 1; q >= 0; --q) {
       const long long D = x - Xs[q];
       if (D > d.S) break;
-      r += W::eval(d, D, 0);
+      r += W::near(d, D, s_tab);
     }
     for (long long q = p + 1; q < d.n; ++q) {
       const long long D = Xs[q] - x;
       if (D > d.S) break;
-      r += W::eval(d, D, 0);
+      r += W::near(d, D, s_tab);
     }
   } else {
     // periodic: the walks continue around the realisation's ring (2 Smax <
@@ -207,12 +191,12 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_walk(Dev d) {
     for (long long k = 1; k < g.n; ++k) {
       const long long D = wrap(x - Xs[ring_step(g, p, -k)], g.Lq);
       if (D > d.S) break;
-      r += W::eval(d, D, 0);
+      r += W::near(d, D, s_tab);
     }
     for (long long k = 1; k < g.n; ++k) {
       const long long D = wrap(Xs[ring_step(g, p, k)] - x, g.Lq);
       if (D > d.S) break;
-      r += W::eval(d, D, 0);
+      r += W::near(d, D, s_tab);
     }
   }
   store_rinv<mixw(PR)>(d, p, r);
@@ -232,6 +216,9 @@ __global__ void __launch_bounds__(kThreads) k_exchange_walk(Dev d, int sp) {
   using T = typename W::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   const bool valid = p < d.n;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -247,7 +234,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_walk(Dev d, int sp) {
     B = MS::load(MB, p);
     typename MS::Acc dA{}, dB{};
     auto pair = [&](long long q, long long D) {
-      const T P = normalised<T>(d.norm, W::eval(d, D, 0), ip, load_rinv<mixw(PR)>(d, q));
+      const T P = normalised<T>(d.norm, W::near(d, D, s_tab), ip, load_rinv<mixw(PR)>(d, q));
       MS::acc(dA, P, MS::diff(MS::load(MA, q), A));
       MS::acc(dB, P, MS::diff(MS::load(MB, q), B));
     };
@@ -346,6 +333,8 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_tile(Dev d) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   __shared__ unsigned int s_x[kTileChunk];
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
   __shared__ long long s_lohi[2];
   const long long b0 = (long long)blockIdx.x * kThreads;
   const long long b1 = min(b0 + (long long)kThreads, d.n);
@@ -371,7 +360,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_tile(Dev d) {
     const int ql = (int)(jl - c0);
     const unsigned int qn = (unsigned int)(jr - jl);
     auto term = [&](int j) {
-      const T w = W::near(d, (int)(s_x[j] - x32));
+      const T w = W::near(d, (int)(s_x[j] - x32), s_tab);
       return (unsigned int)(j - ql) < qn ? w : T(0);
     };
     int j = j0;
@@ -403,6 +392,8 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
   using MS = Mass<PR>;
   using MV = typename MS::V;
   __shared__ unsigned int s_x[kTileChunk];
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
   __shared__ T s_r[kTileChunk];
   __shared__ MV s_a[kTileChunk];
   __shared__ MV s_b[kTileChunk];
@@ -448,7 +439,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
     const int ql = (int)(jl - c0);
     const unsigned int qn = (unsigned int)(jr - jl);
     auto pair = [&](int j, typename MS::Acc& a, typename MS::Acc& b) {
-      const T w = W::near(d, (int)(s_x[j] - x32));
+      const T w = W::near(d, (int)(s_x[j] - x32), s_tab);
       const T P2 = (unsigned int)(j - ql) < qn ? w * (ip + s_r[j]) : T(0);
       MS::acc(a, P2, MS::diff(s_a[j], A));
       MS::acc(b, P2, MS::diff(s_b[j], B));
@@ -524,6 +515,9 @@ template <int PR>
 __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -537,7 +531,7 @@ __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
   for (; k <= kr; ++k) {
     const long long D = gap(d, g, Xs, p, ring(d, g, p, k));
     if (D > d.S) break;
-    const T w = W::eval(d, D, 0);
+    const T w = W::near(d, D, s_tab);
     if (k <= d.band_cap) band[band_at(d, p, k)] = w;
     r.add(w);
   }
@@ -555,6 +549,9 @@ template <int PR>
 __global__ void __launch_bounds__(kThreads) k_band_rowsum(Dev d) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const T* band = static_cast<const T*>(d.band);
@@ -568,7 +565,7 @@ __global__ void __launch_bounds__(kThreads) k_band_rowsum(Dev d) {
   for (int k = 1; k <= kb; ++k) r.add(band[band_at(d, ring(d, g, p, -k), k)]);
   if (kl > kb) {
     const long long* Xs = d.X[xc ^ 1];
-    for (int k = kb + 1; k <= kl; ++k) r.add(W::eval(d, gap(d, g, Xs, ring(d, g, p, -k), p), 0));
+    for (int k = kb + 1; k <= kl; ++k) r.add(W::near(d, gap(d, g, Xs, ring(d, g, p, -k), p), s_tab));
   }
   store_rinv<mixw(PR)>(d, p, r.value());
 }
@@ -579,6 +576,9 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
   using T = typename W::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   const bool valid = p < d.n;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -609,13 +609,13 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
     }
     for (int k = bl + 1; k <= kl; ++k) {
       const long long q = ring(d, g, p, -k);
-      pair(q, W::eval(d, gap(d, g, Xs, q, p), 0));
+      pair(q, W::near(d, gap(d, g, Xs, q, p), s_tab));
     }
 #pragma unroll 2
     for (int k = 1; k <= br; ++k) pair(ring(d, g, p, k), band[band_at(d, p, k)]);
     for (int k = br + 1; k <= kr; ++k) {
       const long long q = ring(d, g, p, k);
-      pair(q, W::eval(d, gap(d, g, Xs, p, q), 0));
+      pair(q, W::near(d, gap(d, g, Xs, p, q), s_tab));
     }
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
@@ -635,7 +635,8 @@ __device__ __forceinline__ void cell2_run(const Dev& d, const long long* Xs, lon
                                           typename Weight<mixw(PR), 2>::T ip,
                                           typename Mass<PR>::V A, typename Mass<PR>::V B,
                                           typename Mass<PR>::Acc& dA,
-                                          typename Mass<PR>::Acc& dB, long long ob) {
+                                          typename Mass<PR>::Acc& dB, long long ob,
+                                          const unsigned long long* s_tab) {
   using W = Weight<mixw(PR), 2>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -646,7 +647,7 @@ __device__ __forceinline__ void cell2_run(const Dev& d, const long long* Xs, lon
       dy = min_image(dy, d.Lq[1]);
     }
     if (!in_range2(dx, dy, d.S)) continue;
-    const T w = W::eval(d, dx, dy);
+    const T w = W::near2(d, dx, dy, s_tab);
     if (!EXCHANGE) {
       r += w;
     } else if (q != p) {
@@ -668,10 +669,11 @@ __device__ __forceinline__ void cell2_loop(const Dev& d, const long long* Xs, lo
                                            typename Weight<mixw(PR), 2>::T ip,
                                            typename Mass<PR>::V A, typename Mass<PR>::V B,
                                            typename Mass<PR>::Acc& dA,
-                                           typename Mass<PR>::Acc& dB, long long ob) {
+                                           typename Mass<PR>::Acc& dB, long long ob,
+                                          const unsigned long long* s_tab) {
   if (PER) {
     cells2_visit(d, x, y, [&](int q0, int q1) {
-      cell2_run<PR, EXCHANGE, true>(d, Xs, p, x, y, q0, q1, r, M, ip, A, B, dA, dB, ob);
+      cell2_run<PR, EXCHANGE, true>(d, Xs, p, x, y, q0, q1, r, M, ip, A, B, dA, dB, ob, s_tab);
     });
     return;
   }
@@ -683,7 +685,7 @@ __device__ __forceinline__ void cell2_loop(const Dev& d, const long long* Xs, lo
   for (long long row = ky - 1; row <= ky + 1; ++row) {
     if (row < 0 || row >= d.ncy) continue;
     cell2_run<PR, EXCHANGE, false>(d, Xs, p, x, y, d.start[row * d.ncx + kx0],
-                                    d.start[row * d.ncx + kx1 + 1], r, M, ip, A, B, dA, dB, ob);
+                                    d.start[row * d.ncx + kx1 + 1], r, M, ip, A, B, dA, dB, ob, s_tab);
   }
 }
 
@@ -692,6 +694,9 @@ __device__ __forceinline__ void cell2_loop(const Dev& d, const long long* Xs, lo
 template <int PR, bool PER>
 __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
   using T = typename Weight<mixw(PR), 2>::T;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -700,7 +705,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
   typename Mass<PR>::Acc dummy{};
   typename Mass<PR>::V z{};
   cell2_loop<PR, false, PER>(d, Xs, p, Xs[p], Xs[d.n + p], r, nullptr, T(0), z, z, dummy,
-                              dummy, 0);
+                              dummy, 0, s_tab);
   store_rinv<mixw(PR)>(d, p, r);
   const int s = d.src[p];
   d.id[xc ^ 1][p] = d.id[xc][s];
@@ -712,6 +717,9 @@ __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
   using T = typename Weight<mixw(PR), 2>::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
+  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
+  if (!mixw(PR)) exp_table<kThreads>(s_tab);
+  if (!mixw(PR)) __syncthreads();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   const bool valid = p < d.n;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -726,7 +734,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
     T r = T(0);
     typename MS::Acc dA{}, dB{};
     cell2_loop<PR, true, PER>(d, Xs, p, Xs[p], Xs[d.n + p], r, MA, load_rinv<mixw(PR)>(d, p), A, B,
-                               dA, dB, sq.ob - sq.oa);
+                               dA, dB, sq.ob - sq.oa, s_tab);
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
     if (sq.store_b) MS::store(d.M[mc] + sq.ob, p, B);
