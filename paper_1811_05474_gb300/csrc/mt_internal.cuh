@@ -480,6 +480,10 @@ cudaError_t launch_move(const Dev& d, bool move, bool hist, cudaStream_t s);
 cudaError_t launch_sort(const Dev& d, cudaStream_t s, Marker& mk);  // scan, scatter, cell sort
 cudaError_t launch_permute(const Dev& d, cudaStream_t s);  // gather id/masses after sort, flip
 cudaError_t launch_transfer(const Dev& d, int search, int precision, cudaStream_t s, Marker& mk);
+// brute force and full matrix by the scan with candidate lists (mt_allpairs.cu);
+// false, with nothing enqueued, where a thread per row is the faster form
+bool launch_allpairs(const Dev& d, bool cut, int precision, cudaStream_t s, Marker& mk,
+                     cudaError_t* e);
 // after a step: the observables row of every realisation
 cudaError_t launch_obs(const Dev& d, int precision, cudaStream_t s);
 // the fused path's graph: snapshot the state's buffer and step, then (beside

@@ -899,86 +899,98 @@ static void launch_exchange_brute(const Dev& d, bool cut, unsigned int g, cudaSt
 // The extra species' passes (pairs 2-3, 4-5, ...) run between the row sums
 // and the A/B pass, which ends the step.
 template <int PR>
-static void transfer_t(const Dev& d, int search, cudaStream_t s, Marker& mk) {
+static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
   const unsigned int g = (unsigned int)((d.n + kThreads - 1) / kThreads);
-  if (search == MT_SEARCH_CELL) {
-    if (d.dim == 1 && d.band_cap > 0) {
-      mk("band_build", s);
-      k_band_build<PR><<<g, kThreads, 0, s>>>(d);
-      mk("band_rowsum", s);
-      k_band_rowsum<PR><<<g, kThreads, 0, s>>>(d);
-      if (d.nspec > 2) {
-        mk("gather_species", s);
-        k_gather_species<<<g, kThreads, 0, s>>>(d);
-      }
-      for (int sp = 2; sp < d.nspec; sp += 2) {
-        mk("band_exchange_species", s);
-        k_band_exchange<PR, true><<<g, kThreads, 0, s>>>(d, sp);
-      }
-      mk("band_exchange", s);
-      k_band_exchange<PR, false><<<g, kThreads, 0, s>>>(d, 0);
-    } else if (d.dim == 1 && d.tile) {
-      mk("rowsum_tile", s);
-      k_rowsum_tile<PR><<<g, kThreads, 0, s>>>(d);
-      if (d.nspec > 2) {
-        mk("gather_species", s);
-        k_gather_species<<<g, kThreads, 0, s>>>(d);
-      }
-      for (int sp = 2; sp < d.nspec; sp += 2) {
-        mk("exchange_tile_species", s);
-        k_exchange_tile<PR, true><<<g, kThreads, 0, s>>>(d, sp);
-      }
-      mk("exchange_tile", s);
-      k_exchange_tile<PR, false><<<g, kThreads, 0, s>>>(d, 0);
-    } else if (d.dim == 1) {
-      mk("rowsum_walk", s);
-      k_rowsum_walk<PR><<<g, kThreads, 0, s>>>(d);
-      if (d.nspec > 2) {
-        mk("gather_species", s);
-        k_gather_species<<<g, kThreads, 0, s>>>(d);
-      }
-      for (int sp = 2; sp < d.nspec; sp += 2) {
-        mk("exchange_walk_species", s);
-        k_exchange_walk<PR, true><<<g, kThreads, 0, s>>>(d, sp);
-      }
-      mk("exchange_walk", s);
-      k_exchange_walk<PR, false><<<g, kThreads, 0, s>>>(d, 0);
-    } else if (d.periodic) {
-      cell2_passes<PR, true>(d, g, s, mk);
-    } else {
-      cell2_passes<PR, false>(d, g, s, mk);
-    }
-  } else {
-    const bool cut = search == MT_SEARCH_BRUTE;
-    mk(cut ? "rowsum_brute" : "rowsum_full", s);
-    if (cut) {
-      if (d.dim == 1)
-        k_rowsum_brute<PR, true, 1><<<g, kThreads, 0, s>>>(d);
-      else
-        k_rowsum_brute<PR, true, 2><<<g, kThreads, 0, s>>>(d);
-    } else {
-      if (d.dim == 1)
-        k_rowsum_brute<PR, false, 1><<<g, kThreads, 0, s>>>(d);
-      else
-        k_rowsum_brute<PR, false, 2><<<g, kThreads, 0, s>>>(d);
+  if (d.dim == 1 && d.band_cap > 0) {
+    mk("band_build", s);
+    k_band_build<PR><<<g, kThreads, 0, s>>>(d);
+    mk("band_rowsum", s);
+    k_band_rowsum<PR><<<g, kThreads, 0, s>>>(d);
+    if (d.nspec > 2) {
+      mk("gather_species", s);
+      k_gather_species<<<g, kThreads, 0, s>>>(d);
     }
     for (int sp = 2; sp < d.nspec; sp += 2) {
-      mk(cut ? "exchange_brute_species" : "exchange_full_species", s);
-      launch_exchange_brute<PR, true>(d, cut, g, s, sp);
+      mk("band_exchange_species", s);
+      k_band_exchange<PR, true><<<g, kThreads, 0, s>>>(d, sp);
     }
-    mk(cut ? "exchange_brute" : "exchange_full", s);
-    launch_exchange_brute<PR, false>(d, cut, g, s, 0);
+    mk("band_exchange", s);
+    k_band_exchange<PR, false><<<g, kThreads, 0, s>>>(d, 0);
+  } else if (d.dim == 1 && d.tile) {
+    mk("rowsum_tile", s);
+    k_rowsum_tile<PR><<<g, kThreads, 0, s>>>(d);
+    if (d.nspec > 2) {
+      mk("gather_species", s);
+      k_gather_species<<<g, kThreads, 0, s>>>(d);
+    }
+    for (int sp = 2; sp < d.nspec; sp += 2) {
+      mk("exchange_tile_species", s);
+      k_exchange_tile<PR, true><<<g, kThreads, 0, s>>>(d, sp);
+    }
+    mk("exchange_tile", s);
+    k_exchange_tile<PR, false><<<g, kThreads, 0, s>>>(d, 0);
+  } else if (d.dim == 1) {
+    mk("rowsum_walk", s);
+    k_rowsum_walk<PR><<<g, kThreads, 0, s>>>(d);
+    if (d.nspec > 2) {
+      mk("gather_species", s);
+      k_gather_species<<<g, kThreads, 0, s>>>(d);
+    }
+    for (int sp = 2; sp < d.nspec; sp += 2) {
+      mk("exchange_walk_species", s);
+      k_exchange_walk<PR, true><<<g, kThreads, 0, s>>>(d, sp);
+    }
+    mk("exchange_walk", s);
+    k_exchange_walk<PR, false><<<g, kThreads, 0, s>>>(d, 0);
+  } else if (d.periodic) {
+    cell2_passes<PR, true>(d, g, s, mk);
+  } else {
+    cell2_passes<PR, false>(d, g, s, mk);
   }
+}
+
+// All pairs, a thread per row: binary32 weights in systems where much of the
+// matrix is nonzero (launch_allpairs takes the others).
+template <int PR>
+static void brute_t(const Dev& d, bool cut, cudaStream_t s, Marker& mk) {
+  const unsigned int g = (unsigned int)((d.n + kThreads - 1) / kThreads);
+  mk(cut ? "rowsum_brute" : "rowsum_full", s);
+  if (cut) {
+    if (d.dim == 1)
+      k_rowsum_brute<PR, true, 1><<<g, kThreads, 0, s>>>(d);
+    else
+      k_rowsum_brute<PR, true, 2><<<g, kThreads, 0, s>>>(d);
+  } else {
+    if (d.dim == 1)
+      k_rowsum_brute<PR, false, 1><<<g, kThreads, 0, s>>>(d);
+    else
+      k_rowsum_brute<PR, false, 2><<<g, kThreads, 0, s>>>(d);
+  }
+  for (int sp = 2; sp < d.nspec; sp += 2) {
+    mk(cut ? "exchange_brute_species" : "exchange_full_species", s);
+    launch_exchange_brute<PR, true>(d, cut, g, s, sp);
+  }
+  mk(cut ? "exchange_brute" : "exchange_full", s);
+  launch_exchange_brute<PR, false>(d, cut, g, s, 0);
 }
 
 cudaError_t launch_transfer(const Dev& d, int search, int precision, cudaStream_t s,
                             Marker& mk) {
-  if (precision == MT_MIXED)
-    transfer_t<MT_MIXED>(d, search, s, mk);
-  else if (precision == MT_MIXED_DF32)
-    transfer_t<MT_MIXED_DF32>(d, search, s, mk);
-  else
-    transfer_t<MT_FP64>(d, search, s, mk);
+  if (search != MT_SEARCH_CELL) {
+    const bool cut = search == MT_SEARCH_BRUTE;
+    cudaError_t e = cudaSuccess;
+    if (launch_allpairs(d, cut, precision, s, mk, &e)) return e;
+    if (precision == MT_MIXED)
+      brute_t<MT_MIXED>(d, cut, s, mk);
+    else
+      brute_t<MT_MIXED_DF32>(d, cut, s, mk);
+  } else if (precision == MT_MIXED) {
+    transfer_t<MT_MIXED>(d, s, mk);
+  } else if (precision == MT_MIXED_DF32) {
+    transfer_t<MT_MIXED_DF32>(d, s, mk);
+  } else {
+    transfer_t<MT_FP64>(d, s, mk);
+  }
   return cudaGetLastError();
 }
 
