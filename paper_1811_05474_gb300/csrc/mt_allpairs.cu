@@ -9,101 +9,111 @@
 // pair adds exact zeros to the row sum and the exchange.  At the usual
 // densities that is a handful of pairs per row out of 10^3 to 10^5.
 //
-// A warp takes R rows.  Positions are staged in shared memory as 32-bit
-// coarse coordinates X >> sh, one j per lane, and the test per pair is a
-// subtraction and an unsigned comparison: it bounds the scan, about 2.5 warp
-// instructions per 32 pairs with R = 8.  A lane's candidates are appended,
-// in the order of j, to the row's list in shared memory (a ballot and a
-// prefix count), and a full list is worked off 32 entries at a time with the
-// exact 64-bit test and the weight.  Row sums in binary32 add the list's
+// A warp takes R rows, a lane one j.  The test uses coarse coordinates X >> sh
+// of 24 bits as binary32 numbers, staged in shared memory: their differences
+// are exact, and a subtraction per row (FMA pipe) and a three-input minimum of
+// magnitudes per two rows (ALU pipe, half rate) leave one comparison and one
+// vote per R rows and 32 pairs, which bounds the scan: ~1.9 warp instructions
+// per row and 32 pairs with R = 16.  Lanes that see a row note it in a bit
+// mask; only the rows of the mask are looked at.  A lane's candidates are
+// appended, in the order of j, to the row's list in shared memory (a ballot
+// and a prefix count), and a full list is worked off 32 entries at a time with
+// the exact 64-bit test and the weight.  Row sums in binary32 add the list's
 // nonzero weights one by one in the order of j, the order (and the bits) of
 // a plain loop over j; binary64 sums and the flux sums use lane partials and
 // a fixed shuffle tree.
 //
-// Measured, one step: N = 10^3 binary64 full matrix 3.0 ms -> 40 us, N = 10^5
-// binary32 weights 22.2 ms -> 4.7 ms (a thread per row and an exponential per pair
-// before: 4 CTAs at N = 10^3, ~25 instructions per pair).
+// Measured, one step: N = 10^3 binary64 full matrix 3.0 ms -> 35 us, N = 10^5
+// binary32 weights 22.2 ms -> 2.6 ms (a thread per row and an exponential per
+// pair before: 4 CTAs at N = 10^3, ~25 instructions per pair; the same lists
+// behind an integer comparison and a predicate per row: 4.7 ms; behind 16-bit
+// add-minimum pairs: 5.3 ms).
+#include <cmath>
+
 #include "mt_pair.cuh"
 
 namespace mt {
 
-constexpr int kApTile = 1024;   // j-particles staged per tile
-constexpr int kApWarps = kThreads / 32;
+constexpr int kApTile = 2048;   // j-particles staged per tile
+constexpr int kApThreads = 128;
+constexpr int kApWarps = kApThreads / 32;
 constexpr int kApCap = 64;      // list entries per row
 
 struct ApGrid {
-  int sh;                 // coarse coordinate: X >> sh, below 2^31
-  unsigned int zc;        // candidate if |difference of coarse coordinates| <= zc
-  unsigned int pc[2];     // periodic walls: ... or >= pc (the wrapped image)
-  int cut;                // 1: the exact cutoff test applies
+  int sh;         // coarse coordinate: X >> sh, below 2^24
+  float zc;       // candidate if the coarse distance is at most zc (per axis)
+  float half[2];  // periodic walls: half the coarse domain length
+  int cut;        // 1: the exact cutoff test applies
 };
+
+__device__ __forceinline__ float min_abs3(float a, float b, float c) {
+  float r;
+  asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 
 // Row state of a warp: the candidates listed and the sums so far.
 template <int PR, int R, bool EX>
 struct ApRow {
   int list[R][kApCap];
-  int cnt[R];
-  unsigned int cx[R], cy[R];
   typename Weight<mixw(PR), 1>::T r[EX ? 1 : R];
   typename Mass<PR>::Acc da[EX ? R : 1], db[EX ? R : 1];
 };
 
-// EX = false: row sums.  EX = true: exchange of A and B and the end of the
+// PER: periodic walls.  EX = false: row sums.  EX = true: exchange of A and B and the end of the
 // step (sp = 0), or of the extra species sp, sp + 1.
-template <int PR, int DIM, int R, bool EX>
-__global__ void __launch_bounds__(kThreads) k_allpairs(Dev d, ApGrid g, int sp) {
+template <int PR, int DIM, int R, bool EX, bool PER>
+__global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_allpairs(Dev d, ApGrid g, int sp) {
   using W = Weight<mixw(PR), DIM>;
   using T = typename W::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
-  __shared__ unsigned int s_cx[kApTile];
-  __shared__ unsigned int s_cy[DIM == 2 ? kApTile : 1];
+  __shared__ float s_cx[kApTile];
+  __shared__ float s_cy[DIM == 2 ? kApTile : 1];
   extern __shared__ __align__(16) unsigned char s_rows[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   ApRow<PR, R, EX>& s = reinterpret_cast<ApRow<PR, R, EX>*>(s_rows)[warp];
   const long long row0 = ((long long)blockIdx.x * kApWarps + warp) * R;
   const long long n = d.n;
+  const int nr = row0 < n ? (int)min((long long)R, n - row0) : 0;
   const long long* X = d.X[d.ctrl->xcur];
   const int mc = d.ctrl->mcur;
   const SpeciesPair sq = sp > 0 ? species_pair<true>(d, sp) : species_pair<false>(d, 0);
   const unsigned long long* MA = d.M[mc] + sq.oa;
   const unsigned long long* MB = d.M[mc] + sq.ob;
-  const unsigned int zc = g.zc, w2 = 2 * zc;
-  unsigned int lx[R], ly[R];  // coarse coordinates of the rows minus zc
+  auto coarse = [&](int a, long long j) {
+    return __int2float_rn((int)(X[(long long)a * n + j] >> g.sh));
+  };
+  float rx[R], ry[R];  // coarse coordinates of the rows (missing rows repeat the last)
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const long long p = row0 + r < n ? row0 + r : n - 1;
-    lx[r] = (unsigned int)(X[p] >> g.sh) - zc;
-    ly[r] = DIM == 2 ? (unsigned int)(X[n + p] >> g.sh) - zc : 0;
-    if (lane == 0) {
-      s.cnt[r] = 0;
-      s.cx[r] = lx[r];
-      s.cy[r] = ly[r];
-      if (EX) {
-        s.da[r] = {};
-        s.db[r] = {};
-      } else {
-        s.r[r] = T(0);
-      }
+    rx[r] = coarse(0, p);
+    ry[r] = DIM == 2 ? coarse(1, p) : 0.0f;
+  }
+  if (lane < nr) {
+    if (EX) {
+      s.da[EX ? lane : 0] = {};
+      s.db[EX ? lane : 0] = {};
+    } else {
+      s.r[EX ? 0 : lane] = T(0);
     }
   }
-  // can the pair of a row (lx, ly) and a lane's coordinates have a weight?
-  auto near = [&](unsigned int cx, unsigned int cy, unsigned int x, unsigned int y) {
-    const unsigned int ux = cx - x;  // difference + zc
-    bool ok = ux <= w2;
-    if (d.periodic) ok = ok || (unsigned int)abs((int)(ux - zc)) >= g.pc[0];
-    if (DIM == 2) {
-      const unsigned int uy = cy - y;
-      bool oky = uy <= w2;
-      if (d.periodic) oky = oky || (unsigned int)abs((int)(uy - zc)) >= g.pc[1];
-      ok = ok && oky;
+  int mycnt = 0;  // lane r: entries in the list of row r
+  int cnt1 = 0;   // R = 1: the row's, in every lane
+  // coarse distance of a lane's coordinates to row r (the larger of the axes')
+  auto dist = [&](float cx, float cy, int r) {
+    float u = cx - rx[r], v = DIM == 2 ? cy - ry[r] : 0.0f;
+    if (PER) {  // min(|u|, L - |u|)
+      u = g.half[0] - fabsf(fabsf(u) - g.half[0]);
+      if (DIM == 2) v = g.half[1] - fabsf(fabsf(v) - g.half[1]);
     }
-    return ok;
+    return DIM == 2 ? fmaxf(fabsf(u), fabsf(v)) : u;
   };
   // work off the list of row r (every lane of the warp)
   auto flush = [&](int r) {
     __syncwarp();
-    const int cnt = s.cnt[r];
+    const int cnt = __shfl_sync(0xffffffffu, mycnt, r);
     const long long p = row0 + r;
     const long long x = X[p], y = DIM == 2 ? X[n + p] : 0;
     MV A{}, B{};
@@ -121,7 +131,7 @@ __global__ void __launch_bounds__(kThreads) k_allpairs(Dev d, ApGrid g, int sp) 
       if (k + lane < cnt) {
         j = s.list[r][k + lane];
         long long dx = X[j] - x, dy = DIM == 2 ? X[n + j] - y : 0;
-        if (d.periodic) {
+        if (PER) {
           dx = min_image(dx, d.Lq[0]);
           if (DIM == 2) dy = min_image(dy, d.Lq[1]);
         }
@@ -157,56 +167,65 @@ __global__ void __launch_bounds__(kThreads) k_allpairs(Dev d, ApGrid g, int sp) 
       if (lane == 0) s.r[EX ? 0 : r] = sum;
     }
     __syncwarp();
-    if (lane == 0) s.cnt[r] = 0;
-    __syncwarp();
+    if (lane == r) mycnt = 0;
   };
   for (long long j0 = 0; j0 < n; j0 += kApTile) {
     __syncthreads();
-    for (int i = threadIdx.x; i < kApTile; i += kThreads) {
+    for (int i = threadIdx.x; i < kApTile; i += kApThreads) {
       const long long j = j0 + i;
-      s_cx[i] = j < n ? (unsigned int)(X[j] >> g.sh) : 0;
-      if (DIM == 2) s_cy[i] = j < n ? (unsigned int)(X[n + j] >> g.sh) : 0;
+      s_cx[i] = j < n ? coarse(0, j) : 0.0f;
+      if (DIM == 2) s_cy[i] = j < n ? coarse(1, j) : 0.0f;
     }
     __syncthreads();
     const int nt = (int)min((long long)kApTile, n - j0);
-    if (row0 >= n) continue;  // a warp without rows only stages
+    if (nr == 0) continue;  // a warp without rows only stages
 #pragma unroll 2
     for (int i0 = 0; i0 < nt; i0 += 32) {
-      const unsigned int cx = s_cx[i0 + lane], cy = DIM == 2 ? s_cy[i0 + lane] : 0;
-      bool any = false;
-      if (d.periodic) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) any |= near(cx, cy, lx[r], ly[r]);
-      } else if (DIM == 1) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) any |= cx - lx[r] <= w2;
-      } else {
-#pragma unroll
-        for (int r = 0; r < R; ++r) any |= cx - lx[r] <= w2 && cy - ly[r] <= w2;
-      }
-      if (!__any_sync(0xffffffffu, any)) continue;
-      const bool in = i0 + lane < nt;
-#pragma unroll 1
-      for (int r = 0; r < R && row0 + r < n; ++r) {
-        const bool c = in && near(cx, cy, s.cx[r], s.cy[r]);
+      const float cx = s_cx[i0 + lane], cy = DIM == 2 ? s_cy[i0 + lane] : 0.0f;
+      if (R == 1) {  // one row: a vote is the list's next entries
+        const bool c = i0 + lane < nt && fabsf(dist(cx, cy, 0)) <= g.zc;
         const unsigned int m = __ballot_sync(0xffffffffu, c);
-        if (!m) continue;
-        int at = s.cnt[r];
+        if (m == 0) continue;
+        if (cnt1 + __popc(m) > kApCap) {
+          mycnt = cnt1;
+          flush(0);
+          cnt1 = 0;
+        }
+        if (c) s.list[0][cnt1 + __popc(m & ((1u << lane) - 1u))] = (int)(j0 + i0 + lane);
+        cnt1 += __popc(m);
+        continue;
+      }
+      float m = 3.0e38f;
+#pragma unroll
+      for (int r = 0; r < R; r += 2)
+        m = min_abs3(dist(cx, cy, r), dist(cx, cy, r + 1 < R ? r + 1 : r), m);
+      if (!__any_sync(0xffffffffu, m <= g.zc)) continue;
+      unsigned int mine = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) mine |= fabsf(dist(cx, cy, r)) <= g.zc ? 1u << r : 0u;
+      if (i0 + lane >= nt) mine = 0;
+      unsigned int rows = __reduce_or_sync(0xffffffffu, mine) & ((1u << nr) - 1u);
+#pragma unroll 1
+      for (; rows; rows &= rows - 1) {
+        const int r = __ffs(rows) - 1;
+        const bool c = (mine >> r) & 1u;
+        const unsigned int m = __ballot_sync(0xffffffffu, c);
+        int at = __shfl_sync(0xffffffffu, mycnt, r);
         if (at + __popc(m) > kApCap) {
           flush(r);
           at = 0;
         }
         if (c) s.list[r][at + __popc(m & ((1u << lane) - 1u))] = (int)(j0 + i0 + lane);
-        __syncwarp();
-        if (lane == 0) s.cnt[r] = at + __popc(m);
-        __syncwarp();
+        if (lane == r) mycnt = at + __popc(m);
       }
     }
   }
-  if (row0 < n) {
-    for (int r = 0; r < R && row0 + r < n; ++r) flush(r);
+  if (nr > 0) {
+    if (R == 1) mycnt = cnt1;
+#pragma unroll 1
+    for (int r = 0; r < nr; ++r) flush(r);
     const long long p = row0 + lane;
-    if (lane < R && p < n) {
+    if (lane < nr) {
       if (!EX) {
         store_rinv<mixw(PR)>(d, p, s.r[EX ? 0 : lane]);
       } else {
@@ -224,19 +243,28 @@ template <int PR, int DIM, int R, bool EX>
 static cudaError_t launch_one(const Dev& d, const ApGrid& g, int sp, cudaStream_t s) {
   const size_t sm = kApWarps * sizeof(ApRow<PR, R, EX>);
   const long long rows = (long long)kApWarps * R;
-  k_allpairs<PR, DIM, R, EX><<<(unsigned int)((d.n + rows - 1) / rows), kThreads, sm, s>>>(d, g, sp);
+  const unsigned int grid = (unsigned int)((d.n + rows - 1) / rows);
+  if (d.periodic)
+    k_allpairs<PR, DIM, R, EX, true><<<grid, kApThreads, sm, s>>>(d, g, sp);
+  else
+    k_allpairs<PR, DIM, R, EX, false><<<grid, kApThreads, sm, s>>>(d, g, sp);
   return cudaGetLastError();
 }
 
-// Rows per warp: 8 amortise a staged coordinate's load and the vote over 8
-// tests; a system that would then leave multiprocessors with less than two
-// CTAs takes a row per warp (N = 10^3: 125 CTAs).
+// Rows per warp: 16 amortise a staged coordinate's load, the comparison and
+// the vote over 24 instructions; a system that would then leave
+// multiprocessors with less than two CTAs takes 4 or 1 (N = 10^3: 250 CTAs).
+template <int PR, int DIM, bool EX>
+static cudaError_t launch_rows(const Dev& d, const ApGrid& g, int sp, cudaStream_t s) {
+  const long long fill = 2LL * d.nsm * kApWarps;
+  if (d.n >= 16 * fill) return launch_one<PR, DIM, 16, EX>(d, g, sp, s);
+  if (d.n >= 4 * fill) return launch_one<PR, DIM, 4, EX>(d, g, sp, s);
+  return launch_one<PR, DIM, 1, EX>(d, g, sp, s);
+}
+
 template <int PR, bool EX>
 static cudaError_t launch_pr(const Dev& d, const ApGrid& g, int sp, cudaStream_t s) {
-  const bool wide = d.n >= 2LL * d.nsm * kApWarps * 8;
-  if (d.dim == 1)
-    return wide ? launch_one<PR, 1, 8, EX>(d, g, sp, s) : launch_one<PR, 1, 1, EX>(d, g, sp, s);
-  return wide ? launch_one<PR, 2, 8, EX>(d, g, sp, s) : launch_one<PR, 2, 1, EX>(d, g, sp, s);
+  return d.dim == 1 ? launch_rows<PR, 1, EX>(d, g, sp, s) : launch_rows<PR, 2, EX>(d, g, sp, s);
 }
 
 // The scan's parameters; false where the list does not pay: binary32 weights
@@ -258,14 +286,11 @@ static bool ap_grid(const Dev& d, bool cut, int precision, ApGrid* g) {
   if (precision != MT_FP64 && reach > 0.25) return false;
   g->cut = cut ? 1 : 0;
   g->sh = 0;
-  while ((Lmax >> g->sh) >= (1LL << 31)) ++g->sh;
-  const long long z = Z < (double)Lmax ? (long long)Z + 1 : Lmax;
-  const long long zc = (z >> g->sh) + 1;
-  g->zc = (unsigned int)(zc < (1LL << 31) - 1 ? zc : (1LL << 31) - 1);
-  for (int k = 0; k < 2; ++k) {
-    const long long p = ((d.Lq[k] - z) >> g->sh) - 1;
-    g->pc[k] = p > 0 ? (unsigned int)p : 0u;
-  }
+  while ((Lmax >> g->sh) >= (1LL << 24)) ++g->sh;
+  // rounding of both coordinates, and of the coarse half length and of its
+  // differences (half a unit each): two more units
+  g->zc = (float)(std::floor(std::ldexp(Z < (double)Lmax ? Z : (double)Lmax, -g->sh)) + 3.0);
+  for (int k = 0; k < 2; ++k) g->half[k] = (float)std::ldexp((double)d.Lq[k], -g->sh - 1);
   return true;
 }
 
