@@ -871,6 +871,9 @@ mt_status mt_batch_create(const mt_params* p, const mt_batch* b, void* workspace
   d.wc_cap = D.wc_cap;
   d.rt = reinterpret_cast<const Real*>(w + D.o_rt);
   d.nreal = D.nreal;
+  d.single = D.nreal == 1 && D.rt[0].base == 0 && D.rt[0].off == 0 ? 1 : 0;
+  d.rLq = D.rt[0].Lq;
+  d.rreal = D.rt[0].real;
   d.lbits = D.lbits;
   d.lmask = (int)((1LL << D.lbits) - 1);
   d.sslot = reinterpret_cast<const int*>(w + D.o_sslot);

@@ -209,8 +209,8 @@ __device__ __forceinline__ void prefetch_next_l2(const Dev& d, const SegPrefetch
 }
 
 // ------------------------------------------------ first tier: pair list --
-// The first tier's transfer (row sums, exchange, reaction) over a list of
-// the unordered pairs of its staged, sorted particles.  Owners are the
+// The first tier's transfer (row sums, exchange, reaction) with binary64
+// weights, over a list of the unordered pairs of its staged, sorted particles.  Owners are the
 // staged slots j with x_j in [xlo - 2 Smax, xhi + Smax); each owns its pairs
 // (j, k), k > j, x_k - x_j <= Smax -- R_j consecutive slots, since the slots
 // are sorted -- and pair q of owner j sits at pfx[j] + (k - j - 1) in the
@@ -232,10 +232,11 @@ __host__ __device__ constexpr size_t pair_region_bytes() {
   return (size_t)kPairCap * sizeof(T) + (size_t)(TR::kCap + 1) * 2 + (size_t)kPairCap * 2;
 }
 
-// Dynamic shared memory of the first tier: staging, bins and the pair list.
+// Dynamic shared memory of the first tier: staging, bins and, with binary64
+// weights, the pair list.
 size_t fused_smem_bytes(int precision) {
   return precision == MT_FP64 ? pair_region_offset<Fast, double>() + pair_region_bytes<Fast, double>()
-                              : pair_region_offset<Fast, float>() + pair_region_bytes<Fast, float>();
+                              : pair_region_offset<Fast, float>();
 }
 
 // First index q in [0, m) with a[q] >= key (a sorted ascending), by one
@@ -259,13 +260,13 @@ __device__ __forceinline__ int warp_lower_at_least(const long long* a, int m, lo
   return lo + __popc(__ballot_sync(0xffffffffu, p < hi && a[p] < key));
 }
 
-template <int PR, typename TR>
-__device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* smem, bool active,
-                              int m, int w0, int w1, long long out0, long long xlo, long long xhi) {
-  using W = Weight<mixw(PR), 1>;
-  using T = typename W::T;
-  using MS = Mass<PR>;
-  using MV = typename MS::V;
+template <typename TR>
+__device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* smem, int m,
+                              int w0, int w1, long long out0, long long xlo, long long xhi) {
+  using W = Weight<false, 1>;
+  using T = double;
+  using MS = Mass<MT_FP64>;
+  using MV = double;
   constexpr int NT = TR::kT, CAP = TR::kCap;
   constexpr int kCnt = 64;  // pair-count bins of the lane assignment
   long long* sx = reinterpret_cast<long long*>(smem);
@@ -285,7 +286,7 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
   // (A) owners [olo, rhi) and row-sum slots [rlo, rhi), one search per warp
   if (warp < 3) {
     const long long key = warp == 0 ? xlo - 2 * S : warp == 1 ? xlo - S : xhi + S;
-    const int v = active ? warp_lower_at_least(sx, m, key) : 0;
+    const int v = warp_lower_at_least(sx, m, key);
     if (lane == 0) s_idx[warp] = v;
   } else if (warp == 3) {
     for (int b = lane; b < kCnt; b += 32) s_hist[b] = 0;
@@ -415,25 +416,23 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
       pair_of(j, jj, left, u, q, partner);
       r += sw[q];
     }
-    sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
+    sr[j] = rcp_ge1(r);
   }
   __syncthreads();
-  // (G) binary64 weights under the symmetric normalisation: each listed
-  // pair's P = nu (1/r_j + 1/r_k) / 2 once, in place of nu (pairs with an
-  // end outside the row-sum range are never read); binary32 weights form P
-  // where they are used (three binary32 operations)
+  // (G) the symmetric normalisation: each listed pair's 2 P = nu (1/r_j +
+  // 1/r_k) once, in place of nu (the flux sums are halved at the end, exactly;
+  // pairs with an end outside the row-sum range are never read)
   const bool sym = d.norm != MT_NORM_ROW;
-  constexpr bool kPairP = !mixw(PR);
-  if (kPairP && sym) {
+  if (sym) {
     for (int q = tid; q < np; q += NT) {
       const int jj = own[q];
       const int j = olo + jj, k = j + 1 + (q - pfx[jj]);
-      if (j >= rlo && k < rhi) sw[q] = normalised<T>(MT_NORM_SYM, sw[q], sr[j], sr[k]);
+      if (j >= rlo && k < rhi) sw[q] *= sr[j] + sr[k];
     }
     __syncthreads();
   }
   // (H) exchange and reaction of own particles
-  if (active) {
+  {
     long long* Xn = d.X[st.xc ^ 1];
     int* In = d.id[st.xc ^ 1];
     unsigned long long* Mn = d.M[st.mc ^ 1];
@@ -448,9 +447,13 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
       for (int u = 0; u < cnt; ++u) {
         int q, i;
         pair_of(j, jj, left, u, q, i);
-        const T P = kPairP && sym ? sw[q] : normalised<T>(d.norm, sw[q], ip, sr[i]);
+        const T P = sym ? sw[q] : sw[q] * ip;
         MS::acc(dA, P, MS::diff(MS::load(sA, i), A));
         MS::acc(dB, P, MS::diff(MS::load(sB, i), B));
+      }
+      if (sym) {
+        dA = acc_half(dA);
+        dB = acc_half(dB);
       }
       MS::update(A, B, dA, dB, d.react);
       const long long o = out0 + (j - w0);
@@ -471,16 +474,474 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
   return true;
 }
 
-// Process one segment with the CTA (all NT threads call it).  The CTA
-// computes the exchange for the own particles j with (j - first own) %
-// nslice == slice, and the cell starts / segment boundaries only for slice
-// 0; each thread adds the particles it updates to its observables
-// accumulators (obs_sum, in shared memory).  Returns kSegOk, or why the
-// segment does not fit this tier (then nothing of it has been written).
+// A dense bin (more than kBinMax particles) of len records at lo, sorted by
+// (x, id) by the whole CTA: up to kRankMax records by rank -- the number of
+// smaller keys, packed into 64 bits as (x - bin start) << 31 | id where bins
+// are at most 2^32 ticks wide -- a record per thread; larger bins by an
+// in-place bitonic sort, every comparator ascending (partner i ^ (2j - 1)
+// first in each merge) so any length sorts.  scratch: free shared words.
+template <typename TR>
+__device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* sA,
+                                            unsigned long long* sB, int* sid, int lo, int len,
+                                            long long blo, bool packs, int* scratch) {
+  constexpr int NT = TR::kT, NB = TR::kBins;
+  constexpr int kRankMax = (NB / 2 - 1) < NT ? (NB / 2 - 1) : NT;
+  const int tid = threadIdx.x;
+  unsigned long long* key = reinterpret_cast<unsigned long long*>(
+      (reinterpret_cast<uintptr_t>(scratch) + 7) & ~static_cast<uintptr_t>(7));
+  if (len <= kRankMax && packs) {
+    long long x = 0;
+    int id = 0, rank = 0;
+    unsigned long long a = 0, b = 0;
+    if (tid < len) {
+      x = sx[lo + tid];
+      id = sid[lo + tid];
+      a = sA[lo + tid];
+      b = sB[lo + tid];
+      key[tid] = ((unsigned long long)(x - blo) << 31) | (unsigned int)id;
+    }
+    __syncthreads();
+    if (tid < len) {
+      const unsigned long long mine = key[tid];
+#pragma unroll 4
+      for (int q = 0; q < len; ++q) rank += key[q] < mine ? 1 : 0;
+      sx[lo + rank] = x;
+      sid[lo + rank] = id;
+      sA[lo + rank] = a;
+      sB[lo + rank] = b;
+    }
+    __syncthreads();
+    return;
+  }
+  int np2 = 1;
+  while (np2 < len) np2 <<= 1;
+  for (int mm = 2; mm <= np2; mm <<= 1) {
+    for (int jj = mm >> 1; jj > 0; jj >>= 1) {
+      for (int i = tid; i < np2; i += NT) {
+        const int l = (jj == (mm >> 1)) ? (i ^ (mm - 1)) : (i ^ jj);
+        if (l > i && l < len) {
+          const int p = lo + i, q = lo + l;
+          if (sx[q] < sx[p] || (sx[q] == sx[p] && sid[q] < sid[p])) {
+            const long long tx = sx[p];
+            sx[p] = sx[q];
+            sx[q] = tx;
+            const int ti = sid[p];
+            sid[p] = sid[q];
+            sid[q] = ti;
+            const unsigned long long ta = sA[p];
+            sA[p] = sA[q];
+            sA[q] = ta;
+            const unsigned long long tb = sB[p];
+            sB[p] = sB[q];
+            sB[q] = tb;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// ------------------------------------------------- first tier: transfer --
+// Binary32 weights (MT_MIXED, MT_MIXED_DF32): row sums, exchange and reaction
+// straight from the sorted slots, without a pair list.  A weight is six
+// instructions here, less than building, indexing and reading back a list
+// entry, so both passes evaluate it (exp_fix's binary64 weights, ten times
+// that, keep the list of pair_transfer).
+//   (A) one thread per slot within Smax of the own cells: left neighbours
+//       (nearest first), then right ones, adding weights to r_j = 1 + ... in
+//       that order (the order of the cluster tiers' walks) and counting both;
+//   (B) own slots are handed to lanes in order of their pair count (a
+//       counting sort): the exchange's binary64 warp instructions hold their
+//       pipe ~19 cycles whatever lanes are active, so a warp's lanes should
+//       run the same number of pairs;
+//   (C) exchange and reaction of own slots over their left then right pairs.
+// A segment with more unordered pairs than the pair list of the binary64 form
+// holds goes to the cluster tier, as there.
+// Measured against the pair list (weights once per pair, six more phases),
+// with the sort of fast_segment: N = 10^6 MT_MIXED 134 -> 123 us per step, 3 10^5
+// MT_MIXED_DF32 40 -> 35 us, 256 realisations 656 -> 580 us; same bits.
+template <int PR>
+__device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* smem, int m,
+                              int w0, int w1, long long out0, long long xlo, long long xhi) {
+  using W = Weight<mixw(PR), 1>;
+  using T = typename W::T;
+  using MS = Mass<PR>;
+  using MV = typename MS::V;
+  constexpr int NT = Fast::kT, CAP = Fast::kCap, PER = Fast::kPer;
+  constexpr int kCnt = 64;  // pair-count bins of the lane assignment
+  const long long* sx = reinterpret_cast<const long long*>(smem);
+  const unsigned long long* sA = reinterpret_cast<const unsigned long long*>(sx + CAP);
+  const unsigned long long* sB = sA + CAP;
+  const int* sid = reinterpret_cast<const int*>(sB + CAP);
+  T* sr = reinterpret_cast<T*>(const_cast<int*>(sid) + CAP);
+  int* perm = reinterpret_cast<int*>(sr + CAP) + Fast::kBins + 1;  // (free after the sort)
+  __shared__ int s_hist[kCnt];
+  __shared__ int s_np;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long S = d.S;
+  if (tid < kCnt) s_hist[tid] = 0;
+  if (tid == kCnt) s_np = 0;
+  __syncthreads();
+  // (A)
+  int v[PER];  // own slots: slot | left pairs << 10 | right pairs << 21
+  int np = 0;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int j = tid + k * NT;
+    v[k] = -1;
+    if (j >= m) continue;
+    const long long x = sx[j];
+    if (x < xlo - 2 * S || x >= xhi + S) continue;
+    const bool sum = x >= xlo - S;  // else only its pairs are counted
+    T r = T(1);
+    int i = j - 1;
+    if (sum) {
+      for (; i >= 0; --i) {
+        const long long D = x - sx[i];
+        if (D > S) break;
+        r += W::near(d, D, nullptr);
+      }
+    }
+    int q = j + 1;
+    for (; q < m; ++q) {
+      const long long D = sx[q] - x;
+      if (D > S) break;
+      if (sum) r += W::near(d, D, nullptr);
+    }
+    np += q - 1 - j;
+    if (sum) sr[j] = T(__frcp_rn((float)r));
+    if (j >= w0 && j < w1) {
+      const int L = j - 1 - i, R = q - 1 - j, c = L + R;
+      v[k] = j | L << 10 | R << 21;
+      atomicAdd(&s_hist[c < kCnt ? c : kCnt - 1], 1);
+    }
+  }
+  np = __reduce_add_sync(0xffffffffu, np);
+  if (lane == 0 && np) atomicAdd(&s_np, np);
+  __syncthreads();
+  if (s_np > kPairCap) return false;  // uniform across the CTA
+  // (B)
+  if (warp == 0) {
+    const int h0 = s_hist[2 * lane], h1 = s_hist[2 * lane + 1];
+    int hin = h0 + h1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, hin, o);
+      if (lane >= o) hin += t;
+    }
+    s_hist[2 * lane] = hin - h0 - h1;
+    s_hist[2 * lane + 1] = hin - h1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    if (v[k] < 0) continue;
+    const int c = ((v[k] >> 10) & 0x7ff) + (v[k] >> 21);
+    perm[atomicAdd(&s_hist[c < kCnt ? c : kCnt - 1], 1)] = v[k];
+  }
+  __syncthreads();
+  // (C)
+  const int nown = w1 - w0;
+  unsigned long long* Mn = d.M[st.mc ^ 1];
+  if (out0 + nown > d.n) raise_error(d.ctrl, kErrIndex, out0);
+  for (int p = tid; p < nown; p += NT) {
+    const int u0 = perm[p], j = u0 & 0x3ff, L = (u0 >> 10) & 0x7ff, c = L + (u0 >> 21);
+    const unsigned int x32 = (unsigned int)sx[j];  // within the cutoff the low words' difference is the separation
+    const T ip = sr[j];
+    MV A = MS::load(sA, j), B = MS::load(sB, j);
+    typename MS::Acc dA{}, dB{};
+    for (int u = 0; u < c; ++u) {
+      const int i = u < L ? j - 1 - u : j + 1 + u - L;
+      const T w = W::near(d, (int)((unsigned int)sx[i] - x32), nullptr);
+      const T P = normalised<T>(d.norm, w, ip, sr[i]);
+      MS::acc(dA, P, MS::diff(MS::load(sA, i), A));
+      MS::acc(dB, P, MS::diff(MS::load(sB, i), B));
+    }
+    MS::update(A, B, dA, dB, d.react);
+    const long long o = out0 + (j - w0);
+    if (o < d.n) {
+      MS::store(Mn, o, A);
+      MS::store(Mn, d.n + o, B);
+    }
+  }
+  long long* Xn = d.X[st.xc ^ 1];
+  int* In = d.id[st.xc ^ 1];
+  for (int j = w0 + tid; j < w1; j += NT) {  // positions and ids, coalesced
+    const long long o = out0 + (j - w0);
+    if (o < d.n) {
+      Xn[o] = sx[j];
+      In[o] = sid[j];
+    }
+  }
+  return true;
+}
+
+// Next step's cell starts and segment boundaries, by the CTA that wrote the
+// segment's particles: sorted slots [w0, w1) of its staging to out0 on.
+template <int NT>
+__device__ __forceinline__ void segment_tables(const Dev& d, int sc, int seg, const long long* sx,
+                                               const int* bstart, int sh2, long long wlo, int c0,
+                                               int c1, int w0, int w1, long long out0) {
+  const int tid = threadIdx.x, wsh = d.cshift;
+  int* Sn = d.fstart[sc ^ 1];
+  for (long long cc = c0 + tid; cc < c1; cc += NT) {
+    const long long key = cc << wsh;
+    int lo;
+    if (sh2 == wsh) {
+      lo = bstart[(key - wlo) >> sh2];  // bins are the cells
+    } else {
+      lo = w0;  // first own slot with x >= key
+      int hi = w1;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (sx[mid] < key)
+          lo = mid + 1;
+        else
+          hi = mid;
+      }
+    }
+    Sn[cc] = (int)(out0 + (lo - w0));
+  }
+  // Segment s2 >= 1 starts after the cell that holds slot sslot[s2] - 1;
+  // this CTA sets the boundaries whose slot it wrote.  The first such s2
+  // is found by a short walk from seg + 1 (out0 is near sslot[seg]).
+  int* CBn = d.cb[sc ^ 1];
+  const long long own = w1 - w0;
+  int s2 = seg + 1;
+  if (d.sslot[seg] > out0) {
+    while (s2 > 1 && d.sslot[s2 - 1] > out0) --s2;
+  } else if (d.sslot[seg + 1] <= out0) {
+    while (s2 < d.nseg && d.sslot[s2] <= out0) ++s2;
+  }
+  for (s2 += tid; s2 < d.nseg; s2 += NT) {
+    const long long q = d.sslot[s2] - 1;  // last slot before segment s2's first
+    if (q >= out0 + own) break;
+    // a realisation's first segment starts at its first cell, fixed
+    if (q >= out0 && d.sreal[s2] == d.sreal[s2 - 1])
+      CBn[s2] = (int)((sx[w0 + (q - out0)] >> wsh) + 1);
+  }
+}
+
+// One segment in the first tier (all threads of the CTA call it): stage and
+// move, counting sort, row sums, exchange, reaction, output.  Returns kSegOk,
+// or why the segment does not fit this tier (then nothing of it has been
+// written).  The sort: each particle takes an arrival number in its bin with
+// the histogram's atomic, (x, id) go to the bin's slots in arrival order, and
+// each thread ranks its own particles among their bin's (two or three of
+// them) and writes the whole record to its final slot, masses included
+// (loaded from global memory meanwhile): no record moves more than once, and
+// no thread sorts a bin alone.
+template <int PR>
+__device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned char* smem,
+                            const SegScalars& g, const SegPrefetch& pf) {
+  using T = typename Weight<mixw(PR), 1>::T;
+  constexpr int NT = Fast::kT, PER = Fast::kPer, CAP = Fast::kCap, NB = Fast::kBins;
+  constexpr int BPT = Fast::kBinsPerThread;
+  long long* sx = reinterpret_cast<long long*>(smem);
+  unsigned long long* sA = reinterpret_cast<unsigned long long*>(sx + CAP);
+  unsigned long long* sB = sA + CAP;
+  int* sid = reinterpret_cast<int*>(sB + CAP);
+  T* sr = reinterpret_cast<T*>(sid + CAP);
+  int* bstart = reinterpret_cast<int*>(sr + CAP);  // [NB + 1]
+  int* bcur = bstart + NB + 1;                     // [NB]
+  __shared__ int s_lt, s_w0, s_w1, s_nbig, s_work;
+  __shared__ int s_big[kBigMax];
+  __shared__ int s_scan[NT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long c0 = g.c0, c1 = g.c1, a0 = g.a0, o0 = g.o0, o1 = g.o1;
+  const int L = g.L, wsh = d.cshift;
+  const long long wlo = lmax(c0 - d.hc, 0) << wsh;
+  const long long whi = lmin(c1 + d.hc, d.ncell) << wsh;
+  const long long xlo = c0 << wsh, xhi = c1 << wsh;  // own cells in ticks
+  int sh2 = wsh;
+  while (sh2 < 62 && ((whi - wlo) >> sh2) >= NB) ++sh2;
+  // bins the window spans (bins are cells unless the window has >= NB cells)
+  const int nb = whi > wlo ? (int)(((whi - 1 - wlo) >> sh2) + 1) : 1;
+  const bool active = c0 < c1;
+  if (active && L > CAP) {
+    if (tid == 0) prefetch_stage2(d, pf);
+    return kSegCapacity;
+  }
+  // ---- stage: the loads are in flight while the bins are cleared ----------
+  long long rx[PER];
+  int rid[PER], rb[PER];  // rb: bin | arrival number << 16
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int e = tid + k * NT;
+    const bool in = active && e < L;
+    rx[k] = in ? d.X[st.xc][a0 + e] : 0;
+    rid[k] = in ? d.id[st.xc][a0 + e] : 0;
+  }
+  if (tid == 0) {
+    s_lt = 0;
+    s_w0 = 0;
+    s_w1 = 0;
+    s_nbig = 0;
+    s_work = 0;
+  }
+  for (int b = tid; b <= nb; b += NT) bstart[b] = 0;
+  __syncthreads();
+  // ---- move and histogram --------------------------------------------------
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    rb[k] = -1;
+    const int e0 = k * NT + (tid & ~31);  // the warp's first slot
+    if (!active || e0 >= L) continue;     // uniform in the warp
+    const int e = tid + k * NT;
+    bool lt = false, in0 = false, in1 = false;
+    if (e < L) {
+      const long long slot = a0 + e;
+      long long base = 0, Lq = d.rLq, off = 0;
+      unsigned int real = d.rreal;
+      int loc = rid[k];
+      if (!d.single) {
+        const Real* R = d.rt + (rid[k] >> d.lbits);
+        base = R->base;
+        Lq = R->Lq;
+        off = R->off;
+        real = R->real;
+        loc &= d.lmask;
+      }
+      float z;
+      if (st.noise) {
+        z = st.noise[off + loc];
+      } else {
+        const uint4 u =
+            philox4x32_10(make_uint4((unsigned int)loc, (unsigned int)st.step,
+                                     (unsigned int)(st.step >> 32), real),
+                          d.key0, d.key1);
+        z = box_muller(u.x, u.y).x;
+      }
+      const long long x = base + reflect(rx[k] - base + d.drift[0] + walk_ticks(d.bq, z), Lq);
+      rx[k] = x;
+      lt = slot >= o0 && slot < o1 && x < xlo;
+      if (x >= wlo && x < whi) {
+        const int b = (int)((x - wlo) >> sh2);
+        rb[k] = b | atomicAdd(&bstart[b + 1], 1) << 16;
+        in0 = x < xlo;
+        in1 = x < xhi;
+      }
+    }
+    // slots that may have moved below the own cells: only the first ones
+    if (a0 + e0 < o1 && a0 + e0 + 32 > o0) {
+      const int n_lt = __popc(__ballot_sync(0xffffffffu, lt));
+      if (lane == 0 && n_lt) atomicAdd(&s_lt, n_lt);
+    }
+    if (sh2 != wsh) {  // else the bins give the own range
+      const int n_0 = __popc(__ballot_sync(0xffffffffu, in0));
+      const int n_1 = __popc(__ballot_sync(0xffffffffu, in1));
+      if (lane == 0 && n_0) atomicAdd(&s_w0, n_0);
+      if (lane == 0 && n_1) atomicAdd(&s_w1, n_1);
+    }
+  }
+  if (tid == 0) prefetch_stage2(d, pf);  // the next segment's cell starts
+  __syncthreads();
+  if (!active) return kSegOk;  // no cells: nothing to write
+  // ---- bin starts ----------------------------------------------------------
+  {
+    int v[BPT];
+    int sum = 0, work = 0;
+#pragma unroll
+    for (int j = 0; j < BPT; ++j) {
+      v[j] = tid * BPT + j < nb ? bstart[1 + tid * BPT + j] : 0;
+      sum += v[j];
+      work += v[j] * v[j];
+      if (v[j] > kBinMax) {
+        const int at = atomicAdd(&s_nbig, 1);
+        if (at < kBigMax) s_big[at] = tid * BPT + j;
+      }
+    }
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_scan[warp] = inc;
+    // (capped per warp: the sum over warps stays in range)
+    work = __reduce_add_sync(0xffffffffu, work < kHeavyWork ? work : kHeavyWork);
+    if (lane == 0 && work > 0) atomicAdd(&s_work, work);
+    __syncthreads();
+    int run = inc - sum;
+    for (int w = 0; w < warp; ++w) run += s_scan[w];
+#pragma unroll
+    for (int j = 0; j < BPT; ++j) {
+      run += v[j];
+      if (tid * BPT + j < nb) bstart[1 + tid * BPT + j] = run;
+    }
+  }
+  if (s_nbig > kBigMax) return kSegDense;  // uniform across the CTA
+  if (s_work >= kHeavyWork) return kSegHeavy;
+  __syncthreads();
+  // ---- (x, id) into the bins in arrival order ------------------------------
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    if (rb[k] < 0) continue;
+    const int at = bstart[rb[k] & 0xffff] + (rb[k] >> 16);
+    sx[at] = rx[k];
+    sid[at] = rid[k];
+  }
+  __syncthreads();
+  // ---- final slots: rank by (x, id) inside the bin -------------------------
+  unsigned long long ra[PER], rm[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    if (rb[k] < 0) continue;
+    const long long e = a0 + tid + k * NT;
+    ra[k] = d.M[st.mc][e];
+    rm[k] = d.M[st.mc][d.n + e];
+    const int b = rb[k] & 0xffff, lo = bstart[b], hi = bstart[b + 1];
+    int to = lo + (rb[k] >> 16);
+    if (hi - lo > 1 && hi - lo <= kBinMax) {  // (larger bins: below)
+      const int self = to;
+      to = lo;
+      for (int q = lo; q < hi; ++q) {
+        const long long y = sx[q];
+        to += y < rx[k] || (y == rx[k] && q != self && sid[q] < rid[k]) ? 1 : 0;
+      }
+    }
+    rb[k] = to;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    if (rb[k] < 0) continue;
+    sx[rb[k]] = rx[k];
+    sid[rb[k]] = rid[k];
+    sA[rb[k]] = ra[k];
+    sB[rb[k]] = rm[k];
+  }
+  __syncthreads();
+  if (s_nbig > 0) {
+    // dense bins: the whole CTA
+    for (int t = 0; t < s_nbig; ++t)
+      sort_dense_bin<Fast>(sx, sA, sB, sid, bstart[s_big[t]], bstart[s_big[t] + 1] - bstart[s_big[t]],
+                           wlo + ((long long)s_big[t] << sh2), sh2 <= 32, bcur);
+  }
+  const int m = bstart[nb];
+  const int w0 = sh2 == wsh ? bstart[(xlo - wlo) >> wsh] : s_w0;
+  const int w1 = sh2 == wsh ? bstart[(xhi - wlo) >> wsh] : s_w1;
+  const long long out0 = o0 + s_lt;
+  if (tid == 0) prefetch_next_l2(d, pf, st);
+  bool fits;
+  if constexpr (mixw(PR))
+    fits = walk_transfer<PR>(d, st, smem, m, w0, w1, out0, xlo, xhi);
+  else
+    fits = pair_transfer<Fast>(d, st, smem, m, w0, w1, out0, xlo, xhi);
+  if (!fits) return kSegHeavy;  // more pairs than the list holds: the second tier takes it
+  segment_tables<NT>(d, st.sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0);
+  return kSegOk;
+}
+
+// One segment in a cluster tier (every thread of the cluster's CL CTAs calls
+// it): all CTAs stage and sort it, CTA `slice` sums every CL-th row and
+// exchanges every CL-th own particle, and CTA 0 writes the cell starts and
+// segment boundaries.  Returns kSegOk, or why the segment does not fit (then
+// nothing of it has been written).
 template <int PR, typename TR, int CL>
 __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigned char* smem,
-                             const SegScalars& g, int slice, int nslice, bool route_heavy,
-                             bool* heavy_out = nullptr, const SegPrefetch* pf = nullptr,
+                             const SegScalars& g, int slice, bool* heavy_out = nullptr,
                              bool cache_w = false) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
@@ -587,7 +1048,6 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       }
     }
   }
-  if (pf && tid == 0) prefetch_stage2(d, *pf);  // the next segment's cell starts
   __syncthreads();
 
   // ---- 3: counting sort into bins, then (x, id) order inside each bin -----
@@ -651,10 +1111,6 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
     active = false;
   }
   if (heavy_out) *heavy_out = s_work >= kHeavyWork || L > Fast::kCap;
-  if (active && route_heavy && s_work >= kHeavyWork) {
-    status = kSegHeavy;
-    active = false;
-  }
   if (active) {
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -693,40 +1149,32 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
     }
   }
   __syncthreads();
-  // Dense bins, sorted by the whole CTA.  Up to kRankMax records (256 in
-  // the first tier, 1023 in the second): each record's rank is the number of
-  // smaller (x, id) keys in the bin, packed into 64 bits as (x - bin start)
-  // << 31 | id (bins are at most 2^32 ticks wide here), then every record
-  // moves to its rank.  Larger bins: in-place
-  // bitonic sort, every comparator ascending (partner i ^ (2j - 1) first in
-  // each merge) so any length sorts.
+  // Dense bins, sorted by the whole cluster: up to kRankMax records by rank
+  // (sort_dense_bin's packed keys, every CL-th rank formed by each CTA);
+  // larger bins by each CTA alone.
   if (active) {
     const int nbig = s_nbig < kBigMax ? s_nbig : kBigMax;
     // the scatter cursors are free now: they hold the packed keys
     unsigned long long* key = reinterpret_cast<unsigned long long*>(
         (reinterpret_cast<uintptr_t>(bcur) + 7) & ~static_cast<uintptr_t>(7));
-    // first tier: one record per thread (registers); second tier: up to 2
-    constexpr int kRankMax = (NB / 2 - 1) < (NT > 256 ? 2 * NT : NT) ? (NB / 2 - 1)
-                                                                      : (NT > 256 ? 2 * NT : NT);
+    constexpr int kRankMax = (NB / 2 - 1) < 2 * NT ? (NB / 2 - 1) : 2 * NT;
     constexpr int E = (kRankMax + NT - 1) / NT;  // records per thread
     for (int t = 0; t < nbig; ++t) {
       const int lo = bstart[s_big[t]], len = bstart[s_big[t] + 1] - lo;
       if (len <= kRankMax && sh2 <= 32) {
-        if constexpr (CL > 1) {
-          // a bin's records sit in scatter order, which differs between the
-          // cluster's CTAs: all take the first CTA's arrangement
-          cg::cluster_group cl = cg::this_cluster();
-          cl.sync();
-          if (slice != 0) {
-            for (int i = tid; i < len; i += NT) {
-              sx[lo + i] = *cl.map_shared_rank(&sx[lo + i], 0u);
-              sid[lo + i] = *cl.map_shared_rank(&sid[lo + i], 0u);
-              sA[lo + i] = *cl.map_shared_rank(&sA[lo + i], 0u);
-              sB[lo + i] = *cl.map_shared_rank(&sB[lo + i], 0u);
-            }
+        // a bin's records sit in scatter order, which differs between the
+        // cluster's CTAs: all take the first CTA's arrangement
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        if (slice != 0) {
+          for (int i = tid; i < len; i += NT) {
+            sx[lo + i] = *cl.map_shared_rank(&sx[lo + i], 0u);
+            sid[lo + i] = *cl.map_shared_rank(&sid[lo + i], 0u);
+            sA[lo + i] = *cl.map_shared_rank(&sA[lo + i], 0u);
+            sB[lo + i] = *cl.map_shared_rank(&sB[lo + i], 0u);
           }
-          __syncthreads();
         }
+        __syncthreads();
         const long long blo = wlo + ((long long)s_big[t] << sh2);
         for (int i = tid; i < len; i += NT)
           key[i] = ((unsigned long long)(sx[lo + i] - blo) << 31) | (unsigned int)sid[lo + i];
@@ -735,62 +1183,33 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         long long vx[E];
         int vid[E];
         unsigned long long va[E], vb[E];
-        if constexpr (CL > 1) {
-          // second tier: the cluster's CTAs rank every CL-th record each (a
-          // warp per record, lanes striding the keys) and read the other
-          // ranks from their peers' shared memory (same arrangement, same
-          // dense-bin order in every CTA)
-          int* srank = reinterpret_cast<int*>(sr);  // free until the row sums
-          cg::cluster_group cl = cg::this_cluster();
-          const int nmine = (len - slice + CL - 1) / CL;
-          for (int k = warp; k < nmine; k += NT / 32) {
-            const int i = slice + k * CL;
-            const unsigned long long mki = key[i];
-            int cnt = 0;
-            for (int q = lane; q < len; q += 32) cnt += key[q] < mki ? 1 : 0;
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            if (lane == 0) srank[i] = cnt;
-          }
-          cl.sync();
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const int i = tid + e * NT;
-            if (i < len) {
-              const unsigned int owner = (unsigned int)(i % CL);
-              rk[e] = *cl.map_shared_rank(&srank[i], owner);
-              vx[e] = sx[lo + i];
-              vid[e] = sid[lo + i];
-              va[e] = sA[lo + i];
-              vb[e] = sB[lo + i];
-            }
-          }
-          cl.sync();  // every peer has read this CTA's ranks
-        } else {
-          unsigned long long mk[E];
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const int i = tid + e * NT;
-            mk[e] = i < len ? key[i] : ~0ULL;
-            rk[e] = 0;
-          }
-#pragma unroll 4
-          for (int q = 0; q < len; ++q) {
-            const unsigned long long kq = key[q];
-#pragma unroll
-            for (int e = 0; e < E; ++e) rk[e] += kq < mk[e] ? 1 : 0;
-          }
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const int i = lo + tid + e * NT;
-            if (tid + e * NT < len) {
-              vx[e] = sx[i];
-              vid[e] = sid[i];
-              va[e] = sA[i];
-              vb[e] = sB[i];
-            }
-          }
-          __syncthreads();
+        // the cluster's CTAs rank every CL-th record each (a warp per record,
+        // lanes striding the keys) and read the other ranks from their peers'
+        // shared memory (same arrangement, same dense-bin order in every CTA)
+        int* srank = reinterpret_cast<int*>(sr);  // free until the row sums
+        const int nmine = (len - slice + CL - 1) / CL;
+        for (int k = warp; k < nmine; k += NT / 32) {
+          const int i = slice + k * CL;
+          const unsigned long long mki = key[i];
+          int cnt = 0;
+          for (int q = lane; q < len; q += 32) cnt += key[q] < mki ? 1 : 0;
+          cnt = __reduce_add_sync(0xffffffffu, cnt);
+          if (lane == 0) srank[i] = cnt;
         }
+        cl.sync();
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int i = tid + e * NT;
+          if (i < len) {
+            const unsigned int owner = (unsigned int)(i % CL);
+            rk[e] = *cl.map_shared_rank(&srank[i], owner);
+            vx[e] = sx[lo + i];
+            vid[e] = sid[lo + i];
+            va[e] = sA[lo + i];
+            vb[e] = sB[lo + i];
+          }
+        }
+        cl.sync();  // every peer has read this CTA's ranks
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           if (tid + e * NT < len) {
@@ -804,33 +1223,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         __syncthreads();
         continue;
       }
-      int np2 = 1;
-      while (np2 < len) np2 <<= 1;
-      for (int mm = 2; mm <= np2; mm <<= 1) {
-        for (int jj = mm >> 1; jj > 0; jj >>= 1) {
-          for (int i = tid; i < np2; i += NT) {
-            const int l = (jj == (mm >> 1)) ? (i ^ (mm - 1)) : (i ^ jj);
-            if (l > i && l < len) {
-              const int a = lo + i, b = lo + l;
-              if (sx[b] < sx[a] || (sx[b] == sx[a] && sid[b] < sid[a])) {
-                const long long tx = sx[a];
-                sx[a] = sx[b];
-                sx[b] = tx;
-                const int ti = sid[a];
-                sid[a] = sid[b];
-                sid[b] = ti;
-                const unsigned long long ta = sA[a];
-                sA[a] = sA[b];
-                sA[b] = ta;
-                const unsigned long long tb = sB[a];
-                sB[a] = sB[b];
-                sB[b] = tb;
-              }
-            }
-          }
-          __syncthreads();
-        }
-      }
+      sort_dense_bin<TR>(sx, sA, sB, sid, lo, len, 0, false, bcur);
     }
   }
 
@@ -839,128 +1232,162 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
   const int w0 = s_w0, w1 = s_w1;
   const long long out0 = o0 + s_lt;
   const long long S = d.S;
-  if constexpr (CL == 1) {
-    if (pf && tid == 0) prefetch_next_l2(d, *pf, st);
-    if (!pair_transfer<PR, TR>(d, st, smem, active, m, w0, w1, out0, xlo, xhi)) {
-      status = kSegHeavy;  // more pairs than the list holds: the second tier takes it
-      active = false;
-    }
-  } else {
-    // Row sums.  A particle with more than kWalk neighbours on a side is
-    // dense: it is queued (in bcur, free by now) and summed by a whole warp,
-    // lanes striding over its neighbour range, combined in a fixed tree.  The
-    // choice and the order depend only on the neighbourhood, so every CTA that
-    // forms r_j forms the same value.
-    int* dlist = bcur;
-    if (active) {
-      for (int t = tid;; t += NT) {
-        const int j = CL > 1 ? t * CL + slice : t;  // with a cluster: every CL-th
-        if (j >= m) break;
-        const long long x = sx[j];
-        if (x < xlo - S || x >= xhi + S) continue;  // not a neighbour of an own particle
-        if (dense_at(sx, m, j, x, S)) {
-          const int at = atomicAdd(&s_nd, 1);
-          if (at < NB) {
-            dlist[at] = j;
-            continue;
-          }
-        }
-        // at most kWalk neighbours a side (or the dense list is full)
-        T r = T(1);
-        for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) r += W::near(d, x - sx[q], st.tab);
-        for (int q = j + 1; q < m && sx[q] - x <= S; ++q) r += W::near(d, sx[q] - x, st.tab);
-        sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
-      }
-    }
-    __syncthreads();
-    // Binary64 weights of dense rows are dear (an exponential each): the
-    // predicted-segment kernel keeps them, row j of the staged slots at
-    // wc[j m + q], between the row sums and the exchange (read through L2:
-    // the rows are written by other CTAs of the cluster)
-    constexpr bool kCache = PR == MT_FP64 && CL > 1;
-    const bool cw = kCache && cache_w && (long long)m * m <= d.wc_cap;
-    if (active) {
-      const int nd = s_nd < NB ? s_nd : NB;
-      for (int k = warp; k < nd; k += NT / 32) {
-        const int j = dlist[k];
-        const long long x = sx[j];
-        const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
-        T* wrow = kCache ? reinterpret_cast<T*>(d.wc) + (size_t)j * m : nullptr;
-        auto nu = [&](int qq) {
-          const T w = W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
-          if (kCache && cw) wrow[qq] = w;
-          return w;
-        };
-        // second tier: four chains per lane (dense particles are its work);
-        // first tier: one (registers are scarce there)
-        T r0 = T(0), r1 = T(0), r2 = T(0), r3 = T(0);
-        int q = lo + lane;
-        if constexpr (CL > 1) {
-          for (; q + 96 < hi; q += 128) {
-            r0 += nu(q);
-            r1 += nu(q + 32);
-            r2 += nu(q + 64);
-            r3 += nu(q + 96);
-          }
-        }
-        for (; q < hi; q += 32) r0 += nu(q);
-        const T r = warp_sum((r0 + r1) + (r2 + r3));
-        if (lane == 0) sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
-      }
-    }
-    if constexpr (CL > 1) {
-      // Every CTA of the cluster staged and sorted the same particles; each
-      // formed the row sums of every CL-th one.  Gather the rest from the
-      // peers' shared memory (distributed shared memory), between two cluster
-      // barriers so no CTA reads a peer that has moved on.
-      cg::cluster_group cl = cg::this_cluster();
-      if (tid == 0) s_wcbad = s_nd > NB ? 1 : 0;  // a dense row summed without the cache
-      cl.sync();
-      if (tid == 0) {
-        int bad = 0;
-        for (int r = 0; r < CL; ++r) bad |= *cl.map_shared_rank(&s_wcbad, r);
-        s_wcok = bad ? 0 : 1;
-      }
-      if (active) {
-        for (int j = tid; j < m; j += NT) {
-          const int owner = j % CL;
-          if (owner == slice) continue;
-          const long long x = sx[j];
-          if (x < xlo - S || x >= xhi + S) continue;
-          sr[j] = *cl.map_shared_rank(&sr[j], owner);
+  // Row sums.  A particle with more than kWalk neighbours on a side is
+  // dense: it is queued (in bcur, free by now) and summed by a whole warp,
+  // lanes striding over its neighbour range, combined in a fixed tree.  The
+  // choice and the order depend only on the neighbourhood, so every CTA that
+  // forms r_j forms the same value.
+  int* dlist = bcur;
+  if (active) {
+    for (int t = tid;; t += NT) {
+      const int j = t * CL + slice;  // every CL-th
+      if (j >= m) break;
+      const long long x = sx[j];
+      if (x < xlo - S || x >= xhi + S) continue;  // not a neighbour of an own particle
+      if (dense_at(sx, m, j, x, S)) {
+        const int at = atomicAdd(&s_nd, 1);
+        if (at < NB) {
+          dlist[at] = j;
+          continue;
         }
       }
-      cl.sync();
-    } else {
-      __syncthreads();
+      // at most kWalk neighbours a side (or the dense list is full)
+      T r = T(1);
+      for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) r += W::near(d, x - sx[q], st.tab);
+      for (int q = j + 1; q < m && sx[q] - x <= S; ++q) r += W::near(d, sx[q] - x, st.tab);
+      sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
     }
-    if (active) {
-      long long* Xn = d.X[xc ^ 1];
-      int* In = d.id[xc ^ 1];
-      unsigned long long* Mn = d.M[mc ^ 1];
-      if (out0 + (w1 - w0) > d.n) raise_error(c, kErrIndex, out0);
-      for (int j = w0 + slice + tid * nslice; j < w1; j += NT * nslice) {
-        const long long x = sx[j];
-        const T ip = sr[j];
-        if (dense_at(sx, m, j, x, S)) {
-          const int at = atomicAdd(&s_nd2, 1);
-          if (at < NB) {
-            dlist[at] = j;  // a warp does it below
-            continue;
-          }
+  }
+  __syncthreads();
+  // Binary64 weights of dense rows are dear (an exponential each): the
+  // predicted-segment kernel keeps them, row j of the staged slots at
+  // wc[j m + q], between the row sums and the exchange (read through L2:
+  // the rows are written by other CTAs of the cluster)
+  constexpr bool kCache = PR == MT_FP64;
+  const bool cw = kCache && cache_w && (long long)m * m <= d.wc_cap;
+  if (active) {
+    const int nd = s_nd < NB ? s_nd : NB;
+    for (int k = warp; k < nd; k += NT / 32) {
+      const int j = dlist[k];
+      const long long x = sx[j];
+      const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
+      T* wrow = kCache ? reinterpret_cast<T*>(d.wc) + (size_t)j * m : nullptr;
+      auto nu = [&](int qq) {
+        const T w = W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
+        if (kCache && cw) wrow[qq] = w;
+        return w;
+      };
+      // four chains per lane
+      T r0 = T(0), r1 = T(0), r2 = T(0), r3 = T(0);
+      int q = lo + lane;
+      for (; q + 96 < hi; q += 128) {
+        r0 += nu(q);
+        r1 += nu(q + 32);
+        r2 += nu(q + 64);
+        r3 += nu(q + 96);
+      }
+      for (; q < hi; q += 32) r0 += nu(q);
+      const T r = warp_sum((r0 + r1) + (r2 + r3));
+      if (lane == 0) sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
+    }
+  }
+  // Every CTA of the cluster staged and sorted the same particles; each
+  // formed the row sums of every CL-th one.  Gather the rest from the
+  // peers' shared memory (distributed shared memory), between two cluster
+  // barriers so no CTA reads a peer that has moved on.
+  cg::cluster_group cl = cg::this_cluster();
+  if (tid == 0) s_wcbad = s_nd > NB ? 1 : 0;  // a dense row summed without the cache
+  cl.sync();
+  if (tid == 0) {
+    int bad = 0;
+    for (int r = 0; r < CL; ++r) bad |= *cl.map_shared_rank(&s_wcbad, r);
+    s_wcok = bad ? 0 : 1;
+  }
+  if (active) {
+    for (int j = tid; j < m; j += NT) {
+      const int owner = j % CL;
+      if (owner == slice) continue;
+      const long long x = sx[j];
+      if (x < xlo - S || x >= xhi + S) continue;
+      sr[j] = *cl.map_shared_rank(&sr[j], owner);
+    }
+  }
+  cl.sync();
+  if (active) {
+    long long* Xn = d.X[xc ^ 1];
+    int* In = d.id[xc ^ 1];
+    unsigned long long* Mn = d.M[mc ^ 1];
+    if (out0 + (w1 - w0) > d.n) raise_error(c, kErrIndex, out0);
+    for (int j = w0 + slice + tid * CL; j < w1; j += NT * CL) {
+      const long long x = sx[j];
+      const T ip = sr[j];
+      if (dense_at(sx, m, j, x, S)) {
+        const int at = atomicAdd(&s_nd2, 1);
+        if (at < NB) {
+          dlist[at] = j;  // a warp does it below
+          continue;
         }
-        MV A = MS::load(sA, j), B = MS::load(sB, j);
-        typename MS::Acc dA{}, dB{};
-        for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) {
-          const T P = normalised<T>(d.norm, W::near(d, x - sx[q], st.tab), ip, sr[q]);
-          MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
-          MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
-        }
-        for (int q = j + 1; q < m && sx[q] - x <= S; ++q) {
-          const T P = normalised<T>(d.norm, W::near(d, sx[q] - x, st.tab), ip, sr[q]);
-          MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
-          MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
-        }
+      }
+      MV A = MS::load(sA, j), B = MS::load(sB, j);
+      typename MS::Acc dA{}, dB{};
+      for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) {
+        const T P = normalised<T>(d.norm, W::near(d, x - sx[q], st.tab), ip, sr[q]);
+        MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
+        MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
+      }
+      for (int q = j + 1; q < m && sx[q] - x <= S; ++q) {
+        const T P = normalised<T>(d.norm, W::near(d, sx[q] - x, st.tab), ip, sr[q]);
+        MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
+        MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
+      }
+      MS::update(A, B, dA, dB, d.react);
+      const long long o = out0 + (j - w0);
+      if (o < d.n) {
+        Xn[o] = x;
+        In[o] = sid[j];
+        MS::store(Mn, o, A);
+        MS::store(Mn, d.n + o, B);
+      }
+    }
+  }
+  __syncthreads();
+  if (active) {
+    // dense own particles: one warp each, lanes striding the neighbourhood
+    long long* Xn = d.X[xc ^ 1];
+    int* In = d.id[xc ^ 1];
+    unsigned long long* Mn = d.M[mc ^ 1];
+    const int nd = s_nd2 < NB ? s_nd2 : NB;
+    for (int k = warp; k < nd; k += NT / 32) {
+      const int j = dlist[k];
+      const long long x = sx[j];
+      const T ip = sr[j];
+      MV A = MS::load(sA, j), B = MS::load(sB, j);
+      typename MS::Acc dA{}, dB{};
+      const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
+      // four chains per lane (q, q + 32, q + 64, q + 96), merged at the end
+      typename MS::Acc cA[4] = {}, cB[4] = {};
+      // the row's weights from the cache where every dense row went in
+      const bool from_c = kCache && cw && s_wcok;
+      const T* wrow = reinterpret_cast<const T*>(d.wc) + (size_t)j * m;
+      auto pair = [&](int qq, int ch) {
+        if (qq == j) return;
+        const T w =
+            from_c ? __ldcg(&wrow[qq]) : W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
+        const T P = normalised<T>(d.norm, w, ip, sr[qq]);
+        MS::acc(cA[ch], P, MS::diff(MS::load(sA, qq), A));
+        MS::acc(cB[ch], P, MS::diff(MS::load(sB, qq), B));
+      };
+      int q = lo + lane;
+      for (; q + 96 < hi; q += 128) {
+        pair(q, 0);
+        pair(q + 32, 1);
+        pair(q + 64, 2);
+        pair(q + 96, 3);
+      }
+      for (; q < hi; q += 32) pair(q, 0);
+      dA = acc_warp_sum(acc_merge(acc_merge(cA[0], cA[1]), acc_merge(cA[2], cA[3])));
+      dB = acc_warp_sum(acc_merge(acc_merge(cB[0], cB[1]), acc_merge(cB[2], cB[3])));
+      if (lane == 0) {
         MS::update(A, B, dA, dB, d.react);
         const long long o = out0 + (j - w0);
         if (o < d.n) {
@@ -971,106 +1398,12 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         }
       }
     }
-    __syncthreads();
-    if (active) {
-      // dense own particles: one warp each, lanes striding the neighbourhood
-      long long* Xn = d.X[xc ^ 1];
-      int* In = d.id[xc ^ 1];
-      unsigned long long* Mn = d.M[mc ^ 1];
-      const int nd = s_nd2 < NB ? s_nd2 : NB;
-      for (int k = warp; k < nd; k += NT / 32) {
-        const int j = dlist[k];
-        const long long x = sx[j];
-        const T ip = sr[j];
-        MV A = MS::load(sA, j), B = MS::load(sB, j);
-        typename MS::Acc dA{}, dB{};
-        const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
-        // second tier: four chains per lane (q, q + 32, q + 64, q + 96),
-        // merged at the end; first tier: one
-        typename MS::Acc cA[4] = {}, cB[4] = {};
-        // the row's weights from the cache where every dense row went in
-        const bool from_c = kCache && cw && s_wcok;
-        const T* wrow = reinterpret_cast<const T*>(d.wc) + (size_t)j * m;
-        auto pair = [&](int qq, int ch) {
-          if (qq == j) return;
-          const T w =
-              from_c ? __ldcg(&wrow[qq]) : W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
-          const T P = normalised<T>(d.norm, w, ip, sr[qq]);
-          MS::acc(cA[ch], P, MS::diff(MS::load(sA, qq), A));
-          MS::acc(cB[ch], P, MS::diff(MS::load(sB, qq), B));
-        };
-        int q = lo + lane;
-        if constexpr (CL > 1) {
-          for (; q + 96 < hi; q += 128) {
-            pair(q, 0);
-            pair(q + 32, 1);
-            pair(q + 64, 2);
-            pair(q + 96, 3);
-          }
-          for (; q < hi; q += 32) pair(q, 0);
-          dA = acc_warp_sum(acc_merge(acc_merge(cA[0], cA[1]), acc_merge(cA[2], cA[3])));
-          dB = acc_warp_sum(acc_merge(acc_merge(cB[0], cB[1]), acc_merge(cB[2], cB[3])));
-        } else {
-          for (; q < hi; q += 32) pair(q, 0);
-          dA = acc_warp_sum(cA[0]);
-          dB = acc_warp_sum(cB[0]);
-        }
-        if (lane == 0) {
-          MS::update(A, B, dA, dB, d.react);
-          const long long o = out0 + (j - w0);
-          if (o < d.n) {
-            Xn[o] = x;
-            In[o] = sid[j];
-            MS::store(Mn, o, A);
-            MS::store(Mn, d.n + o, B);
-          }
-        }
-      }
-    }
-    // no CTA of the cluster writes the next segment's cached rows before
-    // every CTA has read this segment's (cw is the same in all of them)
-    if (kCache && cw) cg::this_cluster().sync();
   }
-  if (active && slice == 0) {
-    // ---- 6: next step's cell starts and segment boundaries ----------------
-    int* Sn = d.fstart[sc ^ 1];
-    for (long long cc = c0 + tid; cc < c1; cc += NT) {
-      const long long key = cc << wsh;
-      int lo;
-      if (sh2 == wsh) {
-        lo = bstart[(key - wlo) >> sh2];  // bins are the cells
-      } else {
-        lo = w0;  // first own slot with x >= key
-        int hi = w1;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (sx[mid] < key)
-            lo = mid + 1;
-          else
-            hi = mid;
-        }
-      }
-      Sn[cc] = (int)(out0 + (lo - w0));
-    }
-    // Segment s2 >= 1 starts after the cell that holds slot sslot[s2] - 1;
-    // this CTA sets the boundaries whose slot it wrote.  The first such s2
-    // is found by a short walk from seg + 1 (out0 is near sslot[seg]).
-    int* CBn = d.cb[sc ^ 1];
-    const long long own = w1 - w0;
-    int s2 = seg + 1;
-    if (d.sslot[seg] > out0) {
-      while (s2 > 1 && d.sslot[s2 - 1] > out0) --s2;
-    } else if (d.sslot[seg + 1] <= out0) {
-      while (s2 < d.nseg && d.sslot[s2] <= out0) ++s2;
-    }
-    for (s2 += tid; s2 < d.nseg; s2 += NT) {
-      const long long q = d.sslot[s2] - 1;  // last slot before segment s2's first
-      if (q >= out0 + own) break;
-      // a realisation's first segment starts at its first cell, fixed
-      if (q >= out0 && d.sreal[s2] == d.sreal[s2 - 1])
-        CBn[s2] = (int)((sx[w0 + (q - out0)] >> wsh) + 1);
-    }
-  }
+  // no CTA of the cluster writes the next segment's cached rows before
+  // every CTA has read this segment's (cw is the same in all of them)
+  if (kCache && cw) cg::this_cluster().sync();
+  if (active && slice == 0)
+    segment_tables<NT>(d, sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0);
   __syncthreads();
   return status;
 }
@@ -1165,7 +1498,7 @@ __global__ void __launch_bounds__(Fast::kT, PR == MT_FP64 ? 3 : kFusedCtasPerSm)
       prefetch_stage1(d, pf);
     }
     if (!pc) {
-      const int rc = fused_segment<PR, Fast, 1>(d, st, seg, smem, cur, 0, 1, true, nullptr, &pf);
+      const int rc = fast_segment<PR>(d, st, seg, smem, cur, pf);
       if (rc != kSegOk && threadIdx.x == 0) d.ovlist[atomicAdd(&c->nov, 1)] = seg;
       if (threadIdx.x == 0) {
         pnext[seg] = rc == kSegOk ? 0 : 1;
@@ -1249,8 +1582,8 @@ __global__ void __launch_bounds__(Big::kT, 1)
       for (int k = 0; k < nl; ++k) {
         const int seg = s_list[k];
         bool heavy = true;
-        const int rc = fused_segment<PR, Big, CL>(d, st, seg, smem, load_seg(d, sc, Dc, seg),
-                                                   rank, CL, false, &heavy, nullptr, true);
+        const int rc = fused_segment<PR, Big, CL>(d, st, seg, smem, load_seg(d, sc, Dc, seg), rank,
+                                                  &heavy, true);
         if (rc != kSegOk && tid == 0 && atomicExch(&c->overflow, 1) == 0) {
           c->ov_reason = rc;
           c->ov_seg = seg;
@@ -1296,8 +1629,7 @@ __global__ void __launch_bounds__(Big::kT, 1)
   const int ncl = gridDim.x / CL;
   for (int q = cid; q < nov; q += ncl) {
     const int seg = d.ovlist[q];
-    const int rc =
-        fused_segment<PR, Big, CL>(d, st, seg, smem, load_seg(d, sc, Dc, seg), rank, CL, false);
+    const int rc = fused_segment<PR, Big, CL>(d, st, seg, smem, load_seg(d, sc, Dc, seg), rank);
     if (rc != kSegOk && threadIdx.x == 0 && atomicExch(&c->overflow, 1) == 0) {
       c->ov_reason = rc;
       c->ov_seg = seg;

@@ -151,6 +151,9 @@ struct Dev {
   int nsm;                  // multiprocessors of the device
   long long hc;             // fused halo in cells (covers 2 Smax)
   const Real* rt;           // [nreal] realisations
+  int single;               // 1: one realisation at base 0: its length and counter word are
+  unsigned int rreal;       // rLq and rreal, its particles' ids their caller indices
+  long long rLq;
   int nreal;
   int lbits;                // id = (realisation << lbits) | index within it
   int lmask;                // (1 << lbits) - 1
