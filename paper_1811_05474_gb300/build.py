@@ -19,7 +19,7 @@ BUILD = PKG / "_build"
 LIB = BUILD / "libmt.so"
 SOURCES = ["mt_api.cu", "mt_move_sort.cu", "mt_transfer.cu", "mt_allpairs.cu", "mt_io.cu", "mt_noalloc.cu", "mt_fused.cu",
            "mt_tune.cu", "mt_server.cu", "mt_probe.cu"]
-HEADERS = [CSRC / "mt_internal.cuh", CSRC / "mt_pair.cuh", ROOT / "include" / "mt.h"]
+HEADERS = [CSRC / "mt_internal.cuh", CSRC / "mt_pair.cuh", CSRC / "mt_fixed.cuh", ROOT / "include" / "mt.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr"]
