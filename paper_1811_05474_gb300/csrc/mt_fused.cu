@@ -44,7 +44,7 @@
 #include <cooperative_groups.h>
 #include <cuda_pipeline.h>
 
-#include "mt_pair.cuh"
+#include "mt_fixed.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -222,21 +222,24 @@ __device__ __forceinline__ void prefetch_next_l2(const Dev& d, const SegPrefetch
 // (j - t, j) for t = 1, 2, ... while R_{j-t} >= t.
 constexpr int kPairCap = kFusedPairCap;
 
-template <typename TR, typename T>
+// The first tier's staging: positions, two masses, an 8-byte word (sort keys,
+// then 1 / r, or the position's low word and 1 / r), ids, bins.
+template <typename TR>
 __host__ __device__ constexpr size_t pair_region_offset() {
-  return ((size_t)TR::kCap * (8 + 8 + 8 + 4 + sizeof(T)) + (size_t)(2 * TR::kBins + 1) * 4 + 7) &
+  return ((size_t)TR::kCap * (8 + 8 + 8 + 8 + 4) + (size_t)(2 * TR::kBins + 2) * 4 + 7) &
          ~(size_t)7;
 }
-template <typename TR, typename T>
+template <typename TR>
 __host__ __device__ constexpr size_t pair_region_bytes() {
-  return (size_t)kPairCap * sizeof(T) + (size_t)(TR::kCap + 1) * 2 + (size_t)kPairCap * 2;
+  return (size_t)kPairCap * 8 + (size_t)(TR::kCap + 1) * 2 + (size_t)kPairCap * 2;
 }
 
 // Dynamic shared memory of the first tier: staging, bins and, with binary64
-// weights, the pair list.
+// weights, the pair list; in MT_MIXED the staged slots' old slots.
 size_t fused_smem_bytes(int precision) {
-  return precision == MT_FP64 ? pair_region_offset<Fast, double>() + pair_region_bytes<Fast, double>()
-                              : pair_region_offset<Fast, float>();
+  return precision == MT_FP64    ? pair_region_offset<Fast>() + pair_region_bytes<Fast>()
+         : precision == MT_MIXED ? pair_region_offset<Fast>() + (size_t)Fast::kCap * 2
+                                 : pair_region_offset<Fast>();
 }
 
 // First index q in [0, m) with a[q] >= key (a sorted ascending), by one
@@ -272,10 +275,10 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
   long long* sx = reinterpret_cast<long long*>(smem);
   unsigned long long* sA = reinterpret_cast<unsigned long long*>(sx + CAP);
   unsigned long long* sB = sA + CAP;
-  int* sid = reinterpret_cast<int*>(sB + CAP);
-  T* sr = reinterpret_cast<T*>(sid + CAP);
-  int* perm = reinterpret_cast<int*>(sr + CAP) + TR::kBins + 1;  // the bins' scatter cursors
-  T* sw = reinterpret_cast<T*>(smem + pair_region_offset<TR, T>());  // [kPairCap]
+  T* sr = reinterpret_cast<T*>(sB + CAP);
+  int* sid = reinterpret_cast<int*>(sr + CAP);
+  int* perm = sid + CAP + TR::kBins + 2;  // free after the sort
+  T* sw = reinterpret_cast<T*>(smem + pair_region_offset<TR>());  // [kPairCap]
   unsigned short* pfx = reinterpret_cast<unsigned short*>(sw + kPairCap);  // [CAP + 1]
   unsigned short* own = pfx + CAP + 1;                                    // [kPairCap]
   __shared__ int s_idx[3];
@@ -479,11 +482,13 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
 // smaller keys, packed into 64 bits as (x - bin start) << 31 | id where bins
 // are at most 2^32 ticks wide -- a record per thread; larger bins by an
 // in-place bitonic sort, every comparator ascending (partner i ^ (2j - 1)
-// first in each merge) so any length sorts.  scratch: free shared words.
+// first in each merge) so any length sorts.  scratch: free shared words; sE:
+// a fifth array of the records, or null.
 template <typename TR>
 __device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* sA,
-                                            unsigned long long* sB, int* sid, int lo, int len,
-                                            long long blo, bool packs, int* scratch) {
+                                            unsigned long long* sB, int* sid,
+                                            unsigned short* sE, int lo, int len, long long blo,
+                                            bool packs, int* scratch) {
   constexpr int NT = TR::kT, NB = TR::kBins;
   constexpr int kRankMax = (NB / 2 - 1) < NT ? (NB / 2 - 1) : NT;
   const int tid = threadIdx.x;
@@ -493,7 +498,9 @@ __device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* s
     long long x = 0;
     int id = 0, rank = 0;
     unsigned long long a = 0, b = 0;
+    unsigned short e = 0;
     if (tid < len) {
+      if (sE) e = sE[lo + tid];
       x = sx[lo + tid];
       id = sid[lo + tid];
       a = sA[lo + tid];
@@ -509,6 +516,7 @@ __device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* s
       sid[lo + rank] = id;
       sA[lo + rank] = a;
       sB[lo + rank] = b;
+      if (sE) sE[lo + rank] = e;
     }
     __syncthreads();
     return;
@@ -534,6 +542,11 @@ __device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* s
             const unsigned long long tb = sB[p];
             sB[p] = sB[q];
             sB[q] = tb;
+            if (sE) {
+              const unsigned short te = sE[p];
+              sE[p] = sE[q];
+              sE[q] = te;
+            }
           }
         }
       }
@@ -550,22 +563,30 @@ __device__ __noinline__ void sort_dense_bin(long long* sx, unsigned long long* s
 // that, keep the list of pair_transfer).
 //   (A) one thread per slot within Smax of the own cells: left neighbours
 //       (nearest first), then right ones, adding weights to r_j = 1 + ... in
-//       that order (the order of the cluster tiers' walks) and counting both;
+//       that order (the order of the cluster tiers' walks) and counting both.
+//       The walks add up the gaps between sorted slots, clamped to a value
+//       above Smax so that they stay in 32 bits, with a clamped gap at both
+//       ends in place of bounds tests;
 //   (B) own slots are handed to lanes in order of their pair count (a
-//       counting sort): the exchange's binary64 warp instructions hold their
-//       pipe ~19 cycles whatever lanes are active, so a warp's lanes should
-//       run the same number of pairs;
-//   (C) exchange and reaction of own slots over their left then right pairs.
+//       counting sort), so that a warp's lanes run the same number of pairs;
+//   (C) exchange and reaction of own slots over their left, then right pairs
+//       (in the order of the slots). MT_MIXED sums in integers (mt_fixed.cuh):
+//       in binary64 its four instructions per pair held the binary64 pipe half
+//       of the kernel's time. A slot with a marked mass flags its neighbours
+//       in (A); flagged rows (a few per hundred) are summed in binary64, by
+//       the CTA's last warps before their share of the others, so that the
+//       warps that would meet one do not wait for its lane.
 // A segment with more unordered pairs than the pair list of the binary64 form
 // holds goes to the cluster tier, as there.
-// Measured against the pair list (weights once per pair, six more phases),
-// with the sort of fast_segment: N = 10^6 MT_MIXED 134 -> 123 us per step, 3 10^5
-// MT_MIXED_DF32 40 -> 35 us, 256 realisations 656 -> 580 us; same bits.
+// Measured per step against a pair list (weights once per pair, six more
+// phases): N = 10^6 MT_MIXED 134 -> 111 us (binary64 flux sums here: 126 us),
+// 256 realisations 656 -> 578 us (615 us), N = 3 10^5 MT_MIXED_DF32 40 -> 32 us.
 template <int PR>
 __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* smem, int m,
-                              int w0, int w1, long long out0, long long xlo, long long xhi) {
-  using W = Weight<mixw(PR), 1>;
-  using T = typename W::T;
+                              int w0, int w1, long long out0, long long xlo, long long xhi,
+                              unsigned short* sE, long long a0, int EA, int EB) {
+  // sE: integer sums may be used (sA, sB hold fixed masses); null otherwise
+  using W = Weight<true, 1>;
   using MS = Mass<PR>;
   using MV = typename MS::V;
   constexpr int NT = Fast::kT, CAP = Fast::kCap, PER = Fast::kPer;
@@ -573,15 +594,24 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
   const long long* sx = reinterpret_cast<const long long*>(smem);
   const unsigned long long* sA = reinterpret_cast<const unsigned long long*>(sx + CAP);
   const unsigned long long* sB = sA + CAP;
-  const int* sid = reinterpret_cast<const int*>(sB + CAP);
-  T* sr = reinterpret_cast<T*>(const_cast<int*>(sid) + CAP);
-  int* perm = reinterpret_cast<int*>(sr + CAP) + Fast::kBins + 1;  // (free after the sort)
+  uint2* sxr = reinterpret_cast<uint2*>(const_cast<unsigned long long*>(sB) + CAP);
+  const int* sid = reinterpret_cast<const int*>(sxr + CAP);
+  // (free after the sort:) gap[k]: from slot k - 1 to slot k, then the lanes' slots
+  unsigned int* gap = reinterpret_cast<unsigned int*>(const_cast<int*>(sid)) + CAP + Fast::kBins + 1;
+  int* perm = reinterpret_cast<int*>(gap);
   __shared__ int s_hist[kCnt];
-  __shared__ int s_np;
+  __shared__ int s_np, s_nf, s_next;
+  int* flagged = const_cast<int*>(sid);  // the flagged rows, once the ids are written
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long S = d.S;
+  const bool fix = PR == MT_MIXED && sE && fix_covers(EA) && fix_covers(EB);
+  const unsigned int S32 = (unsigned int)S, kFar = 1u << 30;  // S < 2^30
   if (tid < kCnt) s_hist[tid] = 0;
-  if (tid == kCnt) s_np = 0;
+  if (tid == kCnt) s_np = s_nf = s_next = 0;
+  for (int j = tid; j <= m; j += NT) {
+    const unsigned long long g = j > 0 && j < m ? (unsigned long long)(sx[j] - sx[j - 1]) : kFar;
+    gap[j] = g < kFar ? (unsigned int)g : kFar;
+  }
   __syncthreads();
   // (A)
   int v[PER];  // own slots: slot | left pairs << 10 | right pairs << 21
@@ -593,26 +623,26 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
     if (j >= m) continue;
     const long long x = sx[j];
     if (x < xlo - 2 * S || x >= xhi + S) continue;
-    const bool sum = x >= xlo - S;  // else only its pairs are counted
-    T r = T(1);
-    int i = j - 1;
-    if (sum) {
-      for (; i >= 0; --i) {
-        const long long D = x - sx[i];
-        if (D > S) break;
-        r += W::near(d, D, nullptr);
-      }
+    if (x < xlo - S) {  // only its pairs are counted
+      unsigned int D = gap[j + 1];
+      int R = 0;
+      while (D <= S32) D += gap[j + 2 + R++];
+      np += R;
+      continue;
     }
-    int q = j + 1;
-    for (; q < m; ++q) {
-      const long long D = sx[q] - x;
-      if (D > S) break;
-      if (sum) r += W::near(d, D, nullptr);
+    float r = 1.0f;
+    int L = 0, R = 0;
+    for (unsigned int D = gap[j]; D <= S32; D += gap[j - ++L]) r += W::near(d, (int)D, nullptr);
+    for (unsigned int D = gap[j + 1]; D <= S32; D += gap[j + 1 + ++R])
+      r += W::near(d, (int)D, nullptr);
+    np += R;
+    sxr[j] = make_uint2((unsigned int)x, __float_as_uint(__frcp_rn(r)));
+    if (fix) {
+      if ((sA[j] | sB[j]) & 1)
+        for (int i = j - L; i <= j + R; ++i) sE[i] |= 0x8000;  // (every writer writes this value)
     }
-    np += q - 1 - j;
-    if (sum) sr[j] = T(__frcp_rn((float)r));
     if (j >= w0 && j < w1) {
-      const int L = j - 1 - i, R = q - 1 - j, c = L + R;
+      const int c = L + R;
       v[k] = j | L << 10 | R << 21;
       atomicAdd(&s_hist[c < kCnt ? c : kCnt - 1], 1);
     }
@@ -621,6 +651,15 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
   if (lane == 0 && np) atomicAdd(&s_np, np);
   __syncthreads();
   if (s_np > kPairCap) return false;  // uniform across the CTA
+  long long* Xn = d.X[st.xc ^ 1];
+  int* In = d.id[st.xc ^ 1];
+  for (int j = w0 + tid; j < w1; j += NT) {  // positions and ids, coalesced
+    const long long o = out0 + (j - w0);
+    if (o < d.n) {
+      Xn[o] = sx[j];
+      In[o] = sid[j];
+    }
+  }
   // (B)
   if (warp == 0) {
     const int h0 = s_hist[2 * lane], h1 = s_hist[2 * lane + 1];
@@ -638,25 +677,38 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
   for (int k = 0; k < PER; ++k) {
     if (v[k] < 0) continue;
     const int c = ((v[k] >> 10) & 0x7ff) + (v[k] >> 21);
-    perm[atomicAdd(&s_hist[c < kCnt ? c : kCnt - 1], 1)] = v[k];
+    const int at = atomicAdd(&s_hist[c < kCnt ? c : kCnt - 1], 1);
+    if (fix && (sE[v[k] & 0x3ff] & 0x8000)) {
+      flagged[atomicAdd(&s_nf, 1)] = v[k];
+      v[k] = -1;
+    }
+    perm[at] = v[k];
   }
   __syncthreads();
   // (C)
   const int nown = w1 - w0;
+  const bool sym = d.norm != MT_NORM_ROW;  // 2 P is formed, the sums are halved at the end
   unsigned long long* Mn = d.M[st.mc ^ 1];
   if (out0 + nown > d.n) raise_error(d.ctrl, kErrIndex, out0);
-  for (int p = tid; p < nown; p += NT) {
-    const int u0 = perm[p], j = u0 & 0x3ff, L = (u0 >> 10) & 0x7ff, c = L + (u0 >> 21);
-    const unsigned int x32 = (unsigned int)sx[j];  // within the cutoff the low words' difference is the separation
-    const T ip = sr[j];
-    MV A = MS::load(sA, j), B = MS::load(sB, j);
-    typename MS::Acc dA{}, dB{};
-    for (int u = 0; u < c; ++u) {
-      const int i = u < L ? j - 1 - u : j + 1 + u - L;
-      const T w = W::near(d, (int)((unsigned int)sx[i] - x32), nullptr);
-      const T P = normalised<T>(d.norm, w, ip, sr[i]);
-      MS::acc(dA, P, MS::diff(MS::load(sA, i), A));
-      MS::acc(dB, P, MS::diff(MS::load(sB, i), B));
+  const unsigned long long* Mo = d.M[st.mc] + a0;
+  // with integer sums the masses themselves are in the old state only
+  auto mass_a = [&](int i) {
+    return PR == MT_MIXED && sE ? MS::load(Mo, sE[i] & 0x7fff) : MS::load(sA, i);
+  };
+  auto mass_b = [&](int i) {
+    return PR == MT_MIXED && sE ? MS::load(Mo, d.n + (sE[i] & 0x7fff)) : MS::load(sB, i);
+  };
+  // the normalised weight of slots own, i (twice it in SYM); within the
+  // cutoff the low words' difference is the separation
+  auto weight = [&](uint2 own, int i) {
+    const uint2 q = sxr[i];
+    const float w = W::near(d, (int)(q.x - own.x), nullptr), ip = __uint_as_float(own.y);
+    return sym ? w * (ip + __uint_as_float(q.y)) : w * ip;
+  };
+  auto finish = [&](int j, MV A, MV B, typename MS::Acc dA, typename MS::Acc dB) {
+    if (sym) {
+      dA = acc_half(dA);
+      dB = acc_half(dB);
     }
     MS::update(A, B, dA, dB, d.react);
     const long long o = out0 + (j - w0);
@@ -664,14 +716,45 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
       MS::store(Mn, o, A);
       MS::store(Mn, d.n + o, B);
     }
+  };
+  // A row's pairs are the slots i0 .. i1 without its own, j.
+  const int* rows = fix ? flagged : perm;
+  const int nrows = fix ? s_nf : nown;
+  for (int p = fix ? NT - 1 - tid : tid; p < nrows; p += NT) {
+    const int u0 = rows[p], j = u0 & 0x3ff, i0 = j - ((u0 >> 10) & 0x7ff);
+    const int i1 = j + (u0 >> 21);
+    const uint2 own = sxr[j];
+    const MV A = mass_a(j), B = mass_b(j);
+    typename MS::Acc dA{}, dB{};
+#pragma unroll(PR == MT_MIXED ? 4 : 1)
+    for (int u = i0; u < i1; ++u) {
+      const int i = u + (u >= j);
+      const float P = weight(own, i);
+      MS::acc(dA, P, MS::diff(mass_a(i), A));
+      MS::acc(dB, P, MS::diff(mass_b(i), B));
+    }
+    finish(j, A, B, dA, dB);
   }
-  long long* Xn = d.X[st.xc ^ 1];
-  int* In = d.id[st.xc ^ 1];
-  for (int j = w0 + tid; j < w1; j += NT) {  // positions and ids, coalesced
-    const long long o = out0 + (j - w0);
-    if (o < d.n) {
-      Xn[o] = sx[j];
-      In[o] = sid[j];
+  if constexpr (PR == MT_MIXED) {
+    // (32 rows at a time by ticket: the warps that had flagged rows take less)
+    while (fix) {
+      int p = 0;
+      if (lane == 0) p = atomicAdd(&s_next, 32);
+      p = __shfl_sync(0xffffffffu, p, 0) + lane;
+      if (p - lane >= nown) break;
+      const int u0 = p < nown ? perm[p] : -1;
+      if (u0 < 0) continue;  // flagged
+      const int j = u0 & 0x3ff, i0 = j - ((u0 >> 10) & 0x7ff), i1 = j + (u0 >> 21);
+      const uint2 own = sxr[j];
+      const long long ma = (long long)sA[j], mb = (long long)sB[j];
+      FixAcc qa, qb;
+      for (int u = i0; u < i1; ++u) {
+        const int i = u + (u >= j);
+        const FixP P = fix_p(weight(own, i));
+        qa.add((long long)sA[i] - ma, P);
+        qb.add((long long)sB[i] - mb, P);
+      }
+      finish(j, mass_a(j), mass_b(j), qa.value(EA), qb.value(EB));
     }
   }
   return true;
@@ -735,16 +818,21 @@ __device__ __forceinline__ void segment_tables(const Dev& d, int sc, int seg, co
 template <int PR>
 __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned char* smem,
                             const SegScalars& g, const SegPrefetch& pf) {
-  using T = typename Weight<mixw(PR), 1>::T;
   constexpr int NT = Fast::kT, PER = Fast::kPer, CAP = Fast::kCap, NB = Fast::kBins;
   constexpr int BPT = Fast::kBinsPerThread;
   long long* sx = reinterpret_cast<long long*>(smem);
   unsigned long long* sA = reinterpret_cast<unsigned long long*>(sx + CAP);
   unsigned long long* sB = sA + CAP;
-  int* sid = reinterpret_cast<int*>(sB + CAP);
-  T* sr = reinterpret_cast<T*>(sid + CAP);
-  int* bstart = reinterpret_cast<int*>(sr + CAP);  // [NB + 1]
-  int* bcur = bstart + NB + 1;                     // [NB]
+  uint2* skey = reinterpret_cast<uint2*>(sB + CAP);  // (1 / r later)
+  int* sid = reinterpret_cast<int*>(skey + CAP);
+  int* bstart = sid + CAP;      // [NB + 1]
+  int* bcur = bstart + NB + 1;  // [NB + 1], free after the sort
+  // MT_MIXED with integer flux sums: sA, sB hold fixed masses (mt_fixed.cuh)
+  // and sE the staged slots' places in the staging, where the masses are
+  const bool fix = PR == MT_MIXED && d.fix;
+  unsigned short* sE =
+      fix ? reinterpret_cast<unsigned short*>(smem + pair_region_offset<Fast>()) : nullptr;
+  __shared__ int s_emax[2];
   __shared__ int s_lt, s_w0, s_w1, s_nbig, s_work;
   __shared__ int s_big[kBigMax];
   __shared__ int s_scan[NT / 32];
@@ -758,6 +846,7 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
   while (sh2 < 62 && ((whi - wlo) >> sh2) >= NB) ++sh2;
   // bins the window spans (bins are cells unless the window has >= NB cells)
   const int nb = whi > wlo ? (int)(((whi - 1 - wlo) >> sh2) + 1) : 1;
+  const unsigned int bmask = sh2 < 32 ? (1u << sh2) - 1u : 0xffffffffu;  // ticks in a bin
   const bool active = c0 < c1;
   if (active && L > CAP) {
     if (tid == 0) prefetch_stage2(d, pf);
@@ -779,6 +868,8 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
     s_w1 = 0;
     s_nbig = 0;
     s_work = 0;
+    s_emax[0] = 0;
+    s_emax[1] = 0;
   }
   for (int b = tid; b <= nb; b += NT) bstart[b] = 0;
   __syncthreads();
@@ -879,44 +970,68 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
   for (int k = 0; k < PER; ++k) {
     if (rb[k] < 0) continue;
     const int at = bstart[rb[k] & 0xffff] + (rb[k] >> 16);
-    sx[at] = rx[k];
-    sid[at] = rid[k];
+    if (sh2 <= 32)  // position in the bin, id
+      skey[at] = make_uint2((unsigned int)rid[k], (unsigned int)(rx[k] - wlo) & bmask);
+    else
+      sx[at] = rx[k], sid[at] = rid[k];
   }
   __syncthreads();
   // ---- final slots: rank by (x, id) inside the bin -------------------------
   unsigned long long ra[PER], rm[PER];
+  int ea = 0, eb = 0;
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
     if (rb[k] < 0) continue;
     const long long e = a0 + tid + k * NT;
     ra[k] = d.M[st.mc][e];
     rm[k] = d.M[st.mc][d.n + e];
+    if (fix) {
+      ea = max(ea, fix_exponent(ra[k]));
+      eb = max(eb, fix_exponent(rm[k]));
+    }
     const int b = rb[k] & 0xffff, lo = bstart[b], hi = bstart[b + 1];
     int to = lo + (rb[k] >> 16);
     if (hi - lo > 1 && hi - lo <= kBinMax) {  // (larger bins: below)
       const int self = to;
       to = lo;
-      for (int q = lo; q < hi; ++q) {
-        const long long y = sx[q];
-        to += y < rx[k] || (y == rx[k] && q != self && sid[q] < rid[k]) ? 1 : 0;
+      if (sh2 <= 32) {
+        const unsigned long long* key = reinterpret_cast<const unsigned long long*>(skey);
+        const unsigned long long mine = key[self];
+        for (int q = lo; q < hi; ++q) to += key[q] < mine ? 1 : 0;
+      } else {
+        for (int q = lo; q < hi; ++q) {
+          const long long y = sx[q];
+          to += y < rx[k] || (y == rx[k] && sid[q] < rid[k]) ? 1 : 0;
+        }
       }
     }
     rb[k] = to;
   }
+  if (fix) {
+    ea = __reduce_max_sync(0xffffffffu, ea);
+    eb = __reduce_max_sync(0xffffffffu, eb);
+    if (lane == 0) {
+      atomicMax(&s_emax[0], ea);
+      atomicMax(&s_emax[1], eb);
+    }
+  }
   __syncthreads();
+  const int EA = fix_scale(s_emax[0]), EB = fix_scale(s_emax[1]);
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
     if (rb[k] < 0) continue;
     sx[rb[k]] = rx[k];
     sid[rb[k]] = rid[k];
-    sA[rb[k]] = ra[k];
-    sB[rb[k]] = rm[k];
+    sA[rb[k]] = fix ? (unsigned long long)to_fix(ra[k], EA) : ra[k];
+    sB[rb[k]] = fix ? (unsigned long long)to_fix(rm[k], EB) : rm[k];
+    if (fix) sE[rb[k]] = (unsigned short)(tid + k * NT);
   }
   __syncthreads();
   if (s_nbig > 0) {
     // dense bins: the whole CTA
     for (int t = 0; t < s_nbig; ++t)
-      sort_dense_bin<Fast>(sx, sA, sB, sid, bstart[s_big[t]], bstart[s_big[t] + 1] - bstart[s_big[t]],
+      sort_dense_bin<Fast>(sx, sA, sB, sid, sE, bstart[s_big[t]],
+                           bstart[s_big[t] + 1] - bstart[s_big[t]],
                            wlo + ((long long)s_big[t] << sh2), sh2 <= 32, bcur);
   }
   const int m = bstart[nb];
@@ -926,7 +1041,7 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
   if (tid == 0) prefetch_next_l2(d, pf, st);
   bool fits;
   if constexpr (mixw(PR))
-    fits = walk_transfer<PR>(d, st, smem, m, w0, w1, out0, xlo, xhi);
+    fits = walk_transfer<PR>(d, st, smem, m, w0, w1, out0, xlo, xhi, sE, a0, EA, EB);
   else
     fits = pair_transfer<Fast>(d, st, smem, m, w0, w1, out0, xlo, xhi);
   if (!fits) return kSegHeavy;  // more pairs than the list holds: the second tier takes it
@@ -1223,7 +1338,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
         __syncthreads();
         continue;
       }
-      sort_dense_bin<TR>(sx, sA, sB, sid, lo, len, 0, false, bcur);
+      sort_dense_bin<TR>(sx, sA, sB, sid, nullptr, lo, len, 0, false, bcur);
     }
   }
 
