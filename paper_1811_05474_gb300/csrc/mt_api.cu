@@ -814,7 +814,6 @@ mt_status mt_batch_create(const mt_params* p, const mt_batch* b, void* workspace
   d.rinv = w + D.o_rinv;
   d.count = reinterpret_cast<int*>(w + D.o_count);
   d.start = reinterpret_cast<int*>(w + D.o_start);
-  d.cursor = reinterpret_cast<int*>(w + D.o_cursor);
   d.scan_status = reinterpret_cast<unsigned long long*>(w + D.o_status);
   d.big = reinterpret_cast<int*>(w + D.o_big);
   d.obs = reinterpret_cast<double*>(w + D.o_obs);

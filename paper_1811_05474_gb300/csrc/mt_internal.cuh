@@ -103,7 +103,6 @@ struct Dev {
   void* rinv;               // 1 / r_i (double in FP64, float in MIXED)
   int* count;               // [ncell] particles per cell
   int* start;               // [ncell + 1] first slot of each cell
-  int* cursor;              // [ncell] scatter cursor
   unsigned long long* scan_status;  // [ntiles] look-back words
   int* big;                 // [nbig_cap] cells for the large-cell sort
   int* ochunk;              // [nochunk + 1] first slot of each observables chunk
@@ -377,10 +376,24 @@ __device__ __forceinline__ double rcp_ge1(double r) {
   return __fma_rn(y, __fma_rn(-r, y, 1.0), y);
 }
 
+// The nearest integer to v (ties to even), as __double2ll_rn, from v's bits with
+// integer operations for 2^-1 <= |v| < 2^52 (the conversion instruction holds
+// the binary64 pipe like an arithmetic one).
+__device__ __forceinline__ long long rint_exact(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  const int sh = 1075 - (int)((u >> 52) & 0x7ff);  // bits below the unit
+  if (sh < 1 || sh > 53) return __double2ll_rn(v);
+  const unsigned long long m = (u & ((1ULL << 52) - 1)) | (1ULL << 52);
+  const unsigned long long q =
+      (m + ((1ULL << (sh - 1)) - 1) + ((m >> sh) & 1)) >> sh;
+  return (long long)u < 0 ? -(long long)q : (long long)q;
+}
+
 // Eq. 2's random-walk displacement on the grid: the nearest tick to b xi,
-// b = sqrt(2 D_rw dt) 2^k, with the product formed in binary64.
+// b = sqrt(2 D_rw dt) 2^k, with the product formed in binary64 (the one
+// binary64 instruction here).
 __device__ __forceinline__ long long walk_ticks(double b, float xi) {
-  return __double2ll_rn(__dmul_rn(b, (double)xi));
+  return rint_exact(__dmul_rn(b, widen_exact(xi)));
 }
 
 // Two standard normals from two 32-bit words (Box-Muller, binary32, with

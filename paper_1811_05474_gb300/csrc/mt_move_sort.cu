@@ -26,18 +26,26 @@ __global__ void __launch_bounds__(kThreads) k_move(Dev d) {
   if (MOVE) {
     const int id = d.id[xc][p];
     // realisation of the particle (always 0 in 2-d, where base = 0)
-    const Real* R = d.rt + (id >> d.lbits);
-    const int loc = id & d.lmask;
-    const long long base = R->base;
+    long long base = 0, Lq = d.rLq, off = 0;
+    unsigned int real = d.rreal;
+    int loc = id;
+    if (DIM == 1 && !d.single) {
+      const Real* R = d.rt + (id >> d.lbits);
+      base = R->base;
+      Lq = R->Lq;
+      off = R->off;
+      real = R->real;
+      loc &= d.lmask;
+    }
     float z[2];
     const float* noise = c->noise;
     if (noise) {
-      z[0] = noise[R->off + loc];
+      z[0] = noise[off + loc];
       if (DIM == 2) z[1] = noise[d.n + loc];
     } else {
       const unsigned long long st = c->step;
       const uint4 u = philox4x32_10(
-          make_uint4((unsigned int)loc, (unsigned int)st, (unsigned int)(st >> 32), R->real),
+          make_uint4((unsigned int)loc, (unsigned int)st, (unsigned int)(st >> 32), real),
           d.key0, d.key1);
       const float2 g = box_muller(u.x, u.y);
       z[0] = g.x;
@@ -48,24 +56,30 @@ __global__ void __launch_bounds__(kThreads) k_move(Dev d) {
       // Eq. 2 on the grid: drift + rint(b * xi), then the wall mirror.
       const long long step = walk_ticks(d.bq, z[a]);
       if (d.periodic && a == 0)
-        pos[0] = base + wrap(pos[0] - base + d.drift[0] + step, R->Lq);
+        pos[0] = base + wrap(pos[0] - base + d.drift[0] + step, Lq);
       else if (d.periodic)
         pos[a] = wrap(pos[a] + d.drift[a] + step, d.Lq[a]);
       else if (a == 0)
-        pos[0] = base + reflect(pos[0] - base + d.drift[0] + step, R->Lq);
+        pos[0] = base + reflect(pos[0] - base + d.drift[0] + step, Lq);
       else
         pos[a] = reflect(pos[a] + d.drift[a] + step, d.Lq[a]);
       X[(long long)a * d.n + p] = pos[a];
     }
   }
-  if (HIST) atomicAdd(&d.count[cell_of(d, pos[0], pos[1])], 1);
+  // its arrival number in the cell (kept in rinv until the row sums)
+  if (HIST)
+    static_cast<int*>(d.rinv)[p] = atomicAdd(&d.count[cell_of(d, pos[0], pos[1])], 1);
 }
 
 // ------------------------------------------------------------------ scan --
-// Exclusive scan of count[] into start[] and cursor[] (and count[] := 0),
-// one pass with decoupled look-back.  Tiles are handed out in launch order
-// by a ticket, so a tile only waits on tiles already running; the wait is
-// bounded anyway and raises kErrTimeout instead of hanging.
+// Exclusive scan of count[] into start[] (and count[] := 0), one pass with
+// decoupled look-back.  Tiles are handed out in launch order by a ticket, so
+// a tile only waits on tiles already running; the wait is bounded anyway and
+// raises kErrTimeout instead of hanging.  A warp takes 512 consecutive counts,
+// four per lane and load (coalesced 16-byte accesses), and the tile's first
+// warp looks back over 32 status words at a time.  Bound: 8 bytes read and 8
+// written per cell; 1.56 10^6 cells: 36 -> 14 us (a thread's 16 consecutive
+// counts one by one, one thread looking back word by word).
 // Status word: [63:48] epoch tag, [47:46] flag (1 aggregate, 2 prefix),
 // [45:0] value.
 __device__ __forceinline__ unsigned long long pack(unsigned long long tag, unsigned long long flag,
@@ -73,120 +87,185 @@ __device__ __forceinline__ unsigned long long pack(unsigned long long tag, unsig
   return (tag << 48) | (flag << 46) | ((unsigned long long)v & ((1ULL << 46) - 1));
 }
 
+__device__ __forceinline__ int warp_inclusive(int v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+
 __global__ void __launch_bounds__(kThreads) k_scan(Dev d) {
+  constexpr int kWarps = kThreads / 32, kVec = kScanItems / 4;
   __shared__ int s_tile;
-  __shared__ long long s_warp[kThreads / 32];
+  __shared__ int s_warp[kWarps];
   __shared__ long long s_excl;
   Ctrl* c = d.ctrl;
   if (threadIdx.x == 0) s_tile = (int)atomicAdd(&c->tile_ctr, 1u);
   __syncthreads();
   const long long tile = s_tile;
-  const long long base = tile * kScanTile + (long long)threadIdx.x * kScanItems;
-  int v[kScanItems];
-  long long mine = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long k = base + i;
-    v[i] = k < d.ncell ? d.count[k] : 0;
-    mine += v[i];
-  }
-  // block-wide exclusive scan of the per-thread sums
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  long long inc = mine;
+  // counts k0 + 128 i + 4 lane .. + 3 (at most 2^31 particles in all)
+  const long long k0 = tile * kScanTile + warp * (32 * kScanItems) + 4 * lane;
+  int4 v[kVec];
+  int excl[kVec];  // within the warp's counts
+  int run = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    long long w = lane < kThreads / 32 ? s_warp[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long t = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += t;
+  for (int i = 0; i < kVec; ++i) {
+    const long long k = k0 + 128 * i;
+    if (k + 3 < d.ncell) {
+      v[i] = *reinterpret_cast<const int4*>(d.count + k);
+      *reinterpret_cast<int4*>(d.count + k) = make_int4(0, 0, 0, 0);
+    } else {
+      int w[4];
+      for (int e = 0; e < 4; ++e) {
+        w[e] = k + e < d.ncell ? d.count[k + e] : 0;
+        if (k + e < d.ncell) d.count[k + e] = 0;
+      }
+      v[i] = make_int4(w[0], w[1], w[2], w[3]);
     }
-    if (lane < kThreads / 32) s_warp[lane] = w;  // inclusive warp totals
   }
+#pragma unroll
+  for (int i = 0; i < kVec; ++i) {
+    const int sum = v[i].x + v[i].y + v[i].z + v[i].w;
+    const int inc = warp_inclusive(sum, lane);
+    excl[i] = run + inc - sum;
+    run += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  if (lane == 0) s_warp[warp] = run;
   __syncthreads();
-  const long long block_total = s_warp[kThreads / 32 - 1];
-  const long long thread_excl = inc - mine + (warp > 0 ? s_warp[warp - 1] : 0);
-  if (threadIdx.x == 0) {
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    if (w < warp) before += s_warp[w];
+    total += s_warp[w];
+  }
+  if (warp == 0) {
     const unsigned long long tag = (c->epoch % 65535ULL) + 1ULL;
     volatile unsigned long long* st = d.scan_status;
-    long long excl = 0;
+    long long sum = 0;
     if (tile == 0) {
       // (the test hook withholds this word: every later tile's wait then
       // runs out and raises kErrTimeout)
-      if (!c->scan_hold) atomicExch(&d.scan_status[0], pack(tag, 2, block_total));
+      if (lane == 0 && !c->scan_hold) atomicExch(&d.scan_status[0], pack(tag, 2, total));
     } else {
-      atomicExch(&d.scan_status[tile], pack(tag, 1, block_total));
+      if (lane == 0) atomicExch(&d.scan_status[tile], pack(tag, 1, total));
       const long long limit = c->spin_limit > 0 ? c->spin_limit : kSpinLimit;
       long long t = tile - 1, spins = 0;
-      while (t >= 0) {
-        const unsigned long long w = st[t];
+      for (;;) {  // tiles t, t - 1, ... t - 31 (before tile 0: an empty prefix)
+        const unsigned long long w = t - lane >= 0 ? st[t - lane] : pack(tag, 2, 0);
         const unsigned long long flag = (w >> 46) & 3ULL;
-        if ((w >> 48) != tag || flag == 0) {
+        const bool ready = (w >> 48) == tag && flag != 0;
+        const unsigned int prefix = __ballot_sync(0xffffffffu, ready && flag == 2);
+        const unsigned int missing = __ballot_sync(0xffffffffu, !ready);
+        const int last = prefix ? __ffs(prefix) - 1 : 31;  // words up to the first prefix count
+        if (missing & (0xffffffffu >> (31 - last))) {
           if (++spins > limit) {
-            raise_error(c, kErrTimeout, tile);
+            if (lane == 0) raise_error(c, kErrTimeout, tile);
             break;
           }
           continue;
         }
-        excl += (long long)(w & ((1ULL << 46) - 1));
-        if (flag == 2) break;
-        --t;
+        long long part = lane <= last ? (long long)(w & ((1ULL << 46) - 1)) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        sum += part;
+        if (prefix) break;
+        t -= 32;
       }
-      atomicExch(&d.scan_status[tile], pack(tag, 2, excl + block_total));
+      if (lane == 0) atomicExch(&d.scan_status[tile], pack(tag, 2, sum + total));
     }
-    s_excl = excl;
+    if (lane == 0) s_excl = sum;
   }
   __syncthreads();
-  long long run = s_excl + thread_excl;
+  const int base = (int)s_excl + before;
 #pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long k = base + i;
-    if (k < d.ncell) {
-      d.start[k] = (int)run;
-      d.cursor[k] = (int)run;
-      d.count[k] = 0;
-      run += v[i];
-      if (k == d.ncell - 1) d.start[d.ncell] = (int)run;
+  for (int i = 0; i < kVec; ++i) {
+    const long long k = k0 + 128 * i;
+    int4 o;
+    o.x = base + excl[i];
+    o.y = o.x + v[i].x;
+    o.z = o.y + v[i].y;
+    o.w = o.z + v[i].z;
+    if (k + 3 < d.ncell) {
+      *reinterpret_cast<int4*>(d.start + k) = o;
+    } else {
+      const int w[4] = {o.x, o.y, o.z, o.w};
+      for (int e = 0; e < 4; ++e)
+        if (k + e < d.ncell) d.start[k + e] = w[e];
+    }
+    // the end of the last cell
+    if (d.ncell - 1 >= k && d.ncell - 1 < k + 4) {
+      const int e = (int)(d.ncell - 1 - k);
+      d.start[d.ncell] = e == 0 ? o.y : e == 1 ? o.z : e == 2 ? o.w : o.w + v[i].w;
     }
   }
 }
 
 // --------------------------------------------------------------- scatter --
+// The slot before the sort into its cell's slots, in arrival order (1-d: the
+// position too).
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_scatter(Dev d) {
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur;
   const long long* X = d.X[xc];
-  long long* Y = d.X[xc ^ 1];
   const long long x = X[p], y = DIM == 2 ? X[d.n + p] : 0;
-  const long long slot = atomicAdd(&d.cursor[cell_of(d, x, y)], 1);
+  const long long slot = (long long)d.start[cell_of(d, x, y)] + static_cast<const int*>(d.rinv)[p];
   if (slot < 0 || slot >= d.n) {
     raise_error(d.ctrl, kErrIndex, slot);
     return;
   }
-  Y[slot] = x;
-  if (DIM == 2) Y[d.n + slot] = y;
+  if (DIM == 1) d.X[xc ^ 1][slot] = x;
   d.src[slot] = (int)p;
 }
 
-// ------------------------------------------------------------- cell sort --
-// Order inside a cell: by (x, src) in 1-d, which makes the whole array
-// sorted by position; by src in 2-d.  src is the slot before the sort, so
-// the result does not depend on the order the atomics handed out slots.
-template <int DIM>
-__device__ __forceinline__ bool before(long long xa, int sa, long long xb, int sb) {
-  if (DIM == 1) return xa < xb || (xa == xb && sa < sb);
-  return sa < sb;
+// 2-d: a particle's final slot is its cell's first slot plus the number of the
+// cell's particles with a smaller src (the slot before the sort), which makes
+// the order unique whatever order they arrived in; it takes its position, id
+// and masses (every species) there.  One thread per particle: a cell of m
+// particles costs m^2 reads of src, less than the m^2 pair tests that the two
+// transfer passes spend on it (a cell is wider than the cutoff).  Bound: the
+// chain of dependent reads src, position, cell start (10^6 particles: 16 us;
+// with the large cells' sort and the gather of ids and masses, which the row
+// sums did, it takes the place of 25 us; two particles per thread: no faster).
+__global__ void __launch_bounds__(kThreads) k_place2(Dev d) {
+  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
+  if (p >= d.n) return;
+  const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
+  const long long s = d.src[p];
+  if (s < 0 || s >= d.n) {  // (a scan that timed out leaves slots unset)
+    raise_error(d.ctrl, kErrIndex, s);
+    return;
+  }
+  const long long* X = d.X[xc];
+  const long long x = X[s], y = X[d.n + s];
+  const long long c = cell_of(d, x, y);
+  const int a = max(d.start[c], 0), b = (int)min((long long)d.start[c + 1], d.n);
+  long long f = a;
+  for (int q = a; q < b; ++q) f += d.src[q] < s ? 1 : 0;
+  if (f >= d.n) {
+    raise_error(d.ctrl, kErrIndex, f);
+    return;
+  }
+  long long* Y = d.X[xc ^ 1];
+  Y[f] = x;
+  Y[d.n + f] = y;
+  d.id[xc ^ 1][f] = d.id[xc][s];
+  gather_masses(d, mc, f, s);
+  gather_species(d, mc, f, s);
 }
 
-template <int DIM>
+// ------------------------------------------------------------- cell sort --
+// 1-d: order inside a cell by (x, src), which makes the whole array sorted by
+// position.  src is the slot before the sort, so the result does not depend
+// on the order of arrival.
+__device__ __forceinline__ bool before(long long xa, int sa, long long xb, int sb) {
+  return xa < xb || (xa == xb && sa < sb);
+}
+
 __global__ void __launch_bounds__(kThreads) k_cellsort(Dev d) {
   const long long k = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (k >= d.ncell) return;
@@ -205,17 +284,14 @@ __global__ void __launch_bounds__(kThreads) k_cellsort(Dev d) {
   int* src = d.src;
   for (int i = a + 1; i < b; ++i) {
     const long long xi = X[i];
-    const long long yi = DIM == 2 ? X[d.n + i] : 0;
     const int si = src[i];
     int j = i - 1;
-    while (j >= a && before<DIM>(xi, si, X[j], src[j])) {
+    while (j >= a && before(xi, si, X[j], src[j])) {
       X[j + 1] = X[j];
-      if (DIM == 2) X[d.n + j + 1] = X[d.n + j];
       src[j + 1] = src[j];
       --j;
     }
     X[j + 1] = xi;
-    if (DIM == 2) X[d.n + j + 1] = yi;
     src[j + 1] = si;
   }
 }
@@ -223,11 +299,9 @@ __global__ void __launch_bounds__(kThreads) k_cellsort(Dev d) {
 // Large cells: one CTA per cell, bitonic sort with every comparator
 // ascending (partner i ^ (2j - 1) in the first stage of each merge), which
 // sorts any length when positions >= len are treated as +infinity.
-template <int DIM>
 __global__ void __launch_bounds__(1024) k_bigsort(Dev d) {
   __shared__ long long s_key[kBigSortCap];
   __shared__ int s_src[kBigSortCap];
-  __shared__ int s_idx[kBigSortCap];
   Ctrl* c = d.ctrl;
   const int nbig = min(c->nbig, d.nbig_cap);
   long long* X = d.X[c->xcur ^ 1];
@@ -236,79 +310,48 @@ __global__ void __launch_bounds__(1024) k_bigsort(Dev d) {
     const long long k = d.big[b];
     const int a = d.start[k];
     const int len = d.start[k + 1] - a;
-    if (len <= kBigSortCap) {
-      int np2 = 1;
-      while (np2 < len) np2 <<= 1;
+    const bool shared = len <= kBigSortCap;
+    long long* key = shared ? s_key : X + a;
+    int* tag = shared ? s_src : src + a;
+    if (shared) {
       for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        s_key[i] = DIM == 1 ? X[a + i] : 0;
+        s_key[i] = X[a + i];
         s_src[i] = src[a + i];
-        s_idx[i] = i;
       }
-      __syncthreads();
-      for (int m = 2; m <= np2; m <<= 1) {
-        for (int j = m >> 1; j > 0; j >>= 1) {
-          for (int i = threadIdx.x; i < np2; i += blockDim.x) {
-            const int l = (j == (m >> 1)) ? (i ^ (m - 1)) : (i ^ j);
-            if (l > i && l < len) {
-              if (before<DIM>(s_key[l], s_src[l], s_key[i], s_src[i])) {
-                const long long tk = s_key[i]; s_key[i] = s_key[l]; s_key[l] = tk;
-                const int ts = s_src[i]; s_src[i] = s_src[l]; s_src[l] = ts;
-                const int ti = s_idx[i]; s_idx[i] = s_idx[l]; s_idx[l] = ti;
-              }
+    }
+    __syncthreads();
+    long long np2 = 1;
+    while (np2 < len) np2 <<= 1;
+    for (long long m = 2; m <= np2; m <<= 1) {
+      for (long long j = m >> 1; j > 0; j >>= 1) {
+        for (long long i = threadIdx.x; i < np2; i += blockDim.x) {
+          const long long l = (j == (m >> 1)) ? (i ^ (m - 1)) : (i ^ j);
+          if (l > i && l < len) {
+            const long long xi = key[i], xl = key[l];
+            if (before(xl, tag[l], xi, tag[i])) {
+              key[i] = xl;
+              key[l] = xi;
+              const int ts = tag[i];
+              tag[i] = tag[l];
+              tag[l] = ts;
             }
           }
-          __syncthreads();
         }
+        __syncthreads();
       }
-      // apply the permutation: gather into registers, then write
-      long long ry[kBigSortCap / 1024 + 1];
-      long long rx[kBigSortCap / 1024 + 1];
-      int t = 0;
-      for (int i = threadIdx.x; i < len; i += blockDim.x, ++t) {
-        rx[t] = X[a + s_idx[i]];
-        if (DIM == 2) ry[t] = X[d.n + a + s_idx[i]];
-      }
-      __syncthreads();
-      t = 0;
-      for (int i = threadIdx.x; i < len; i += blockDim.x, ++t) {
-        X[a + i] = rx[t];
-        if (DIM == 2) X[d.n + a + i] = ry[t];
+    }
+    if (shared) {
+      for (int i = threadIdx.x; i < len; i += blockDim.x) {
+        X[a + i] = s_key[i];
         src[a + i] = s_src[i];
       }
       __syncthreads();
-    } else {
-      // same network directly on global memory (very large cells only)
-      long long np2l = 1;
-      while (np2l < len) np2l <<= 1;
-      for (long long m = 2; m <= np2l; m <<= 1) {
-        for (long long j = m >> 1; j > 0; j >>= 1) {
-          for (long long i = threadIdx.x; i < np2l; i += blockDim.x) {
-            const long long l = (j == (m >> 1)) ? (i ^ (m - 1)) : (i ^ j);
-            if (l > i && l < len) {
-              const long long xi = X[a + i], xl = X[a + l];
-              if (before<DIM>(xl, src[a + l], xi, src[a + i])) {
-                X[a + i] = xl;
-                X[a + l] = xi;
-                if (DIM == 2) {
-                  const long long yi = X[d.n + a + i];
-                  X[d.n + a + i] = X[d.n + a + l];
-                  X[d.n + a + l] = yi;
-                }
-                const int ts = src[a + i];
-                src[a + i] = src[a + l];
-                src[a + l] = ts;
-              }
-            }
-          }
-          __syncthreads();
-        }
-      }
     }
   }
 }
 
 // ------------------------------------------------------------- permute --
-// After a sort without a transfer (upload): gather id and masses into the
+// After a 1-d sort without a transfer (upload): gather id and masses into the
 // sorted slots, then the next kernel flips the selectors.
 __global__ void __launch_bounds__(kThreads) k_permute(Dev d) {
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
@@ -359,29 +402,24 @@ cudaError_t launch_sort(const Dev& d, cudaStream_t s, Marker& mk) {
   mk("scan", s);
   k_scan<<<gs, kThreads, 0, s>>>(d);
   const unsigned int gp = blocks_for(d.n, kThreads);
-  const unsigned int gc = blocks_for(d.ncell, kThreads);
-  const unsigned int gb = (unsigned int)(d.nbig_cap < 304 ? d.nbig_cap : 304);
+  mk("scatter", s);
   if (d.dim == 1) {
-    mk("scatter", s);
     k_scatter<1><<<gp, kThreads, 0, s>>>(d);
     mk("cellsort", s);
-    k_cellsort<1><<<gc, kThreads, 0, s>>>(d);
+    k_cellsort<<<blocks_for(d.ncell, kThreads), kThreads, 0, s>>>(d);
     mk("bigsort", s);
-    k_bigsort<1><<<gb, 1024, 0, s>>>(d);
+    k_bigsort<<<(unsigned int)(d.nbig_cap < 304 ? d.nbig_cap : 304), 1024, 0, s>>>(d);
   } else {
-    mk("scatter", s);
     k_scatter<2><<<gp, kThreads, 0, s>>>(d);
-    mk("cellsort", s);
-    k_cellsort<2><<<gc, kThreads, 0, s>>>(d);
-    mk("bigsort", s);
-    k_bigsort<2><<<gb, 1024, 0, s>>>(d);
+    mk("place", s);
+    k_place2<<<gp, kThreads, 0, s>>>(d);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_permute(const Dev& d, cudaStream_t s) {
-  k_permute<<<blocks_for(d.n, kThreads), kThreads, 0, s>>>(d);
-  k_flip<<<1, 1, 0, s>>>(d, 1, 1);
+  if (d.dim == 1) k_permute<<<blocks_for(d.n, kThreads), kThreads, 0, s>>>(d);
+  k_flip<<<1, 1, 0, s>>>(d, 1, 1);  // (2-d: placed by the sort)
   return cudaGetLastError();
 }
 

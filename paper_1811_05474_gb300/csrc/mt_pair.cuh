@@ -270,14 +270,27 @@ struct Mass<MT_FP64> {
                                                 int react) {
     A = __fma_rn(0.5, dA, A);  // 0.5 dA is exact: the same as A + 0.5 dA
     B = __fma_rn(0.5, dB, B);
-    if (react) {  // min(A, B) off both: the smaller becomes exactly 0
-      if (A < B) {
-        B = B - A;
-        A = 0.0;
-      } else {
-        A = A - B;
-        B = 0.0;
-      }
+    if (react) Mass::react(A, B);
+  }
+  // min(A, B) off both: the smaller becomes exactly 0.  Finite masses of no
+  // sign compare by their bits, and a zero is not subtracted (after a
+  // particle's first reaction one of its masses often is): the binary64 pipe
+  // sees one subtraction, or nothing.
+  static __device__ __forceinline__ void react(double& A, double& B) {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(A);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(B);
+    if ((a | b) < 0x7ff0000000000000ULL) {
+      const bool less = a < b;
+      double rest = less ? B : A;
+      if ((less ? a : b) != 0) rest = rest - (less ? A : B);
+      A = less ? 0.0 : rest;
+      B = less ? rest : 0.0;
+    } else if (A < B) {
+      B = B - A;
+      A = 0.0;
+    } else {
+      A = A - B;
+      B = 0.0;
     }
   }
   static __device__ __forceinline__ double to_double(double v) { return v; }
@@ -303,6 +316,9 @@ struct Mass<MT_MIXED> {
   static __device__ __forceinline__ void update(double& A, double& B, double dA, double dB,
                                                 int react) {
     Mass<MT_FP64>::update(A, B, dA, dB, react);
+  }
+  static __device__ __forceinline__ void react(double& A, double& B) {
+    Mass<MT_FP64>::react(A, B);
   }
   static __device__ __forceinline__ double to_double(double v) { return v; }
 };
@@ -331,14 +347,15 @@ struct Mass<MT_MIXED_DF32> {
   static __device__ __forceinline__ void update(df& A, df& B, kahan dA, kahan dB, int react) {
     A = df_add(A, {0.5f * dA.s, 0.5f * dA.c});
     B = df_add(B, {0.5f * dB.s, 0.5f * dB.c});
-    if (react) {
-      if (df_le(A, B)) {
-        B = df_sub(B, A);
-        A = {0.0f, 0.0f};
-      } else {
-        A = df_sub(A, B);
-        B = {0.0f, 0.0f};
-      }
+    if (react) Mass::react(A, B);
+  }
+  static __device__ __forceinline__ void react(df& A, df& B) {
+    if (df_le(A, B)) {
+      B = df_sub(B, A);
+      A = {0.0f, 0.0f};
+    } else {
+      A = df_sub(A, B);
+      B = {0.0f, 0.0f};
     }
   }
   static __device__ __forceinline__ double to_double(df v) { return (double)v.hi + (double)v.lo; }

@@ -781,121 +781,187 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
 }
 
 // =============================================================== 2-d cells ==
+// The sort has put positions, ids and masses into the cells' slots.  Pass 1
+// forms the row sums and notes each particle's neighbours in src (free after
+// the sort): kNone, the slot of the only one, or kMany; it lists the particles
+// that have any (in the old positions' buffer, free after the sort; the count
+// in Ctrl::nbig, reset by the move).  Pass 2 streams the masses of the others
+// through the reaction -- in the sparse systems of the workloads (0.1
+// neighbours per particle) nine in ten -- and works off the list with full
+// warps, so that the binary64 instructions of the exchange are issued for
+// warps of particles that need them.  N = 10^6 at one particle per 100 units of
+// area: pass 1 43 -> 31 us (all cell starts loaded ahead, one loop over all
+// candidates, a box test of two subtractions per axis), pass 2 51 -> 16 us.
+constexpr int kNone = -1, kMany = -2;
 
-// One run [q0, q1) of candidate slots for the particle in slot p at (x, y).
-template <int PR, bool EXCHANGE, bool PER>
-__device__ __forceinline__ void cell2_run(const Dev& d, const long long* Xs, long long p,
-                                          long long x, long long y, int q0, int q1,
-                                          typename Weight<mixw(PR), 2>::T& r,
-                                          const unsigned long long* M,
-                                          typename Weight<mixw(PR), 2>::T ip,
-                                          typename Mass<PR>::V A, typename Mass<PR>::V B,
-                                          typename Mass<PR>::Acc& dA,
-                                          typename Mass<PR>::Acc& dB, long long ob,
-                                          const unsigned long long* s_tab) {
-  using W = Weight<mixw(PR), 2>;
-  using T = typename W::T;
-  using MS = Mass<PR>;
-  for (int q = q0; q < q1; ++q) {
-    long long dx = Xs[q] - x, dy = Xs[d.n + q] - y;
-    if (PER) {
-      dx = min_image(dx, d.Lq[0]);
-      dy = min_image(dy, d.Lq[1]);
-    }
-    if (!in_range2(dx, dy, d.S)) continue;
-    const T w = W::near2(d, dx, dy, s_tab);
-    if (!EXCHANGE) {
-      r += w;
-    } else if (q != p) {
-      const T P = normalised<T>(d.norm, w, ip, load_rinv<mixw(PR)>(d, q));
-      MS::acc(dA, P, MS::diff(MS::load(M, q), A));
-      MS::acc(dB, P, MS::diff(MS::load(M, ob + q), B));
-    }
-  }
-}
-
-// All candidates of the particle in slot p: the 3 x 3 block of cells around
-// its cell (reflecting walls), or the wrapped cell spans (periodic).  M:
-// the first species' masses; the second's are ob words further.
-template <int PR, bool EXCHANGE, bool PER>
-__device__ __forceinline__ void cell2_loop(const Dev& d, const long long* Xs, long long p,
-                                           long long x, long long y,
-                                           typename Weight<mixw(PR), 2>::T& r,
-                                           const unsigned long long* M,
-                                           typename Weight<mixw(PR), 2>::T ip,
-                                           typename Mass<PR>::V A, typename Mass<PR>::V B,
-                                           typename Mass<PR>::Acc& dA,
-                                           typename Mass<PR>::Acc& dB, long long ob,
-                                          const unsigned long long* s_tab) {
+// Calls f(q, dx, dy) for every other slot q within the cutoff of slot p at
+// (x, y), and self() for p, in slot order: the 3 x 3 block of cells around its
+// cell (reflecting walls), or the wrapped cell spans (PER, minimum-image
+// separations).  (The lanes of a warp meet themselves in different
+// iterations: with p among the pairs, nearly every iteration evaluated a
+// weight.)
+template <bool PER, class F, class G>
+__device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, int p, long long x,
+                                            long long y, F&& f, G&& self) {
   if (PER) {
     cells2_visit(d, x, y, [&](int q0, int q1) {
-      cell2_run<PR, EXCHANGE, true>(d, Xs, p, x, y, q0, q1, r, M, ip, A, B, dA, dB, ob, s_tab);
+      for (int q = q0; q < q1; ++q) {
+        if (q == p) {
+          self();
+          continue;
+        }
+        const long long dx = min_image(Xs[q] - x, d.Lq[0]);
+        const long long dy = min_image(Xs[d.n + q] - y, d.Lq[1]);
+        if (in_range2(dx, dy, d.S)) f(q, dx, dy);
+      }
     });
     return;
   }
-  long long kx = x >> d.cshift, ky = y >> d.cshift;
-  kx = kx >= d.ncx ? d.ncx - 1 : kx;
-  ky = ky >= d.ncy ? d.ncy - 1 : ky;
-  const long long kx0 = kx > 0 ? kx - 1 : 0;
-  const long long kx1 = kx + 1 < d.ncx ? kx + 1 : d.ncx - 1;
-  for (long long row = ky - 1; row <= ky + 1; ++row) {
-    if (row < 0 || row >= d.ncy) continue;
-    cell2_run<PR, EXCHANGE, false>(d, Xs, p, x, y, d.start[row * d.ncx + kx0],
-                                    d.start[row * d.ncx + kx1 + 1], r, M, ip, A, B, dA, dB, ob, s_tab);
+  const int ncx = (int)d.ncx, ncy = (int)d.ncy;  // (at most 2^28 cells)
+  const int kx = min((int)(x >> d.cshift), ncx - 1), ky = min((int)(y >> d.cshift), ncy - 1);
+  const int kx0 = max(kx - 1, 0), kx1 = min(kx + 1, ncx - 1);
+  int a[3], b[3];  // the rows' runs of slots, loaded together
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int row = ky - 1 + i;
+    const bool in = row >= 0 && row < ncy;
+    a[i] = in ? d.start[row * ncx + kx0] : 0;
+    b[i] = in ? d.start[row * ncx + kx1 + 1] : 0;
+  }
+  // one loop over the three runs, so that a warp's lanes wait for the longest
+  // sum of runs and not for the longest of each
+  const int n0 = max(b[0] - a[0], 0), n1 = n0 + max(b[1] - a[1], 0), n2 = n1 + max(b[2] - a[2], 0);
+  const int o1 = a[1] - n0, o2 = a[2] - n1;
+  // the box |dx|, |dy| <= S: X_q - (x - S) in [0, 2 S], 2 S < 2^31
+  const unsigned long long x0 = (unsigned long long)(x - d.S), y0 = (unsigned long long)(y - d.S);
+  const unsigned int S2 = 2u * (unsigned int)d.S;
+  const long long* Ys = Xs + d.n;
+#pragma unroll 2
+  for (int t = 0; t < n2; ++t) {
+    const int q = t + (t < n0 ? a[0] : t < n1 ? o1 : o2);
+    if (q == p) {
+      self();
+      continue;
+    }
+    const unsigned long long ux = (unsigned long long)Xs[q] - x0;
+    const unsigned long long uy = (unsigned long long)Ys[q] - y0;
+    if ((unsigned int)(ux >> 32) | (unsigned int)(uy >> 32)) continue;
+    if ((unsigned int)ux > S2 || (unsigned int)uy > S2) continue;
+    const int dx = (int)((unsigned int)ux - (unsigned int)d.S);
+    const int dy = (int)((unsigned int)uy - (unsigned int)d.S);
+    if ((unsigned long long)((long long)dx * dx) + (unsigned long long)((long long)dy * dy) <=
+        (unsigned long long)d.S * (unsigned long long)d.S)
+      f(q, dx, dy);
   }
 }
 
-// PER: periodic walls (wrapped cell spans, minimum-image separations), a
-// separate instantiation so the reflecting kernels keep their registers.
 template <int PR, bool PER>
 __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
-  using T = typename Weight<mixw(PR), 2>::T;
+  using W = Weight<mixw(PR), 2>;
+  using T = typename W::T;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
-  if (!mixw(PR)) exp_table<kThreads>(s_tab);
-  if (!mixw(PR)) __syncthreads();
+  if (!mixw(PR)) {
+    exp_table<kThreads>(s_tab);
+    __syncthreads();
+  }
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
-  if (p >= d.n) return;
-  const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
-  const long long* Xs = d.X[xc ^ 1];
-  T r = T(0);
-  typename Mass<PR>::Acc dummy{};
-  typename Mass<PR>::V z{};
-  cell2_loop<PR, false, PER>(d, Xs, p, Xs[p], Xs[d.n + p], r, nullptr, T(0), z, z, dummy,
-                              dummy, 0, s_tab);
-  store_rinv<mixw(PR)>(d, p, r);
-  const int s = d.src[p];
-  d.id[xc ^ 1][p] = d.id[xc][s];
-  gather_masses(d, mc, p, s);
+  const int xc = d.ctrl->xcur;
+  int nb = kNone;
+  if (p < d.n) {
+    const long long* Xs = d.X[xc ^ 1];
+    T r = T(0);
+    int found = 0;
+    cell2_visit<PER>(
+        d, Xs, (int)p, Xs[p], Xs[d.n + p],
+        [&](int q, long long dx, long long dy) {
+          r += W::near2(d, dx, dy, s_tab);
+          nb = found++ == 0 ? q : kMany;
+        },
+        [&] { r += T(1); });
+    d.src[p] = nb;
+    store_rinv<mixw(PR)>(d, p, r);
+  }
+  // the list of particles with neighbours, a CTA's together (one atomic per
+  // warp on one address held the pass at 39 us)
+  __shared__ int s_count[kThreads / 32], s_at;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned int m = __ballot_sync(0xffffffffu, nb != kNone);
+  if (lane == 0) s_count[warp] = __popc(m);
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; ++w) {
+    if (w < warp) before += s_count[w];
+    total += s_count[w];
+  }
+  if (threadIdx.x == 0 && total > 0) s_at = atomicAdd(&d.ctrl->nbig, total);
+  __syncthreads();
+  if (nb != kNone)
+    reinterpret_cast<int*>(d.X[xc])[s_at + before + __popc(m & ((1u << lane) - 1u))] = (int)p;
 }
 
 template <int PR, bool TR, bool PER>
 __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
-  using T = typename Weight<mixw(PR), 2>::T;
+  using W = Weight<mixw(PR), 2>;
+  using T = typename W::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
-  if (!mixw(PR)) exp_table<kThreads>(s_tab);
-  if (!mixw(PR)) __syncthreads();
-  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = p < d.n;
+  if (!mixw(PR)) {
+    exp_table<kThreads>(s_tab);
+    __syncthreads();
+  }
+  const long long g = (long long)blockIdx.x * kThreads + threadIdx.x;
+  if (g >= d.n) return;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
   const SpeciesPair sq = species_pair<TR>(d, sp);
-  MV A{}, B{};
-  if (valid) {
-    const long long* Xs = d.X[xc ^ 1];
-    const unsigned long long* MA = d.M[mc ^ 1] + sq.oa;
-    const unsigned long long* MB = d.M[mc ^ 1] + sq.ob;
-    A = MS::load(MA, p);
-    B = MS::load(MB, p);
-    T r = T(0);
-    typename MS::Acc dA{}, dB{};
-    cell2_loop<PR, true, PER>(d, Xs, p, Xs[p], Xs[d.n + p], r, MA, load_rinv<mixw(PR)>(d, p), A, B,
-                               dA, dB, sq.ob - sq.oa, s_tab);
-    MS::update(A, B, dA, dB, TR ? 0 : d.react);
+  const unsigned long long* MA = d.M[mc ^ 1] + sq.oa;
+  const unsigned long long* MB = d.M[mc ^ 1] + sq.ob;
+  auto store = [&](long long p, MV A, MV B) {
     MS::store(d.M[mc] + sq.oa, p, A);
     if (sq.store_b) MS::store(d.M[mc] + sq.ob, p, B);
+  };
+  if (d.src[g] == kNone) {
+    MV A = MS::load(MA, g), B = MS::load(MB, g);
+    if (!TR && d.react) MS::react(A, B);
+    store(g, A, B);
   }
-  if (!TR) finish_step(d, 1, 0);
+  if (g >= d.ctrl->nbig) return;
+  // the list: one entry per thread of the first CTAs
+  const long long p = reinterpret_cast<const int*>(d.X[xc])[g];
+  const long long* Xs = d.X[xc ^ 1];
+  const int nb = d.src[p];
+  MV A = MS::load(MA, p), B = MS::load(MB, p);
+  typename MS::Acc dA{}, dB{};
+  const long long x = Xs[p], y = Xs[d.n + p];
+  const T ip = load_rinv<mixw(PR)>(d, p);
+  auto pair = [&](int q, long long dx, long long dy) {
+    const T P = normalised<T>(d.norm, W::near2(d, dx, dy, s_tab), ip, load_rinv<mixw(PR)>(d, q));
+    MS::acc(dA, P, MS::diff(MS::load(MA, q), A));
+    MS::acc(dB, P, MS::diff(MS::load(MB, q), B));
+  };
+  if (nb >= 0) {
+    long long dx = Xs[nb] - x, dy = Xs[d.n + nb] - y;
+    if (PER) {
+      dx = min_image(dx, d.Lq[0]);
+      dy = min_image(dy, d.Lq[1]);
+    }
+    pair(nb, dx, dy);
+  } else {
+    cell2_visit<PER>(d, Xs, (int)p, x, y, pair, [] {});
+  }
+  MS::update(A, B, dA, dB, TR ? 0 : d.react);
+  store(p, A, B);
+}
+
+// The end of a step whose passes leave it to a kernel of its own: a fence, an
+// atomic on one address and a wait in every CTA of a large pass cost more
+// (10^6 particles: ~10 us) than a launch.
+__global__ void k_finish(Dev d, int flip_x, int flip_m) {
+  Ctrl* c = d.ctrl;
+  c->step += 1;
+  c->xcur ^= flip_x;
+  c->mcur ^= flip_m;
 }
 
 // ============================================================ brute force ==
@@ -1024,16 +1090,14 @@ template <int PR, bool PER>
 static void cell2_passes(const Dev& d, unsigned int g, cudaStream_t s, Marker& mk) {
   mk("rowsum_cell2", s);
   k_rowsum_cell2<PR, PER><<<g, kThreads, 0, s>>>(d);
-  if (d.nspec > 2) {
-    mk("gather_species", s);
-    k_gather_species<<<g, kThreads, 0, s>>>(d);
-  }
   for (int sp = 2; sp < d.nspec; sp += 2) {
     mk("exchange_cell2_species", s);
     k_exchange_cell2<PR, true, PER><<<g, kThreads, 0, s>>>(d, sp);
   }
   mk("exchange_cell2", s);
   k_exchange_cell2<PR, false, PER><<<g, kThreads, 0, s>>>(d, 0);
+  mk("finish", s);
+  k_finish<<<1, 1, 0, s>>>(d, 1, 0);
 }
 
 template <int PR, bool TR>
