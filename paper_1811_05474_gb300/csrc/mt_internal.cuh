@@ -201,10 +201,18 @@ __device__ __forceinline__ void gather_species(const Dev& d, int mc, long long p
   for (int k = 2; k < d.nspec; ++k) out[k * d.n + p] = in[k * d.n + s];
 }
 
-// Periodic walls: y modulo Lq into [0, Lq).
+// Periodic walls: y modulo Lq into [0, Lq) (a 64-bit division takes ~100
+// instructions: only for what a step carries further than one domain).
 __device__ __forceinline__ long long wrap(long long y, long long Lq) {
+  if (y >= 0 && y < Lq) return y;
+  if (y < 0 && y >= -Lq) return y + Lq;
+  if (y >= Lq && y < 2 * Lq) return y - Lq;
   const long long m = y % Lq;
   return m < 0 ? m + Lq : m;
+}
+// The same for the difference of two positions in [0, Lq).
+__device__ __forceinline__ long long wrap_gap(long long y, long long Lq) {
+  return y < 0 ? y + Lq : y;
 }
 
 // Periodic walls in 1-d: the ring of sorted slots a particle's walks go
