@@ -40,6 +40,10 @@ constexpr double kTwo61 = 2305843009213693952.0;   // 2^61
 constexpr size_t kAlign = 256;
 constexpr long long kWcCap = 1LL << 22;  // 32 MiB of cached weights (rows of up to 2048 slots)
 constexpr long long kWcMinN = 1LL << 17;
+// Steps of one graph of several: the frame (two conditional nodes and two
+// one-thread kernels, ~15 us) is spread over them, and 25-step chunks and runs
+// of 50 or 100 steps leave few over.
+constexpr int kMultiSteps = 12;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -458,6 +462,7 @@ struct mt_handle {
   long long steps = 0;     // host mirror of the step counter
   const float* noise = nullptr;
   cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t multi = nullptr;  // kMultiSteps steps (fused path, no predicted segments)
   bool profile = false;
   cudaEvent_t ev[kMaxMarks + 1] = {};
   const char* ev_names[kMaxMarks] = {};
@@ -585,6 +590,141 @@ mt_status enqueue_step(mt_handle* h, const Dev& d) {
   return MT_OK;
 }
 
+// The second tier and, inside a conditional node behind it, the general
+// pipeline, captured into the body of the conditional node after a first tier.
+mt_status capture_second_tier(mt_handle* h, cudaGraph_t body1) {
+  const Dev& d = h->dev;
+  const cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+  cudaGraphConditionalHandle cond2;
+  CU(cudaGraphConditionalHandleCreate(&cond2, body1, 0, 0));
+  CU(cudaStreamBeginCaptureToGraph(h->stream, body1, nullptr, nullptr, 0, mode));
+  const cudaError_t e1 = launch_fused_big(d, h->D.p.precision, cond2, 1, h->stream);
+  const cudaError_t e2 = cudaStreamEndCapture(h->stream, &body1);
+  if (e1 != cudaSuccess || e2 != cudaSuccess)
+    return fail(MT_ERR_CUDA, "graph capture of the second fused tier failed");
+  cudaGraphNode_t bnode = nullptr, cnode = nullptr;
+  size_t nn = 1;
+  CU(cudaGraphGetNodes(body1, &bnode, &nn));
+  cudaGraphNodeParams cp = {};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = cond2;
+  cp.conditional.type = cudaGraphCondTypeIf;
+  cp.conditional.size = 1;
+  CU(cudaGraphAddNode(&cnode, body1, &bnode, nullptr, 1, &cp));
+  cudaGraph_t body2 = cp.conditional.phGraph_out[0];
+  Marker none;
+  CU(cudaStreamBeginCaptureToGraph(h->stream, body2, nullptr, nullptr, 0, mode));
+  const mt_status s = enqueue_general(h, d, none);
+  const cudaError_t e3 = cudaStreamEndCapture(h->stream, &body2);
+  if (s == MT_OK && e3 != cudaSuccess)
+    return fail(MT_ERR_CUDA, "graph capture of the fallback failed");
+  return s;
+}
+
+// Capture the kernels `body` enqueues into graph g, behind node `after` (null:
+// at its root), and return the last of them.
+template <class F>
+mt_status capture_into(mt_handle* h, cudaGraph_t g, const cudaGraphNode_t* after, F&& body,
+                       cudaGraphNode_t* last) {
+  CU(cudaStreamBeginCaptureToGraph(h->stream, g, after, nullptr, after ? 1 : 0,
+                                   cudaStreamCaptureModeThreadLocal));
+  const cudaError_t e1 = body();
+  cudaStreamCaptureStatus st;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t nd = 0;
+  const cudaError_t e2 =
+      cudaStreamGetCaptureInfo(h->stream, &st, nullptr, nullptr, &deps, nullptr, &nd);
+  if (e2 == cudaSuccess && nd == 1) *last = deps[0];
+  const cudaError_t e3 = cudaStreamEndCapture(h->stream, &g);
+  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || nd != 1)
+    return fail(MT_ERR_CUDA, "graph capture of several fused steps failed");
+  return MT_OK;
+}
+
+// A conditional node on `handle` behind node `after` of g.
+mt_status add_conditional(cudaGraph_t g, cudaGraphNode_t after, cudaGraphConditionalHandle handle,
+                          cudaGraphConditionalNodeType type, cudaGraphNode_t* node,
+                          cudaGraph_t* body) {
+  cudaGraphNodeParams cp = {};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = handle;
+  cp.conditional.type = type;
+  cp.conditional.size = 1;
+  CU(cudaGraphAddNode(node, g, &after, nullptr, 1, &cp));
+  *body = cp.conditional.phGraph_out[0];
+  return MT_OK;
+}
+
+// kMultiSteps steps in one graph, for systems without the predicted-segment
+// kernel (their step is tens of microseconds, of which the conditional node
+// after each step and the boundary between two graphs took ~7):
+//   begin -> IF(last graph needed no second tier) { step, step, ... } -> next
+//   -> WHILE(steps to do) { step -> IF(queued) { second tier -> IF(overflow)
+//   { general } } -> next }
+// A first tier of the IF body that queues segments leaves the step pending;
+// the first tiers after it do nothing, and the WHILE body first completes that
+// step and then does the rest, one checked step at a time.  Each step's
+// observables follow it.
+mt_status build_multi_into(mt_handle* h, cudaGraph_t g) {
+  const Dev& d = h->dev;
+  const int pr = h->D.p.precision;
+  cudaGraphConditionalHandle fast, more, queued;
+  CU(cudaGraphConditionalHandleCreate(&fast, g, 0, 0));
+  CU(cudaGraphConditionalHandleCreate(&more, g, 0, 0));
+  cudaGraphNode_t at = nullptr, cnode = nullptr;
+  cudaGraph_t body = nullptr, wbody = nullptr, qbody = nullptr;
+  mt_status s = capture_into(
+      h, g, nullptr, [&] { return launch_multi_begin(d, kMultiSteps, fast, h->stream); }, &at);
+  if (s == MT_OK) s = add_conditional(g, at, fast, cudaGraphCondTypeIf, &cnode, &body);
+  if (s == MT_OK)
+    s = capture_into(
+        h, body, nullptr,
+        [&] {
+          cudaError_t e = cudaSuccess;
+          for (int j = 1; j <= kMultiSteps && e == cudaSuccess; ++j) {
+            e = launch_fused_step(d, pr, 0, 0, h->stream);
+            if (e == cudaSuccess) e = launch_obs_step(d, pr, j, kMultiSteps, h->stream);
+          }
+          return e;
+        },
+        &at);
+  if (s == MT_OK)
+    s = capture_into(h, g, &cnode, [&] { return launch_multi_next(d, more, h->stream); }, &at);
+  if (s == MT_OK) s = add_conditional(g, at, more, cudaGraphCondTypeWhile, &cnode, &wbody);
+  if (s != MT_OK) return s;
+  CU(cudaGraphConditionalHandleCreate(&queued, wbody, 0, cudaGraphCondAssignDefault));
+  s = capture_into(
+      h, wbody, nullptr, [&] { return launch_fused_step(d, pr, queued, 1, h->stream); }, &at);
+  if (s == MT_OK) s = add_conditional(wbody, at, queued, cudaGraphCondTypeIf, &cnode, &qbody);
+  if (s == MT_OK) s = capture_second_tier(h, qbody);
+  if (s == MT_OK)
+    s = capture_into(
+        h, wbody, &cnode,
+        [&] {
+          const cudaError_t e = launch_obs(d, pr, h->stream);
+          return e == cudaSuccess ? launch_multi_next(d, more, h->stream) : e;
+        },
+        &at);
+  return s;
+}
+
+mt_status build_multi(mt_handle* h) {
+  cudaGraph_t g = nullptr;
+  CU(cudaGraphCreate(&g, 0));
+  const mt_status s = build_multi_into(h, g);
+  if (s != MT_OK) {
+    cudaGraphDestroy(g);
+    return s;
+  }
+  const cudaError_t e = cudaGraphInstantiate(&h->multi, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    h->multi = nullptr;
+    return fail(MT_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+  }
+  return MT_OK;
+}
+
 // Capture one step into an executable graph.  On the fused path the graph
 // is [fused step] -> IF(overflow) {general pipeline}.
 mt_status build_graph(mt_handle* h) {
@@ -598,7 +738,7 @@ mt_status build_graph(mt_handle* h) {
     // g: { [predicted segments, taking the observables' snapshot] ->
     //   [previous step's observables] | [fast tier] } -> IF(queued)
     //   { [second tier] -> IF(overflow) { general } }
-    cudaGraphConditionalHandle cond1, cond2;
+    cudaGraphConditionalHandle cond1;
     CU(cudaGraphConditionalHandleCreate(&cond1, g, 0, 0));
     // large systems fork: the predicted-segment kernel on the side stream,
     // the first tier on the handle's stream; with observables, the previous
@@ -665,32 +805,7 @@ mt_status build_graph(mt_handle* h) {
       CU(cudaGraphAddNode(&cnode, g, leaves, nullptr, nleaf, &cp));
       body1 = cp.conditional.phGraph_out[0];
     }
-    CU(cudaGraphConditionalHandleCreate(&cond2, body1, 0, 0));
-    CU(cudaStreamBeginCaptureToGraph(h->stream, body1, nullptr, nullptr, 0, mode));
-    e1 = launch_fused_big(d, h->D.p.precision, cond2, 1, h->stream);
-    e2 = cudaStreamEndCapture(h->stream, &body1);
-    if (e1 != cudaSuccess || e2 != cudaSuccess) {
-      cudaGraphDestroy(g);
-      return fail(MT_ERR_CUDA, "graph capture of the second fused tier failed");
-    }
-    cudaGraph_t body2 = nullptr;
-    {
-      cudaGraphNode_t bnode = nullptr;
-      size_t nn = 1;
-      CU(cudaGraphGetNodes(body1, &bnode, &nn));
-      cudaGraphNodeParams cp = {};
-      cp.type = cudaGraphNodeTypeConditional;
-      cp.conditional.handle = cond2;
-      cp.conditional.type = cudaGraphCondTypeIf;
-      cp.conditional.size = 1;
-      cudaGraphNode_t cnode = nullptr;
-      CU(cudaGraphAddNode(&cnode, body1, &bnode, nullptr, 1, &cp));
-      body2 = cp.conditional.phGraph_out[0];
-    }
-    CU(cudaStreamBeginCaptureToGraph(h->stream, body2, nullptr, nullptr, 0, mode));
-    s = enqueue_general(h, d, none);
-    const cudaError_t e3 = cudaStreamEndCapture(h->stream, &body2);
-    if (s == MT_OK && e3 != cudaSuccess) s = fail(MT_ERR_CUDA, "graph capture of the fallback failed");
+    s = capture_second_tier(h, body1);
     // the step's own observables: the next step's graph (or flush_obs)
     // where they are deferred, else after the IF node
     if (s == MT_OK && !obs && h->D.p.observe_cap > 0) {
@@ -1010,15 +1125,28 @@ mt_status mt_run(mt_handle* h, int64_t nsteps) {
     }
     return MT_OK;
   }
-  if (!h->graph) {
+  int64_t left = nsteps;
+  if (h->D.fused && !h->dev.use_pred && left >= kMultiSteps) {
+    if (!h->multi) {
+      const mt_status s = build_multi(h);
+      if (s != MT_OK) return s;
+    }
+    const mt_status s = flush_obs(h);  // the graph's first step overwrites what they read
+    if (s != MT_OK) return s;
+    for (; left >= kMultiSteps; left -= kMultiSteps) {
+      CU(cudaGraphLaunch(h->multi, h->stream));
+      h->steps += kMultiSteps;
+    }
+  }
+  if (left > 0 && !h->graph) {
     const mt_status s = build_graph(h);
     if (s != MT_OK) return s;
   }
-  for (int64_t i = 0; i < nsteps; ++i) {
+  for (; left > 0; --left) {
     CU(cudaGraphLaunch(h->graph, h->stream));
     ++h->steps;
+    if (h->obs_defer) h->obs_pending = true;
   }
-  if (nsteps > 0 && h->obs_defer) h->obs_pending = true;
   return MT_OK;
 }
 
@@ -1403,6 +1531,7 @@ void mt_destroy(mt_handle* h) {
   if (!h) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->graph) cudaGraphExecDestroy(h->graph);
+  if (h->multi) cudaGraphExecDestroy(h->multi);
   for (int i = 0; i <= kMaxMarks; ++i)
     if (h->ev[i]) cudaEventDestroy(h->ev[i]);
   if (h->side) {

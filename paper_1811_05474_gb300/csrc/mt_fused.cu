@@ -1533,6 +1533,8 @@ __device__ __forceinline__ void fused_advance(const Dev& d) {
   c->fallback = 0;
   c->npred = c->npred_next;
   c->npred_next = 0;
+  c->pending = 0;
+  c->todo -= 1;
 }
 
 // The first tier and the predicted-segment kernel run side by side; the
@@ -1556,7 +1558,10 @@ __device__ __forceinline__ void join_finish(const Dev& d, int role,
   Ctrl* c = d.ctrl;
   const bool more = role == 2;
   if (!more) fused_advance(d);
-  if (more) c->big_steps += 1;
+  if (more) {
+    c->big_steps += 1;
+    c->pending = 1;
+  }
   if (c->nov > c->ov_value) c->ov_value = c->nov;  // largest queue seen (diagnostic)
   c->kjoin = 0;
   c->seg_ctr = 0;
@@ -1582,6 +1587,10 @@ __global__ void __launch_bounds__(Fast::kT, PR == MT_FP64 ? 3 : kFusedCtasPerSm)
   __shared__ bool s_last;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
   Ctrl* c = d.ctrl;
+  if (c->pending) {  // an earlier step of the graph is not complete: the second tier's turn
+    if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 1u);
+    return;
+  }
   const StepState st = step_state<PR, Fast::kT>(d, s_tab);
   const int sc = st.sc;
   const long long Dc = (c->dmax >> d.cshift) + 2;
@@ -1815,7 +1824,11 @@ __global__ void k_fused_prep(Dev d, int flip) {
 }
 
 __global__ void k_fused_flip(Dev d, int flip) {
-  if (flip) d.ctrl->scur ^= 1;
+  if (flip) {
+    d.ctrl->scur ^= 1;
+    d.ctrl->todo -= 1;
+  }
+  d.ctrl->pending = 0;
   d.ctrl->fallback = 0;
   d.ctrl->nov = 0;
   d.ctrl->npred = d.ctrl->npred_next;
@@ -2058,6 +2071,34 @@ __global__ void k_join_stub(Dev d) { end_of_tier(d, 0, 0); }
 
 cudaError_t launch_join_stub(const Dev& d, cudaStream_t s) {
   k_join_stub<<<1, 1, 0, s>>>(d);
+  return cudaGetLastError();
+}
+
+// Start of a graph of several steps: the fast form (first tiers one after
+// another) unless the last graph met segments for the second tier.
+__global__ void k_multi_begin(Dev d, int steps, cudaGraphConditionalHandle fast) {
+  Ctrl* c = d.ctrl;
+  c->todo = steps;
+  c->big_mark = c->big_steps;
+  cudaGraphSetConditional(fast, c->careful ? 0u : 1u);
+}
+
+// Whether the careful form has a step to do or to complete.
+__global__ void k_multi_next(Dev d, cudaGraphConditionalHandle more) {
+  Ctrl* c = d.ctrl;
+  const bool go = c->todo > 0;
+  if (!go) c->careful = c->big_steps != c->big_mark;
+  cudaGraphSetConditional(more, go ? 1u : 0u);
+}
+
+cudaError_t launch_multi_begin(const Dev& d, int steps, cudaGraphConditionalHandle fast,
+                               cudaStream_t s) {
+  k_multi_begin<<<1, 1, 0, s>>>(d, steps, fast);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_multi_next(const Dev& d, cudaGraphConditionalHandle more, cudaStream_t s) {
+  k_multi_next<<<1, 1, 0, s>>>(d, more);
   return cudaGetLastError();
 }
 

@@ -65,7 +65,15 @@ struct Ctrl {
   int obs_prev_todo;
   unsigned long long obs_step;
   unsigned long long obs_done_step;
+  // Graphs of several steps: a first tier that queued segments sets pending
+  // (the following first tiers of the graph then do nothing) until the second
+  // tier or the general pipeline has completed the step.
+  int pending;
+  int todo;                  // steps of the running graph not yet done
+  int careful;               // the graph checks after every step
+  unsigned long long big_mark;  // big_steps at the graph's start
 };
+static_assert(sizeof(Ctrl) <= 256, "the control block's place in the workspace");
 
 // The snapshot the previous step's observables read (one thread, at the
 // start of a step, before the step advances the control block).
@@ -536,6 +544,13 @@ cudaError_t launch_fused_step(const Dev& d, int precision, cudaGraphConditionalH
 cudaError_t launch_fused_pred(const Dev& d, int precision, cudaGraphConditionalHandle cond,
                               int use_cond, cudaStream_t s, cudaEvent_t started = nullptr);  // predicted heavy segments
 cudaError_t launch_join_stub(const Dev& d, cudaStream_t s);
+// The frame of a graph of several steps (mt_fused.cu)
+cudaError_t launch_multi_begin(const Dev& d, int steps, cudaGraphConditionalHandle fast,
+                               cudaStream_t s);
+cudaError_t launch_multi_next(const Dev& d, cudaGraphConditionalHandle more, cudaStream_t s);
+// the observables of the state if it is one the running graph reached by its
+// j-th step (its first: 1)
+cudaError_t launch_obs_step(const Dev& d, int precision, int j, int steps, cudaStream_t s);
 cudaError_t launch_fused_big(const Dev& d, int precision, cudaGraphConditionalHandle cond,
                              int use_cond, cudaStream_t s);
 cudaError_t launch_fused_prep(const Dev& d, int flip, cudaStream_t s);  // start/cb from d.start

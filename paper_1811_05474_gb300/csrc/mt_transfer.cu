@@ -69,16 +69,19 @@ struct ThreadObs<true> {  // double-binary32 masses
 // PREV: the state at the step's start (obs_snapshot, by k_obs_snapshot or
 // the predicted-segment kernel), while
 // the step runs beside it (it writes the other mass buffer); otherwise the
-// current state.  Either writes the row of the step the state follows.
+// current state (left > 0: only if left - 1 of the running graph's steps are
+// still to do).  Either writes the row of the step the state follows.
 template <int PR, bool PREV>
-__global__ void __launch_bounds__(kThreads) k_obs(Dev d) {
+__global__ void __launch_bounds__(kThreads) k_obs(Dev d, int left) {
   using MS = Mass<PR>;
   using MV = typename MS::V;
   constexpr int kPer = kObsChunk / kThreads;  // slots per thread
   __shared__ Obs3<MV> s_w[kThreads / 32];
   __shared__ bool s_last;
   Ctrl* c = d.ctrl;
-  if (PREV && !c->obs_prev_todo) return;  // fixed before the launch: every CTA agrees
+  // (both fixed before the launch: every CTA agrees)
+  if (PREV && !c->obs_prev_todo) return;
+  if (left > 0 && c->todo != left - 1) return;
   const unsigned long long step = PREV ? c->obs_step : c->step;
   const int ch = blockIdx.x;
   const unsigned long long* M = d.M[PREV ? c->obs_mc : c->mcur];
@@ -143,19 +146,27 @@ cudaError_t launch_obs_snapshot(const Dev& d, cudaStream_t s) {
 cudaError_t launch_obs_prev(const Dev& d, int precision, cudaStream_t s) {
   if (d.observe_cap <= 0 || d.nochunk <= 0) return cudaSuccess;
   if (precision == MT_MIXED_DF32)
-    k_obs<MT_MIXED_DF32, true><<<d.nochunk, kThreads, 0, s>>>(d);
+    k_obs<MT_MIXED_DF32, true><<<d.nochunk, kThreads, 0, s>>>(d, 0);
   else
-    k_obs<MT_FP64, true><<<d.nochunk, kThreads, 0, s>>>(d);  // binary64 masses
+    k_obs<MT_FP64, true><<<d.nochunk, kThreads, 0, s>>>(d, 0);  // binary64 masses
+  return cudaGetLastError();
+}
+
+static cudaError_t obs_of_state(const Dev& d, int precision, int left, cudaStream_t s) {
+  if (d.observe_cap <= 0 || d.nochunk <= 0) return cudaSuccess;
+  if (precision == MT_MIXED_DF32)
+    k_obs<MT_MIXED_DF32, false><<<d.nochunk, kThreads, 0, s>>>(d, left);
+  else
+    k_obs<MT_FP64, false><<<d.nochunk, kThreads, 0, s>>>(d, left);  // binary64 masses
   return cudaGetLastError();
 }
 
 cudaError_t launch_obs(const Dev& d, int precision, cudaStream_t s) {
-  if (d.observe_cap <= 0 || d.nochunk <= 0) return cudaSuccess;
-  if (precision == MT_MIXED_DF32)
-    k_obs<MT_MIXED_DF32, false><<<d.nochunk, kThreads, 0, s>>>(d);
-  else
-    k_obs<MT_FP64, false><<<d.nochunk, kThreads, 0, s>>>(d);  // binary64 masses
-  return cudaGetLastError();
+  return obs_of_state(d, precision, 0, s);
+}
+
+cudaError_t launch_obs_step(const Dev& d, int precision, int j, int steps, cudaStream_t s) {
+  return obs_of_state(d, precision, steps - j + 1, s);
 }
 
 // ================================================================ 1-d walk ==
