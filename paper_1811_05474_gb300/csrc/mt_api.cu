@@ -781,7 +781,11 @@ mt_status build_graph(mt_handle* h) {
     cudaGraph_t body1 = nullptr;
     cudaGraphNode_t cnode = nullptr;  // the IF node
     {
-      // the IF node follows every kernel node without a dependent
+      // The IF node waits for every kernel's completion.  (Not only for those
+      // without a dependent: the first tier depends on the predicted-segment
+      // kernel's launch alone, and without observables behind it nothing else
+      // would wait for its end -- the condition was then evaluated, with the
+      // last step's value, while predicted segments were still running.)
       const size_t want = 1 + (fork ? 1 : 0) + (obs ? (fork ? 1 : 2) : 0);
       cudaGraphNode_t knodes[4] = {nullptr, nullptr, nullptr, nullptr};
       size_t nn = 4;
@@ -790,19 +794,12 @@ mt_status build_graph(mt_handle* h) {
         cudaGraphDestroy(g);
         return fail(MT_ERR_CUDA, "fused step graph: expected %zu kernel nodes, got %zu", want, nn);
       }
-      cudaGraphNode_t leaves[4];
-      size_t nleaf = 0;
-      for (size_t i = 0; i < nn; ++i) {
-        size_t ndep = 0;
-        CU(cudaGraphNodeGetDependentNodes(knodes[i], nullptr, nullptr, &ndep));
-        if (ndep == 0) leaves[nleaf++] = knodes[i];
-      }
       cudaGraphNodeParams cp = {};
       cp.type = cudaGraphNodeTypeConditional;
       cp.conditional.handle = cond1;
       cp.conditional.type = cudaGraphCondTypeIf;
       cp.conditional.size = 1;
-      CU(cudaGraphAddNode(&cnode, g, leaves, nullptr, nleaf, &cp));
+      CU(cudaGraphAddNode(&cnode, g, knodes, nullptr, nn, &cp));
       body1 = cp.conditional.phGraph_out[0];
     }
     s = capture_second_tier(h, body1);

@@ -53,3 +53,26 @@ def test_batch(precision):
     x = np.concatenate([synth.uniform_positions(n, L, seed=5)[0] for n, L in zip(ns, Ls)])[None]
     A, B = synth.uniform_masses(sum(ns), seed=6)
     compare(p, x, A, B, [25, 2, 36], batch=mt.make_batch(ns, Ls))
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+def test_step_waits_for_its_predicted_segments(precision):
+    """A large system whose wall layer keeps the predicted-segment kernel busy
+    longer than the first tier: the state after graph steps without observables
+    is the one with them (whose kernel, behind the predicted segments, the
+    step's end waits for)."""
+    n, L = 700000, 700000.0
+    x = synth.uniform_positions(n, L, seed=1)
+    x[0, :900] = L - 0.25 * synth.rng(5).exponential(size=900)
+    A, B = synth.uniform_masses(n, seed=2)
+    out = []
+    for observe in (0, 8):
+        p = mt.mt_params_init(n=n, L=(L,), v=(0.5, 0.0), precision=precision, seed=4,
+                              observe_cap=observe)
+        sim = mt.Simulation(p)
+        sim.upload(x, A, B)
+        sim.run(8)
+        out.append((sim.ticks(), *sim.masses()))
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
