@@ -194,12 +194,13 @@ __device__ __forceinline__ StepState step_state(const Dev& d, unsigned long long
 
 // The next segment's staged slots [a0, a0 + L) (positions, ids, both mass
 // arrays) asked into L2 while the current segment runs its transfer, once
-// its cell starts have arrived (thread 0, after prefetch_stage2), so that
-// its staging loads do not wait on HBM.
+// its cell starts have arrived (thread 0 has waited for them, and a barrier
+// followed), so that its staging loads do not wait on HBM.  Called by the
+// CTA's last warp: the instructions take their thread over a thousand cycles,
+// which thread 0 would keep the next barrier waiting for.
 __device__ __forceinline__ void prefetch_next_l2(const Dev& d, const SegPrefetch& pf,
                                                  const StepState& st) {
   if (pf.seg >= d.nseg) return;
-  __pipeline_wait_prior(0);
   const long long a0 = pf.w[2], e = pf.w[3];
   if (e <= a0 || e - a0 > 2 * (long long)kFusedCap) return;  // nothing, or not staged
   l2_prefetch(d.X[st.xc], a0 * 8, e * 8);
@@ -761,11 +762,13 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
 }
 
 // Next step's cell starts and segment boundaries, by the CTA that wrote the
-// segment's particles: sorted slots [w0, w1) of its staging to out0 on.
+// segment's particles: sorted slots [w0, w1) of its staging to out0 on; slot0
+// and slot1: sslot of the segment and the next.
 template <int NT>
 __device__ __forceinline__ void segment_tables(const Dev& d, int sc, int seg, const long long* sx,
                                                const int* bstart, int sh2, long long wlo, int c0,
-                                               int c1, int w0, int w1, long long out0) {
+                                               int c1, int w0, int w1, long long out0,
+                                               long long slot0, long long slot1) {
   const int tid = threadIdx.x, wsh = d.cshift;
   int* Sn = d.fstart[sc ^ 1];
   for (long long cc = c0 + tid; cc < c1; cc += NT) {
@@ -792,9 +795,9 @@ __device__ __forceinline__ void segment_tables(const Dev& d, int sc, int seg, co
   int* CBn = d.cb[sc ^ 1];
   const long long own = w1 - w0;
   int s2 = seg + 1;
-  if (d.sslot[seg] > out0) {
+  if (slot0 > out0) {
     while (s2 > 1 && d.sslot[s2 - 1] > out0) --s2;
-  } else if (d.sslot[seg + 1] <= out0) {
+  } else if (slot1 <= out0) {
     while (s2 < d.nseg && d.sslot[s2] <= out0) ++s2;
   }
   for (s2 += tid; s2 < d.nseg; s2 += NT) {
@@ -853,6 +856,7 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
     return kSegCapacity;
   }
   // ---- stage: the loads are in flight while the bins are cleared ----------
+  const int slot0 = d.sslot[seg], slot1 = d.sslot[seg + 1];  // (read at the end)
   long long rx[PER];
   int rid[PER], rb[PER];  // rb: bin | arrival number << 16
 #pragma unroll
@@ -904,7 +908,8 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
                           d.key0, d.key1);
         z = box_muller(u.x, u.y).x;
       }
-      const long long x = base + reflect(rx[k] - base + d.drift[0] + walk_ticks(d.bq, z), Lq);
+      const long long x =
+          base + reflect(rx[k] - base + d.drift[0] + walk_ticks<!mixw(PR)>(d.bq, z), Lq);
       rx[k] = x;
       lt = slot >= o0 && slot < o1 && x < xlo;
       if (x >= wlo && x < whi) {
@@ -1016,6 +1021,7 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
     }
   }
   __syncthreads();
+  if (tid == 0) __pipeline_wait_prior(0);  // the next segment's cell starts
   const int EA = fix_scale(s_emax[0]), EB = fix_scale(s_emax[1]);
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
@@ -1038,14 +1044,14 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
   const int w0 = sh2 == wsh ? bstart[(xlo - wlo) >> wsh] : s_w0;
   const int w1 = sh2 == wsh ? bstart[(xhi - wlo) >> wsh] : s_w1;
   const long long out0 = o0 + s_lt;
-  if (tid == 0) prefetch_next_l2(d, pf, st);
+  if (tid == NT - 32) prefetch_next_l2(d, pf, st);
   bool fits;
   if constexpr (mixw(PR))
     fits = walk_transfer<PR>(d, st, smem, m, w0, w1, out0, xlo, xhi, sE, a0, EA, EB);
   else
     fits = pair_transfer<Fast>(d, st, smem, m, w0, w1, out0, xlo, xhi);
   if (!fits) return kSegHeavy;  // more pairs than the list holds: the second tier takes it
-  segment_tables<NT>(d, st.sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0);
+  segment_tables<NT>(d, st.sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0, slot0, slot1);
   return kSegOk;
 }
 
@@ -1518,7 +1524,8 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
   // every CTA has read this segment's (cw is the same in all of them)
   if (kCache && cw) cg::this_cluster().sync();
   if (active && slice == 0)
-    segment_tables<NT>(d, sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0);
+    segment_tables<NT>(d, sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0, d.sslot[seg],
+                       d.sslot[seg + 1]);
   __syncthreads();
   return status;
 }

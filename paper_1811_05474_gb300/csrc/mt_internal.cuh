@@ -406,10 +406,13 @@ __device__ __forceinline__ long long rint_exact(double v) {
 }
 
 // Eq. 2's random-walk displacement on the grid: the nearest tick to b xi,
-// b = sqrt(2 D_rw dt) 2^k, with the product formed in binary64 (the one
-// binary64 instruction here).
+// b = sqrt(2 D_rw dt) 2^k, with the product formed in binary64.  INTEGER: the
+// conversions around it from the bits, for kernels that the binary64 pipe
+// bounds (the same values).
+template <bool INTEGER = true>
 __device__ __forceinline__ long long walk_ticks(double b, float xi) {
-  return rint_exact(__dmul_rn(b, widen_exact(xi)));
+  return INTEGER ? rint_exact(__dmul_rn(b, widen_exact(xi)))
+                 : __double2ll_rn(__dmul_rn(b, (double)xi));
 }
 
 // Two standard normals from two 32-bit words (Box-Muller, binary32, with
