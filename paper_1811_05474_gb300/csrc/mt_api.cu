@@ -682,7 +682,7 @@ mt_status build_multi_into(mt_handle* h, cudaGraph_t g) {
         [&] {
           cudaError_t e = cudaSuccess;
           for (int j = 1; j <= kMultiSteps && e == cudaSuccess; ++j) {
-            e = launch_fused_step(d, pr, 0, 0, h->stream);
+            e = launch_fused_step(d, pr, 0, kChained, h->stream);
             if (e == cudaSuccess) e = launch_obs_step(d, pr, j, kMultiSteps, h->stream);
           }
           return e;

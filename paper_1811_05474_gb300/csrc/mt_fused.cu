@@ -1594,6 +1594,10 @@ __global__ void __launch_bounds__(Fast::kT, PR == MT_FP64 ? 3 : kFusedCtasPerSm)
   __shared__ bool s_last;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
   Ctrl* c = d.ctrl;
+  if (use_cond == kChained) {
+    chained();
+    use_cond = 0;
+  }
   if (c->pending) {  // an earlier step of the graph is not complete: the second tier's turn
     if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 1u);
     return;
@@ -1981,15 +1985,17 @@ cudaError_t launch_fused_step(const Dev& d, int precision, cudaGraphConditionalH
   const int per_sm = g_fast_ctas_per_sm[precision == MT_FP64 ? 0 : precision == MT_MIXED ? 1 : 2];
   const int g = d.nseg < per_sm * d.nsm ? d.nseg : per_sm * d.nsm;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributePriority;
   at[0].val.priority = g_fast_priority;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3((unsigned int)g);
   cfg.blockDim = dim3(Fast::kT);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = use_cond == kChained ? 2 : 1;
   if (precision == MT_MIXED) return cudaLaunchKernelEx(&cfg, k_step1d<MT_MIXED>, d, cond, use_cond);
   if (precision == MT_MIXED_DF32)
     return cudaLaunchKernelEx(&cfg, k_step1d<MT_MIXED_DF32>, d, cond, use_cond);

@@ -12,6 +12,7 @@ namespace mt {
 // (if HIST).  Thread 0 also resets the per-step counters of the sort.
 template <int DIM, bool MOVE, bool HIST>
 __global__ void __launch_bounds__(kThreads) k_move(Dev d) {
+  chained();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   Ctrl* c = d.ctrl;
   if (p == 0) {
@@ -97,6 +98,7 @@ __device__ __forceinline__ int warp_inclusive(int v, int lane) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_scan(Dev d) {
+  chained();
   constexpr int kWarps = kThreads / 32, kVec = kScanItems / 4;
   __shared__ int s_tile;
   __shared__ int s_warp[kWarps];
@@ -208,6 +210,7 @@ __global__ void __launch_bounds__(kThreads) k_scan(Dev d) {
 // position too).
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_scatter(Dev d) {
+  chained();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur;
@@ -232,6 +235,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(Dev d) {
 // with the large cells' sort and the gather of ids and masses, which the row
 // sums did, it takes the place of 25 us; two particles per thread: no faster).
 __global__ void __launch_bounds__(kThreads) k_place2(Dev d) {
+  chained();
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (p >= d.n) return;
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -267,6 +271,7 @@ __device__ __forceinline__ bool before(long long xa, int sa, long long xb, int s
 }
 
 __global__ void __launch_bounds__(kThreads) k_cellsort(Dev d) {
+  chained();
   const long long k = (long long)blockIdx.x * kThreads + threadIdx.x;
   if (k >= d.ncell) return;
   const int a = d.start[k], b = d.start[k + 1];
@@ -300,6 +305,7 @@ __global__ void __launch_bounds__(kThreads) k_cellsort(Dev d) {
 // ascending (partner i ^ (2j - 1) in the first stage of each merge), which
 // sorts any length when positions >= len are treated as +infinity.
 __global__ void __launch_bounds__(1024) k_bigsort(Dev d) {
+  chained();
   __shared__ long long s_key[kBigSortCap];
   __shared__ int s_src[kBigSortCap];
   Ctrl* c = d.ctrl;
@@ -386,13 +392,13 @@ static unsigned int blocks_for(long long n, int t) { return (unsigned int)((n + 
 cudaError_t launch_move(const Dev& d, bool move, bool hist, cudaStream_t s) {
   const unsigned int g = blocks_for(d.n, kThreads);
   if (d.dim == 1) {
-    if (move && hist) k_move<1, true, true><<<g, kThreads, 0, s>>>(d);
-    else if (move) k_move<1, true, false><<<g, kThreads, 0, s>>>(d);
-    else k_move<1, false, true><<<g, kThreads, 0, s>>>(d);
+    if (move && hist) launch_chained(k_move<1, true, true>, g, kThreads, 0, s, d);
+    else if (move) launch_chained(k_move<1, true, false>, g, kThreads, 0, s, d);
+    else launch_chained(k_move<1, false, true>, g, kThreads, 0, s, d);
   } else {
-    if (move && hist) k_move<2, true, true><<<g, kThreads, 0, s>>>(d);
-    else if (move) k_move<2, true, false><<<g, kThreads, 0, s>>>(d);
-    else k_move<2, false, true><<<g, kThreads, 0, s>>>(d);
+    if (move && hist) launch_chained(k_move<2, true, true>, g, kThreads, 0, s, d);
+    else if (move) launch_chained(k_move<2, true, false>, g, kThreads, 0, s, d);
+    else launch_chained(k_move<2, false, true>, g, kThreads, 0, s, d);
   }
   return cudaGetLastError();
 }
@@ -400,19 +406,19 @@ cudaError_t launch_move(const Dev& d, bool move, bool hist, cudaStream_t s) {
 cudaError_t launch_sort(const Dev& d, cudaStream_t s, Marker& mk) {
   const unsigned int gs = blocks_for(d.ncell, kScanTile);
   mk("scan", s);
-  k_scan<<<gs, kThreads, 0, s>>>(d);
+  launch_chained(k_scan, gs, kThreads, 0, s, d);
   const unsigned int gp = blocks_for(d.n, kThreads);
   mk("scatter", s);
   if (d.dim == 1) {
-    k_scatter<1><<<gp, kThreads, 0, s>>>(d);
+    launch_chained(k_scatter<1>, gp, kThreads, 0, s, d);
     mk("cellsort", s);
-    k_cellsort<<<blocks_for(d.ncell, kThreads), kThreads, 0, s>>>(d);
+    launch_chained(k_cellsort, blocks_for(d.ncell, kThreads), kThreads, 0, s, d);
     mk("bigsort", s);
-    k_bigsort<<<(unsigned int)(d.nbig_cap < 304 ? d.nbig_cap : 304), 1024, 0, s>>>(d);
+    launch_chained(k_bigsort, (unsigned int)(d.nbig_cap < 304 ? d.nbig_cap : 304), 1024, 0, s, d);
   } else {
-    k_scatter<2><<<gp, kThreads, 0, s>>>(d);
+    launch_chained(k_scatter<2>, gp, kThreads, 0, s, d);
     mk("place", s);
-    k_place2<<<gp, kThreads, 0, s>>>(d);
+    launch_chained(k_place2, gp, kThreads, 0, s, d);
   }
   return cudaGetLastError();
 }

@@ -73,6 +73,7 @@ struct ThreadObs<true> {  // double-binary32 masses
 // still to do).  Either writes the row of the step the state follows.
 template <int PR, bool PREV>
 __global__ void __launch_bounds__(kThreads) k_obs(Dev d, int left) {
+  chained();
   using MS = Mass<PR>;
   using MV = typename MS::V;
   constexpr int kPer = kObsChunk / kThreads;  // slots per thread
@@ -155,9 +156,9 @@ cudaError_t launch_obs_prev(const Dev& d, int precision, cudaStream_t s) {
 static cudaError_t obs_of_state(const Dev& d, int precision, int left, cudaStream_t s) {
   if (d.observe_cap <= 0 || d.nochunk <= 0) return cudaSuccess;
   if (precision == MT_MIXED_DF32)
-    k_obs<MT_MIXED_DF32, false><<<d.nochunk, kThreads, 0, s>>>(d, left);
+    launch_chained(k_obs<MT_MIXED_DF32, false>, d.nochunk, kThreads, 0, s, d, left);
   else
-    k_obs<MT_FP64, false><<<d.nochunk, kThreads, 0, s>>>(d, left);  // binary64 masses
+    launch_chained(k_obs<MT_FP64, false>, d.nochunk, kThreads, 0, s, d, left);  // binary64 masses
   return cudaGetLastError();
 }
 
@@ -212,6 +213,7 @@ constexpr int kWalkBins = 64;  // neighbour-count bins of the exchange's lanes
 // leaves the neighbour count, clipped to the bins, in src.
 template <int PR>
 __global__ void __launch_bounds__(kThreads) k_rowsum_walk(Dev d) {
+  chained();
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
@@ -246,6 +248,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_walk(Dev d) {
 // 96 us, with separations wrapped by an addition instead of a 64-bit division).
 template <int PR, int NP>
 __global__ void __launch_bounds__(kThreads) k_exchange_walk(Dev d) {
+  chained();
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -362,6 +365,7 @@ __device__ __forceinline__ TileRanges tile_ranges(long long jl, long long jr, lo
 
 template <int PR>
 __global__ void __launch_bounds__(kThreads) k_rowsum_tile(Dev d) {
+  chained();
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   __shared__ unsigned int s_x[kTileChunk];
@@ -419,6 +423,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_tile(Dev d) {
 
 template <int PR, bool TR>
 __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
+  chained();
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -510,6 +515,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
 // in binary64.  N = 10^6 at 200 per unit length: 4.09 -> 1.09 ms (step 4.47 -> 1.43 ms).
 template <bool TR>
 __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
+  chained();
   using W = Weight<true, 1>;
   using MS = Mass<MT_MIXED>;
   constexpr int kWarps = kThreads / 32, kPer = kTileChunk / kThreads;
@@ -647,11 +653,11 @@ template <int PR, bool TR>
 static void launch_exchange_tile(const Dev& d, unsigned int g, cudaStream_t s, int sp) {
   if constexpr (PR == MT_MIXED) {
     if (d.fix) {
-      k_exchange_tile_fix<TR><<<g, kThreads, 0, s>>>(d, sp);
+      launch_chained(k_exchange_tile_fix<TR>, g, kThreads, 0, s, d, sp);
       return;
     }
   }
-  k_exchange_tile<PR, TR><<<g, kThreads, 0, s>>>(d, sp);
+  launch_chained(k_exchange_tile<PR, TR>, g, kThreads, 0, s, d, sp);
 }
 
 // ================================================== 1-d SPaM (stored P) ==
@@ -889,6 +895,7 @@ __device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, i
 
 template <int PR, bool PER>
 __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
+  chained();
   using W = Weight<mixw(PR), 2>;
   using T = typename W::T;
   __shared__ unsigned long long s_tab[exp_tab_words(PR)];
@@ -934,6 +941,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
 
 template <int PR, bool TR, bool PER>
 __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
+  chained();
   using W = Weight<mixw(PR), 2>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -990,6 +998,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
 // atomic on one address and a wait in every CTA of a large pass cost more
 // (10^6 particles: ~10 us) than a launch.
 __global__ void k_finish(Dev d, int flip_x, int flip_m) {
+  chained();
   Ctrl* c = d.ctrl;
   c->step += 1;
   c->xcur ^= flip_x;
@@ -1121,15 +1130,15 @@ __global__ void __launch_bounds__(kThreads) k_gather_species(Dev d) {
 template <int PR, bool PER>
 static void cell2_passes(const Dev& d, unsigned int g, cudaStream_t s, Marker& mk) {
   mk("rowsum_cell2", s);
-  k_rowsum_cell2<PR, PER><<<g, kThreads, 0, s>>>(d);
+  launch_chained(k_rowsum_cell2<PR, PER>, g, kThreads, 0, s, d);
   for (int sp = 2; sp < d.nspec; sp += 2) {
     mk("exchange_cell2_species", s);
-    k_exchange_cell2<PR, true, PER><<<g, kThreads, 0, s>>>(d, sp);
+    launch_chained(k_exchange_cell2<PR, true, PER>, g, kThreads, 0, s, d, sp);
   }
   mk("exchange_cell2", s);
-  k_exchange_cell2<PR, false, PER><<<g, kThreads, 0, s>>>(d, 0);
+  launch_chained(k_exchange_cell2<PR, false, PER>, g, kThreads, 0, s, d, 0);
   mk("finish", s);
-  k_finish<<<1, 1, 0, s>>>(d, 1, 0);
+  launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
 }
 
 template <int PR, bool TR>
@@ -1170,7 +1179,7 @@ static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
     k_band_exchange<PR, false><<<g, kThreads, 0, s>>>(d, 0);
   } else if (d.dim == 1 && d.tile) {
     mk("rowsum_tile", s);
-    k_rowsum_tile<PR><<<g, kThreads, 0, s>>>(d);
+    launch_chained(k_rowsum_tile<PR>, g, kThreads, 0, s, d);
     if (d.nspec > 2) {
       mk("gather_species", s);
       k_gather_species<<<g, kThreads, 0, s>>>(d);
@@ -1183,18 +1192,18 @@ static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
     launch_exchange_tile<PR, false>(d, g, s, 0);
   } else if (d.dim == 1) {
     mk("rowsum_walk", s);
-    k_rowsum_walk<PR><<<g, kThreads, 0, s>>>(d);
+    launch_chained(k_rowsum_walk<PR>, g, kThreads, 0, s, d);
     mk("exchange_walk", s);
     if (d.nspec <= 2)
-      k_exchange_walk<PR, 1><<<g, kThreads, 0, s>>>(d);
+      launch_chained(k_exchange_walk<PR, 1>, g, kThreads, 0, s, d);
     else if (d.nspec <= 4)
-      k_exchange_walk<PR, 2><<<g, kThreads, 0, s>>>(d);
+      launch_chained(k_exchange_walk<PR, 2>, g, kThreads, 0, s, d);
     else if (d.nspec <= 6)
-      k_exchange_walk<PR, 3><<<g, kThreads, 0, s>>>(d);
+      launch_chained(k_exchange_walk<PR, 3>, g, kThreads, 0, s, d);
     else
-      k_exchange_walk<PR, 4><<<g, kThreads, 0, s>>>(d);
+      launch_chained(k_exchange_walk<PR, 4>, g, kThreads, 0, s, d);
     mk("finish", s);
-    k_finish<<<1, 1, 0, s>>>(d, 1, 0);
+    launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
   } else if (d.periodic) {
     cell2_passes<PR, true>(d, g, s, mk);
   } else {
