@@ -1137,7 +1137,6 @@ static void cell2_passes(const Dev& d, unsigned int g, cudaStream_t s, Marker& m
   }
   mk("exchange_cell2", s);
   launch_chained(k_exchange_cell2<PR, false, PER>, g, kThreads, 0, s, d, 0);
-  mk("finish", s);
   launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
 }
 
@@ -1202,7 +1201,6 @@ static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
       launch_chained(k_exchange_walk<PR, 3>, g, kThreads, 0, s, d);
     else
       launch_chained(k_exchange_walk<PR, 4>, g, kThreads, 0, s, d);
-    mk("finish", s);
     launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
   } else if (d.periodic) {
     cell2_passes<PR, true>(d, g, s, mk);
