@@ -410,7 +410,10 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
       partner = j + 1 + (u - left);
     }
   };
-  // (F) row sums: 1 + left pairs' weights + right pairs' weights, in that order
+  // (F) row sums: 1 + left pairs' weights + right pairs' weights, in that order;
+  // 1 / r_j, or (SYM) 1 / (2 r_j), exactly half of it
+  const bool sym = d.norm != MT_NORM_ROW;
+  const T scale = sym ? T(0.5) : T(1);
   for (int p = tid; p < nrs; p += NT) {
     const int v = perm[p], j = v & 0xffff, left = v >> 16, jj = j - olo;
     const int c = left + (pfx[jj + 1] - pfx[jj]);
@@ -420,13 +423,12 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
       pair_of(j, jj, left, u, q, partner);
       r += sw[q];
     }
-    sr[j] = rcp_ge1(r);
+    sr[j] = scale * rcp_ge1(r);
   }
   __syncthreads();
-  // (G) the symmetric normalisation: each listed pair's 2 P = nu (1/r_j +
-  // 1/r_k) once, in place of nu (the flux sums are halved at the end, exactly;
-  // pairs with an end outside the row-sum range are never read)
-  const bool sym = d.norm != MT_NORM_ROW;
+  // (G) the symmetric normalisation: each listed pair's P = nu (1 / (2 r_j) +
+  // 1 / (2 r_k)) once, in place of nu (pairs with an end outside the row-sum
+  // range are never read)
   if (sym) {
     for (int q = tid; q < np; q += NT) {
       const int jj = own[q];
@@ -454,10 +456,6 @@ __device__ bool pair_transfer(const Dev& d, const StepState& st, unsigned char* 
         const T P = sym ? sw[q] : sw[q] * ip;
         MS::acc(dA, P, MS::diff(MS::load(sA, i), A));
         MS::acc(dB, P, MS::diff(MS::load(sB, i), B));
-      }
-      if (sym) {
-        dA = acc_half(dA);
-        dB = acc_half(dB);
       }
       MS::update(A, B, dA, dB, d.react);
       const long long o = out0 + (j - w0);
@@ -614,6 +612,13 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
     gap[j] = g < kFar ? (unsigned int)g : kFar;
   }
   __syncthreads();
+  // SYM: the integer sums take 2 P = w (1/r_j + 1/r_i) and are halved at the
+  // end; MT_MIXED's binary64 rows halve 2 P (their sums of masses near the end
+  // of binary64's range would overflow otherwise), and MT_MIXED_DF32 keeps
+  // 1 / (2 r): all exact.
+  const bool sym = d.norm != MT_NORM_ROW;
+  const float scale = sym && PR != MT_MIXED ? 0.5f : 1.0f;
+  const float p_scale = sym && PR == MT_MIXED ? 0.5f : 1.0f;
   // (A)
   int v[PER];  // own slots: slot | left pairs << 10 | right pairs << 21
   int np = 0;
@@ -637,7 +642,7 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
     for (unsigned int D = gap[j + 1]; D <= S32; D += gap[j + 1 + ++R])
       r += W::near(d, (int)D, nullptr);
     np += R;
-    sxr[j] = make_uint2((unsigned int)x, __float_as_uint(__frcp_rn(r)));
+    sxr[j] = make_uint2((unsigned int)x, __float_as_uint(__fmul_rn(scale, __frcp_rn(r))));
     if (fix) {
       if ((sA[j] | sB[j]) & 1)
         for (int i = j - L; i <= j + R; ++i) sE[i] |= 0x8000;  // (every writer writes this value)
@@ -688,7 +693,6 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
   __syncthreads();
   // (C)
   const int nown = w1 - w0;
-  const bool sym = d.norm != MT_NORM_ROW;  // 2 P is formed, the sums are halved at the end
   unsigned long long* Mn = d.M[st.mc ^ 1];
   if (out0 + nown > d.n) raise_error(d.ctrl, kErrIndex, out0);
   const unsigned long long* Mo = d.M[st.mc] + a0;
@@ -699,18 +703,14 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
   auto mass_b = [&](int i) {
     return PR == MT_MIXED && sE ? MS::load(Mo, d.n + (sE[i] & 0x7fff)) : MS::load(sB, i);
   };
-  // the normalised weight of slots own, i (twice it in SYM); within the
-  // cutoff the low words' difference is the separation
+  // the normalised weight of slots own, i (MT_MIXED, SYM: twice it); within
+  // the cutoff the low words' difference is the separation
   auto weight = [&](uint2 own, int i) {
     const uint2 q = sxr[i];
     const float w = W::near(d, (int)(q.x - own.x), nullptr), ip = __uint_as_float(own.y);
     return sym ? w * (ip + __uint_as_float(q.y)) : w * ip;
   };
   auto finish = [&](int j, MV A, MV B, typename MS::Acc dA, typename MS::Acc dB) {
-    if (sym) {
-      dA = acc_half(dA);
-      dB = acc_half(dB);
-    }
     MS::update(A, B, dA, dB, d.react);
     const long long o = out0 + (j - w0);
     if (o < d.n) {
@@ -730,7 +730,7 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
 #pragma unroll(PR == MT_MIXED ? 4 : 1)
     for (int u = i0; u < i1; ++u) {
       const int i = u + (u >= j);
-      const float P = weight(own, i);
+      const float P = PR == MT_MIXED ? p_scale * weight(own, i) : weight(own, i);
       MS::acc(dA, P, MS::diff(mass_a(i), A));
       MS::acc(dB, P, MS::diff(mass_b(i), B));
     }
@@ -755,7 +755,8 @@ __device__ bool walk_transfer(const Dev& d, const StepState& st, unsigned char* 
         qa.add((long long)sA[i] - ma, P);
         qb.add((long long)sB[i] - mb, P);
       }
-      finish(j, mass_a(j), mass_b(j), qa.value(EA), qb.value(EB));
+      const double half = sym ? 0.5 : 1.0;
+      finish(j, mass_a(j), mass_b(j), half * qa.value(EA), half * qb.value(EB));
     }
   }
   return true;

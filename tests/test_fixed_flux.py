@@ -168,3 +168,30 @@ def test_exchange_on_the_gpu(kind, norm, L):
         assert np.array_equal(want[~ok & ~np.isnan(want)], got[~ok & ~np.isnan(want)])
         assert np.all(off[ok] <= tol[ok]), np.max(off[ok] / tol[ok])
     sim.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("norm", [mt.MT_NORM_SYM, mt.MT_NORM_ROW])
+@pytest.mark.parametrize("precision", [mt.MT_FP64, mt.MT_MIXED])
+def test_masses_near_the_largest_binary64(precision, norm):
+    """One-kernel step with masses of 0 and 1.79e308: the results, weighted
+    means of the two, are finite, and equal those of the masses scaled by
+    2^-40 (sums of at most ~30 terms in binary64, or in integers: within
+    1e-13 of the largest mass)."""
+    n, L = 3000, 1000.0
+    p = mt.mt_params_init(n=n, L=(L,), D_mt=0.1, D_rw=0.0, dt=1.0, precision=precision, norm=norm,
+                          react=0)
+    x = synth.uniform_positions(n, L, seed=8)
+    g = np.random.default_rng(8)
+    A = np.where(g.random(n) < 0.1, 0.0, 1.79e308)
+    B = np.where(g.random(n) < 0.5, 0.0, 1.79e308)
+    out = []
+    for scale in (1.0, 2.0 ** -40):
+        sim = mt.Simulation(p)
+        sim.upload(x, A * scale, B * scale)
+        sim.step()
+        out.append([m * (2.0 ** -40 / scale) for m in sim.masses()])
+        sim.close()
+    for big, small in zip(*out):
+        assert np.isfinite(big).all()
+        assert np.abs(big - small).max() <= 1e-13 * 1.79e308 * 2.0 ** -40
