@@ -974,8 +974,8 @@ mt_status mt_batch_create(const mt_params* p, const mt_batch* b, void* workspace
   d.scale = std::ldexp(1.0, -D.p.frac_bits);
   d.inv8f = (float)(d.inv8 * d.scale * d.scale);
   exp_constants(d);
-  // P >= e^-7 2^-20 (the row sums are at most a realisation's particles)
-  d.fix = (double)d.S * (double)d.S * d.inv8 * d.scale * d.scale <= 7.0 ? 1 : 0;
+  // P >= e^-6.9 2^-20 > 2^-30 (the row sums are at most a realisation's particles)
+  d.fix = (double)d.S * (double)d.S * d.inv8 * d.scale * d.scale <= 6.9 ? 1 : 0;
   for (const Real& R : D.rt)
     if (R.n > (1LL << 20)) d.fix = 0;
   d.key0 = (unsigned int)(D.p.seed & 0xffffffffu);

@@ -18,7 +18,7 @@
 // staged one is summed in binary64 instead (its result may be as small as
 // the unit lets through), and so is everything when E is out of range
 // (infinities, NaNs, masses near the ends of binary64's range).  Weights below
-// e^-7 (cutoffs far beyond the kernel's width) and realisations of more than
+// e^-6.9 (cutoffs far beyond the kernel's width) and realisations of more than
 // 2^20 particles (row sums that large could take P below 2^-30) keep the
 // binary64 form throughout (Dev::fix).
 #pragma once

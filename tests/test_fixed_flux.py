@@ -4,7 +4,9 @@ on the GPU against a binary64 reference for masses over many decades, of both
 signs, zero, near the ends of binary64's range, infinite and NaN, in the
 sparse (one-kernel step) and the dense (tiled) exchange."""
 import math
+import pathlib
 import random
+import re
 import struct
 from fractions import Fraction
 
@@ -106,6 +108,17 @@ def test_replay_is_no_less_exact_than_binary64(kind):
         err["fix"].append(abs(float(Fraction(value(acc, E)) - exact)) / largest)
         err["f64"].append(abs(float(Fraction(ref) - exact)) / largest)
     assert np.mean(np.square(err["fix"])) <= max(np.mean(np.square(err["f64"])), 2.0 ** -108)
+
+
+def test_smallest_weights_stay_in_the_shift():
+    """The dispatch's bound on the weights and on a realisation's particles
+    keeps P's shift below a word's 32 bits, down to the row normalisation's
+    smallest P (a far neighbour of all the others at one place)."""
+    src = (pathlib.Path(mt.__file__).parent / "csrc" / "mt_api.cu").read_text()
+    limit = float(re.search(r"d\.fix = .* <= ([0-9.]+) \?", src).group(1))
+    most = 1 << int(re.search(r"R\.n > \(1LL << (\d+)\)\) d\.fix", src).group(1))
+    P = math.exp(-limit) * (1 - 1e-5) / most  # (binary32 rounding: < 1e-6)
+    assert 0 <= fix_p(P)[1] <= 31
 
 
 def masses(kind, n, g):
