@@ -1511,7 +1511,17 @@ mt_status mt_load(mt_handle* h, const char* path) {
   CU(cudaStreamSynchronize(h->stream));
   if (h->side) CU(cudaStreamSynchronize(h->side));
   if (h->side2) CU(cudaStreamSynchronize(h->side2));
-  if (!ws.empty()) CU(cudaMemcpy(h->ws, ws.data(), ws.size(), cudaMemcpyHostToDevice));
+  if (!ws.empty()) {
+    // A state is saved between steps, with no graph of several steps running.
+    // (Files written before the control block had these words hold anything
+    // there: the block's place in the workspace was cleared to its size only.)
+    Ctrl c;
+    std::memcpy(&c, ws.data() + h->D.o_ctrl, sizeof c);
+    c.pending = c.todo = c.careful = 0;
+    c.big_mark = 0;
+    std::memcpy(ws.data() + h->D.o_ctrl, &c, sizeof c);
+    CU(cudaMemcpy(h->ws, ws.data(), ws.size(), cudaMemcpyHostToDevice));
+  }
   h->steps = hd.steps;
   h->obs_pending = false;  // the saved state's rows were written before it was saved
   h->uploaded = true;

@@ -76,3 +76,25 @@ def test_step_waits_for_its_predicted_segments(precision):
         sim.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1000, 400000])  # graphs of several steps; of one step
+def test_checkpoint_without_the_graph_words(tmp_path, n):
+    """A file from before the control block held the words of the several-step
+    graphs (bytes 184 on of its 256, the workspace's first) has anything there."""
+    p = mt.mt_params_init(n=n, L=(float(n),), v=(0.5,), precision=mt.MT_MIXED, seed=9)
+    a, b = mt.Simulation(p), mt.Simulation(p)
+    a.upload(synth.uniform_positions(n, float(n), seed=1), *synth.uniform_masses(n, seed=1))
+    a.run(14)
+    path = tmp_path / "old.ckpt"
+    a.save(path)
+    data = bytearray(path.read_bytes())
+    at = len(data) - a.nbytes
+    data[at + 184:at + 256] = b"\xa5" * 72
+    path.write_bytes(data)
+    a.run(26)
+    b.load(path)
+    b.run(26)
+    assert np.array_equal(a.ticks(), b.ticks())
+    for u, v in zip(a.masses(), b.masses()):
+        assert np.array_equal(u, v)
