@@ -1111,7 +1111,9 @@ def fp64_ops_per_step(npairs: int, n: int) -> float:
     orders per unordered pair); per particle and species the update (one
     fused multiply-add), per particle the reaction (a comparison and one
     subtraction: the smaller mass becomes exactly 0) and the walk's product
-    (1)."""
+    (1).  MIXED's first tier forms the flux terms in exact integer
+    arithmetic instead, off this pipe: its fraction says how the step compares
+    with the binary64 form, not how busy the pipe is."""
     return 8.0 * npairs + 5.0 * n
 
 
@@ -1168,8 +1170,9 @@ def variant_object(r, steps: int, name: str, peak: float, peak_kind: str, clocks
         obj["exp_roofline"] = {"bound": "alu", "kernel": "fused_step || fused_pred (concurrent)",
                                "achieved": rate,
                                "peak": exp_peak, "unit": "binary64 exp/s", "frac": rate / exp_peak,
-                               "peak_kind": "measured (mt_probe_rate: the weights' binary64 "
-                                            "exp(-t), exp_neg)",
+                               "peak_kind": "measured (mt_probe_rate: a binary64 "
+                                            "exp(-t), exp_neg; the step forms its "
+                                            "weights in integer arithmetic)",
                                "algo": "one exponential per unordered pair within the cutoff"}
     return obj
 

@@ -10,10 +10,10 @@
 //      into registers;
 //   2. moves them (Eq. 2 on the grid, Sec. 3 walls) -- a particle near a
 //      segment edge is moved by more than one CTA, with the same result;
-//   3. keeps those whose new cell lies in [c0 - hc, c1 + hc), counting-sorts
-//      them into shared-memory bins and sorts each bin by (x, id) (bins of
-//      more than kBinMax particles, e.g. particles piled against a wall, are
-//      sorted by the whole CTA);
+//   3. keeps those whose new cell lies in [c0 - hc, c1 + hc) and sorts them by
+//      (x, id): bins, and in each bin every particle's rank among the bin's
+//      keys (in the first tier a bin of more than kBinMax particles, e.g.
+//      piled against a wall, is sorted by the whole CTA);
 //   4. finds its output offset without a global scan: every particle whose
 //      old cell is below c0 - Dc ends below c0, every particle whose old cell
 //      is at or above c0 + Dc ends at or above c0, so the offset is fstart
@@ -21,7 +21,9 @@
 //      below c0;
 //   5. forms r_i = sum_j nu_ij for every staged particle within Smax of its
 //      cells and dM_i = 1/2 sum_j P_ij (M_j - M_i) for its own particles
-//      (Eq. 3, 4, 7), walking the sorted shared-memory array, then reacts;
+//      (Eq. 3, 4, 7), then reacts: in the first tier binary32 weights by walks
+//      over the sorted slots (walk_transfer) and binary64 ones through a list
+//      of the unordered pairs (pair_transfer), in the cluster tiers by walks;
 //   6. writes its own particles, the next step's fstart for its cells and
 //      the next step's segment boundaries that fall in its output range.
 //
@@ -39,8 +41,7 @@
 // stretch of the tick axis and its own segments (segment starts sslot[] are
 // fixed slots, since a realisation's particles stay in its slot range, and a
 // realisation's first segment starts at its first cell, which no other
-// realisation's particle can reach).  The CTA that finishes the last segment
-// of a realisation reduces that realisation's observables.
+// realisation's particle can reach).
 #include <cooperative_groups.h>
 #include <cuda_pipeline.h>
 

@@ -1,8 +1,8 @@
 // mt_probe.cu -- throughput probes for the non-HBM rooflines of the
 // transfer kernels: binary64 fused multiply-add, binary32 fused
 // multiply-add, the binary32 fast exponential (__expf), the library's
-// binary64 exponential (exp) and the weights' own binary64 exponential
-// (exp_neg).  Not part of the paper: they measure the device peaks the FP64
+// binary64 exponential (exp) and the all-pairs weights' own binary64
+// exponential (exp_neg).  Not part of the paper: they measure the device peaks the FP64
 // and brute-force passes are compared against.  Also the test hook that
 // evaluates exp_neg on a device array.
 //
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe(double* out, int iters,
       if (WHICH == 1) f[k] = __fmaf_rn(f[k], mf, cf);           // binary32 FMA
       if (WHICH == 2) f[k] = __expf(-f[k]);                     // binary32 fast exp
       if (WHICH == 3) a[k] = exp(-a[k]);                        // binary64 exp
-      if (WHICH == 4) a[k] = mt::exp_neg(a[k]);                 // the weights' exp(-t)
+      if (WHICH == 4) a[k] = mt::exp_neg(a[k]);                 // all-pairs exp(-t)
     }
   }
   double s = 0.0;

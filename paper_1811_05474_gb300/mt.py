@@ -421,7 +421,7 @@ def mt_probe_rate(which: int, device="cuda") -> float:
 
 
 def mt_test_exp_neg(t_ptr, out_ptr, n: int, stream_ptr=None) -> None:
-    """Test hook: the weights' binary64 exp(-t) on device arrays (see include/mt.h)."""
+    """Test hook: the all-pairs weights' binary64 exp(-t) on device arrays (see include/mt.h)."""
     check(lib().mt_test_exp_neg(t_ptr, out_ptr, n, stream_ptr))
 
 
