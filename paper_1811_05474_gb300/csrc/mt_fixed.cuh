@@ -1,6 +1,5 @@
-// mt_fixed.cuh -- the flux sum sum_j P_ij (M_j - M_i) of binary64 masses (Eq. 4)
-// with binary32 P (MT_MIXED; described here) or binary64 P (MT_FP64's dense
-// tiles) in exact integer arithmetic.
+// mt_fixed.cuh -- the flux sum of MT_MIXED, sum_j P_ij (M_j - M_i) with
+// binary32 P and binary64 masses (Eq. 4), in exact integer arithmetic.
 //
 // The binary64 pipe takes ~19 cycles of a multiprocessor per warp instruction
 // (one sixty-fourth of the binary32 rate), so the four binary64 operations per
@@ -71,21 +70,6 @@ __device__ __forceinline__ FixP fix_p(float P) {
   return {((u & 0x7fffffu) | 0x800000u) << 7, 128 - (int)(u >> 23)};
 }
 
-// A binary64 P (or 2 P, same range) as a 62-bit integer, in a signed low word
-// and the rest, and a right shift: P = p 2^-60 after the shift.
-struct FixP64 {
-  int hi, lo;
-  int s;
-};
-__device__ __forceinline__ FixP64 fix_p(double P) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(P);
-  const unsigned int h = (unsigned int)(u >> 32), l = (unsigned int)u;
-  const int lo = (int)(l << 9);
-  const int hi = (int)((((h & 0xfffffu) | 0x100000u) << 9) | (l >> 23)) + (int)(l << 9 >> 31);
-  return {hi, lo, 1024 - (int)(h >> 20)};
-}
-constexpr int kFixP64Unit = 1;  // a sum's unit is 2^-28 with P in binary64, 2^-29 in binary32
-
 // 96-bit sum of (difference p) >> s.
 struct FixAcc {
   unsigned int a0 = 0, a1 = 0, a2 = 0;
@@ -96,21 +80,6 @@ struct FixAcc {
     const int x2 = (int)(t1 >> 32);
     const unsigned int y0 = __funnelshift_r(x0, x1, f.s), y1 = __funnelshift_r(x1, x2, f.s);
     const int y2 = x2 >> f.s;
-    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
-        : "+r"(a0), "+r"(a1), "+r"(a2)
-        : "r"(y0), "r"(y1), "r"(y2));
-  }
-  // The same with a binary64 P: the product's words 1 to 3 (its lowest 32 bits
-  // are 2^-92 of the largest term), from the four 32-bit products of signed
-  // low words.
-  __device__ __forceinline__ void add(long long diff, FixP64 f) {
-    const int dl = (int)diff, dh = (int)(diff >> 32) + (int)((unsigned int)dl >> 31);
-    const long long mid = (long long)dl * f.hi + __mulhi(dl, f.lo) + (long long)dh * f.lo;
-    const long long t1 = (long long)dh * f.hi + (mid >> 32);
-    const unsigned int x0 = (unsigned int)mid, x1 = (unsigned int)t1;
-    const int x2 = (int)(t1 >> 32);
-    const unsigned int y0 = __funnelshift_r(x0, x1, f.s), y1 = __funnelshift_r(x1, x2, f.s);
-    const int y2 = x2 >> (f.s & 31);
     asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
         : "+r"(a0), "+r"(a1), "+r"(a2)
         : "r"(y0), "r"(y1), "r"(y2));

@@ -150,7 +150,7 @@ struct Dev {
   unsigned long long ec;    // binary64 weights: log2(e) inv8 2^-2k in fixed point (exp_fix),
   unsigned long long emax;  // ... the largest squared separation that does not underflow,
   int eq, eib;              // ... left shift of the square, integer bits of the exponent
-  int fix;                  // 1: integer flux sums (mt_fixed.cuh): 2^-30 <= P <= 1
+  int fix;                  // 1: integer flux sums in MT_MIXED (mt_fixed.cuh): 2^-30 <= P <= 1
   unsigned int key0, key1;  // Philox key (seed)
   unsigned int real;        // realisation counter word
   int nbig_cap;

@@ -503,39 +503,23 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
   if (!TR) finish_step(d, 1, 0);
 }
 
-// The exchange of binary64 masses over the same tiles with the flux sums in exact integer
+// MT_MIXED's exchange over the same tiles with the flux sums in exact integer
 // arithmetic (mt_fixed.cuh): the binary64 form above spends its time in four
 // binary64 instructions per ordered pair (~76 of ~80 cycles per warp and
 // pair at the paper's density); here a pair is ~55 integer and binary32
 // instructions, issue-bound.  Each chunk's masses, and the rows' own, are
 // converted with the largest exponent among them, and a chunk's sum is rounded
-// to binary64 once.
-// MT_MIXED: a lane whose neighbours in the chunk hold a marked mass
+// to binary64 once.  A lane whose neighbours in the chunk hold a marked mass
 // and no large one (fix_large; looked for only where the chunk holds marked
 // masses, first in blocks of 32 slots wholly inside its range) sums the chunk
 // in binary64.  N = 10^6 at 200 per unit length: 4.09 -> 1.09 ms (step 4.47 -> 1.43 ms).
-// MT_FP64: the same with binary64 weights (exp_fix) and 2 P, of ~95
-// instructions per pair two in binary64 in place of six.  The marked masses'
-// lost bits add up to at most 2^-60 of the largest mass in a row's result; a
-// row with marked masses whose flux sum and own mass are both below 2^-4 of
-// the largest (elsewhere that is less than a quarter of the result's own
-// rounding) is summed again in binary64.  75 realisations at up to 500 per
-// unit length: exchange 1.31 -> 0.99 ms (step 1.78 -> 1.46 ms).
-template <int PR, bool TR>
+template <bool TR>
 __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   chained();
-  using W = Weight<mixw(PR), 1>;
-  using T = typename W::T;
-  using MS = Mass<PR>;
+  using W = Weight<true, 1>;
+  using MS = Mass<MT_MIXED>;
   constexpr int kWarps = kThreads / 32, kPer = kTileChunk / kThreads;
-  constexpr int kUnit = PR == MT_FP64 ? kFixP64Unit : 0;
-  __shared__ unsigned long long s_tab[exp_tab_words(PR)];
-  if (!mixw(PR)) exp_table<kThreads>(s_tab);
-  struct alignas(8) Slot {
-    unsigned int x;  // low word of the position
-    T r;             // 1 / r
-  };
-  __shared__ Slot s_xr[kTileChunk];
+  __shared__ uint2 s_xr[kTileChunk];       // low word of the position, 1 / r
   __shared__ longlong2 s_ab[kTileChunk];   // fixed masses
   __shared__ long long s_lohi[2];
   __shared__ int s_e[kWarps][2];                       // largest exponents
@@ -558,11 +542,8 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   const unsigned int x32 = (unsigned int)x;
   const bool sym = d.norm != MT_NORM_ROW;  // 2 P is formed, the sums are halved at the end
   const unsigned long long Ab = valid ? MA[p] : 0, Bb = valid ? MB[p] : 0;
-  const T ip = valid ? load_rinv<mixw(PR)>(d, p) : T(0);
+  const float ip = valid ? load_rinv<true>(d, p) : 0.0f;
   double dA = 0.0, dB = 0.0;
-  // MT_FP64: the largest exponent among the row's chunks with marked masses
-  constexpr int kNever = 1 << 20;
-  int maxa = 0, maxb = 0;
   for (long long c0 = t.lo; c0 < t.hi; c0 += kTileChunk) {
     const int nc = (int)min((long long)kTileChunk, t.hi - c0);
     unsigned long long va[kPer], vb[kPer];
@@ -572,8 +553,10 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       const int i = threadIdx.x + k * kThreads;
       va[k] = i < nc ? MA[c0 + i] : 0;
       vb[k] = i < nc ? MB[c0 + i] : 0;
-      if (i < nc)
-        s_xr[i] = Slot{(unsigned int)Xs[c0 + i], sym ? load_rinv<mixw(PR)>(d, c0 + i) : T(0)};
+      if (i < nc) {
+        s_xr[i] = make_uint2((unsigned int)Xs[c0 + i],
+                             sym ? __float_as_uint(load_rinv<true>(d, c0 + i)) : 0u);
+      }
       ea = max(ea, fix_exponent(va[k]));
       eb = max(eb, fix_exponent(vb[k]));
     }
@@ -614,7 +597,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
     // this lane's slots of the chunk
     const int l0 = (int)(max(jl, c0) - c0), l1 = (int)(min(jr, c0 + nc) - c0);
     auto small = [&](int h, long long own) {
-      if (PR == MT_FP64 || (!s_mark[h] && !(own & 1))) return false;
+      if (!s_mark[h] && !(own & 1)) return false;
       unsigned int z = fix_size(own);
       for (int b = (l0 + 31) / 32; b < l1 / 32; ++b) z |= s_size[h][b];
       for (int j = l0; j < l1 && !fix_large(z); ++j) z |= fix_size(h ? s_ab[j].y : s_ab[j].x);
@@ -625,32 +608,23 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
     FixAcc qa, qb;
 #pragma unroll 2
     for (int j = j0; j < j1; ++j) {
-      const Slot xr = s_xr[j];
+      const uint2 xr = s_xr[j];
       const longlong2 ab = s_ab[j];
-      const T w = W::near(d, (int)(xr.x - x32), s_tab);
-      auto P = fix_p(w * (ip + xr.r));
-      const bool out = (unsigned int)(j - ql) >= qn;
-      if constexpr (PR == MT_FP64) {
-        if (out) P.hi = P.lo = 0;
-      } else {
-        if (out) P.p = 0;
-      }
+      const float w = W::near(d, (int)(xr.x - x32), nullptr);
+      FixP P = fix_p(w * (ip + __uint_as_float(xr.y)));
+      if ((unsigned int)(j - ql) >= qn) P.p = 0;
       qa.add(ab.x - fa, P);
       qb.add(ab.y - fb, P);
     }
     if (l0 < l1) {
-      // units: 2^(E - 1083) of the masses, 2^-29 (binary64: 2^-28) of 2 P
-      double ca = qa.value(EA + kUnit), cb = qb.value(EB + kUnit);
-      if constexpr (PR == MT_FP64) {
-        if (s_mark[0] || (fa & 1)) maxa = max(maxa, EA);
-        if (s_mark[1] || (fb & 1)) maxb = max(maxb, EB);
-        if (!fixa) maxa = kNever;
-        if (!fixb) maxb = kNever;
-      } else if (!fixa || !fixb) {
+      double ca = qa.value(EA), cb = qb.value(EB);
+      // units: 2^(E - 1083) of the masses, 2^-29 of 2 P
+      if (!fixa || !fixb) {
         double ga = 0.0, gb = 0.0;
         const double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
         for (int j = l0; j < l1; ++j) {
-          const T P = W::near(d, (int)(s_xr[j].x - x32), s_tab) * (ip + s_xr[j].r);
+          const float P = W::near(d, (int)(s_xr[j].x - x32), nullptr) *
+                          (ip + __uint_as_float(s_xr[j].y));
           MS::acc(ga, P, MS::diff(MS::load(MA, c0 + j), A));
           MS::acc(gb, P, MS::diff(MS::load(MB, c0 + j), B));
         }
@@ -661,25 +635,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       dB += cb;
     }
     __syncthreads();
-  }
-  if constexpr (PR == MT_FP64) {
-    auto small = [](double sum, unsigned long long own, int E) {
-      const unsigned long long s = (unsigned long long)__double_as_longlong(sum);
-      return max(fix_exponent(s), fix_exponent(own)) < E - 4;
-    };
-    const bool reda = small(dA, Ab, maxa), redb = small(dB, Bb, maxb);
-    if (reda || redb) {
-      double ga = 0.0, gb = 0.0;
-      const double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
-      for (long long j = jl; j < jr; ++j) {
-        const T P = W::near(d, (int)((unsigned int)Xs[j] - x32), s_tab) *
-                    (ip + (sym ? load_rinv<false>(d, j) : T(0)));
-        MS::acc(ga, P, MS::diff(MS::load(MA, j), A));
-        MS::acc(gb, P, MS::diff(MS::load(MB, j), B));
-      }
-      if (reda) dA = ga;
-      if (redb) dB = gb;
-    }
   }
   if (sym) {
     dA = acc_half(dA);
@@ -696,9 +651,9 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
 
 template <int PR, bool TR>
 static void launch_exchange_tile(const Dev& d, unsigned int g, cudaStream_t s, int sp) {
-  if constexpr (PR != MT_MIXED_DF32) {
+  if constexpr (PR == MT_MIXED) {
     if (d.fix) {
-      launch_chained(k_exchange_tile_fix<PR, TR>, g, kThreads, 0, s, d, sp);
+      launch_chained(k_exchange_tile_fix<TR>, g, kThreads, 0, s, d, sp);
       return;
     }
   }
