@@ -1123,13 +1123,14 @@ mt_status mt_run(mt_handle* h, int64_t nsteps) {
     return MT_OK;
   }
   int64_t left = nsteps;
-  if (h->D.fused && !h->dev.use_pred && left >= kMultiSteps) {
+  // With observables of binary64 masses the one-step graphs are the faster
+  // form: they run a step's observables beside the next step (N = 46773
+  // MT_FP64: 44 us per step against 51 in a graph of several steps).
+  if (h->D.fused && !h->dev.use_pred && !h->obs_defer && left >= kMultiSteps) {
     if (!h->multi) {
       const mt_status s = build_multi(h);
       if (s != MT_OK) return s;
     }
-    const mt_status s = flush_obs(h);  // the graph's first step overwrites what they read
-    if (s != MT_OK) return s;
     for (; left >= kMultiSteps; left -= kMultiSteps) {
       CU(cudaGraphLaunch(h->multi, h->stream));
       h->steps += kMultiSteps;
