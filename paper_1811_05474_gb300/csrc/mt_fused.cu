@@ -1064,8 +1064,7 @@ __device__ int fast_segment(const Dev& d, const StepState& st, int seg, unsigned
 // nothing of it has been written).
 template <int PR, typename TR, int CL>
 __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigned char* smem,
-                             const SegScalars& g, int slice, bool* heavy_out = nullptr,
-                             bool cache_w = false) {
+                             const SegScalars& g, int slice, bool* heavy_out = nullptr) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -1078,7 +1077,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
   T* sr = reinterpret_cast<T*>(sid + CAP);
   int* bstart = reinterpret_cast<int*>(sr + CAP);  // [NB + 1]
   int* bcur = bstart + NB + 1;                     // [NB]
-  __shared__ int s_lt, s_w0, s_w1, s_bad, s_nbig, s_work, s_nd, s_nd2, s_wcbad, s_wcok;
+  __shared__ int s_lt, s_w0, s_w1, s_bad, s_nbig, s_work, s_nd, s_nd2;
   __shared__ int s_big[kBigMax];
   __shared__ int s_scan[NT / 32];
 
@@ -1355,6 +1354,13 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
   const int w0 = s_w0, w1 = s_w1;
   const long long out0 = o0 + s_lt;
   const long long S = d.S;
+  // 1 / r_j, or (SYM) 1 / (2 r_j), exactly half of it: P without a product
+  const bool sym = d.norm != MT_NORM_ROW;
+  const T scale = sym ? T(0.5) : T(1);
+  auto scaled_inverse = [&](T r) {
+    return scale * (mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r)));
+  };
+  auto weight = [&](T w, T ip, T iq) { return sym ? w * (ip + iq) : w * ip; };
   // Row sums.  A particle with more than kWalk neighbours on a side is
   // dense: it is queued (in bcur, free by now) and summed by a whole warp,
   // lanes striding over its neighbour range, combined in a fixed tree.  The
@@ -1378,27 +1384,22 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       T r = T(1);
       for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) r += W::near(d, x - sx[q], st.tab);
       for (int q = j + 1; q < m && sx[q] - x <= S; ++q) r += W::near(d, sx[q] - x, st.tab);
-      sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
+      sr[j] = scaled_inverse(r);
     }
   }
   __syncthreads();
-  // Binary64 weights of dense rows are dear (an exponential each): the
-  // predicted-segment kernel keeps them, row j of the staged slots at
-  // wc[j m + q], between the row sums and the exchange (read through L2:
-  // the rows are written by other CTAs of the cluster)
-  constexpr bool kCache = PR == MT_FP64;
-  const bool cw = kCache && cache_w && (long long)m * m <= d.wc_cap;
+  // (dense rows' weights are formed again in the exchange: with integer
+  // arithmetic that is faster than keeping them in the workspace and reading
+  // them back through L2, 5 10^5 particles with a wall layer in MT_FP64:
+  // 161 -> 154 us per step, and 143 without the product by 1/2 per pair)
   if (active) {
     const int nd = s_nd < NB ? s_nd : NB;
     for (int k = warp; k < nd; k += NT / 32) {
       const int j = dlist[k];
       const long long x = sx[j];
       const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
-      T* wrow = kCache ? reinterpret_cast<T*>(d.wc) + (size_t)j * m : nullptr;
       auto nu = [&](int qq) {
-        const T w = W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
-        if (kCache && cw) wrow[qq] = w;
-        return w;
+        return W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
       };
       // four chains per lane
       T r0 = T(0), r1 = T(0), r2 = T(0), r3 = T(0);
@@ -1411,7 +1412,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       }
       for (; q < hi; q += 32) r0 += nu(q);
       const T r = warp_sum((r0 + r1) + (r2 + r3));
-      if (lane == 0) sr[j] = mixw(PR) ? T(__frcp_rn((float)r)) : T(rcp_ge1((double)r));
+      if (lane == 0) sr[j] = scaled_inverse(r);
     }
   }
   // Every CTA of the cluster staged and sorted the same particles; each
@@ -1419,13 +1420,7 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
   // peers' shared memory (distributed shared memory), between two cluster
   // barriers so no CTA reads a peer that has moved on.
   cg::cluster_group cl = cg::this_cluster();
-  if (tid == 0) s_wcbad = s_nd > NB ? 1 : 0;  // a dense row summed without the cache
   cl.sync();
-  if (tid == 0) {
-    int bad = 0;
-    for (int r = 0; r < CL; ++r) bad |= *cl.map_shared_rank(&s_wcbad, r);
-    s_wcok = bad ? 0 : 1;
-  }
   if (active) {
     for (int j = tid; j < m; j += NT) {
       const int owner = j % CL;
@@ -1454,12 +1449,12 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       MV A = MS::load(sA, j), B = MS::load(sB, j);
       typename MS::Acc dA{}, dB{};
       for (int q = j - 1; q >= 0 && x - sx[q] <= S; --q) {
-        const T P = normalised<T>(d.norm, W::near(d, x - sx[q], st.tab), ip, sr[q]);
+        const T P = weight(W::near(d, x - sx[q], st.tab), ip, sr[q]);
         MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
         MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
       }
       for (int q = j + 1; q < m && sx[q] - x <= S; ++q) {
-        const T P = normalised<T>(d.norm, W::near(d, sx[q] - x, st.tab), ip, sr[q]);
+        const T P = weight(W::near(d, sx[q] - x, st.tab), ip, sr[q]);
         MS::acc(dA, P, MS::diff(MS::load(sA, q), A));
         MS::acc(dB, P, MS::diff(MS::load(sB, q), B));
       }
@@ -1489,14 +1484,9 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       const int lo = lower_at_least(sx, m, x - S), hi = lower_at_least(sx, m, x + S + 1);
       // four chains per lane (q, q + 32, q + 64, q + 96), merged at the end
       typename MS::Acc cA[4] = {}, cB[4] = {};
-      // the row's weights from the cache where every dense row went in
-      const bool from_c = kCache && cw && s_wcok;
-      const T* wrow = reinterpret_cast<const T*>(d.wc) + (size_t)j * m;
       auto pair = [&](int qq, int ch) {
         if (qq == j) return;
-        const T w =
-            from_c ? __ldcg(&wrow[qq]) : W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab);
-        const T P = normalised<T>(d.norm, w, ip, sr[qq]);
+        const T P = weight(W::near(d, x > sx[qq] ? x - sx[qq] : sx[qq] - x, st.tab), ip, sr[qq]);
         MS::acc(cA[ch], P, MS::diff(MS::load(sA, qq), A));
         MS::acc(cB[ch], P, MS::diff(MS::load(sB, qq), B));
       };
@@ -1522,9 +1512,6 @@ __device__ int fused_segment(const Dev& d, const StepState& st, int seg, unsigne
       }
     }
   }
-  // no CTA of the cluster writes the next segment's cached rows before
-  // every CTA has read this segment's (cw is the same in all of them)
-  if (kCache && cw) cg::this_cluster().sync();
   if (active && slice == 0)
     segment_tables<NT>(d, sc, seg, sx, bstart, sh2, wlo, g.c0, g.c1, w0, w1, out0, d.sslot[seg],
                        d.sslot[seg + 1]);
@@ -1720,7 +1707,7 @@ __global__ void __launch_bounds__(Big::kT, 1)
         const int seg = s_list[k];
         bool heavy = true;
         const int rc = fused_segment<PR, Big, CL>(d, st, seg, smem, load_seg(d, sc, Dc, seg), rank,
-                                                  &heavy, true);
+                                                  &heavy);
         if (rc != kSegOk && tid == 0 && atomicExch(&c->overflow, 1) == 0) {
           c->ov_reason = rc;
           c->ov_seg = seg;
