@@ -216,10 +216,6 @@ __device__ __forceinline__ long long wrap(long long y, long long Lq) {
   const long long m = y % Lq;
   return m < 0 ? m + Lq : m;
 }
-// The same for the difference of two positions in [0, Lq).
-__device__ __forceinline__ long long wrap_gap(long long y, long long Lq) {
-  return y < 0 ? y + Lq : y;
-}
 
 // Periodic walls in 1-d: the ring of sorted slots a particle's walks go
 // around -- its realisation's slot range [off, off + n) -- and the domain
@@ -237,6 +233,14 @@ __device__ __forceinline__ long long ring_step(const Ring& g, long long p, long 
   if (q < g.off) q += g.n;
   else if (q >= g.off + g.n) q -= g.n;
   return q;
+}
+// Ticks from position xa, of sorted slot a, up to xb, of slot b != a to its
+// right on the ring.  A walk that has come round to a lower slot has crossed
+// the wall, also where the two positions are equal: particles that all lie
+// within Smax of one another meet once, and not again around the ring.
+__device__ __forceinline__ long long ring_gap(const Ring& g, long long a, long long xa,
+                                              long long b, long long xb) {
+  return xb - xa + (b < a ? g.Lq : 0);
 }
 
 // Periodic walls: the minimum-image separation of two positions in [0, Lq),

@@ -183,7 +183,7 @@ __global__ void k_pairs_walk(Dev d, int* pi, int* pj, long long cap) {
   const Ring g = ring_of(d, id[p]);
   for (long long k = 1; k < g.n; ++k) {
     const long long q = ring_step(g, p, k);
-    const long long D = wrap_gap(X[q] - x, g.Lq);
+    const long long D = ring_gap(g, p, x, q, X[q]);
     if (D > d.S) break;
     emit(d, id[p], id[q], pi, pj, cap);
   }

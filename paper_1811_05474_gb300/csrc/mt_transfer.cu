@@ -174,8 +174,8 @@ cudaError_t launch_obs_step(const Dev& d, int precision, int j, int steps, cudaS
 
 // Calls f(q, D) for the neighbours of the particle in sorted slot p at x, left
 // ones (nearest first), then right ones.  id: the particle's (periodic walls:
-// the walks go around its realisation's ring; 2 Smax < L, so no slot is
-// reached from both sides).
+// the walks go around its realisation's ring; 2 Smax < L and a walk that comes
+// round has crossed the wall (ring_gap), so no slot is reached from both sides).
 template <class F>
 __device__ __forceinline__ void walk_visit(const Dev& d, const long long* Xs, long long p,
                                            long long x, int id, F&& f) {
@@ -194,13 +194,13 @@ __device__ __forceinline__ void walk_visit(const Dev& d, const long long* Xs, lo
     const Ring g = ring_of(d, id);
     for (long long k = 1; k < g.n; ++k) {
       const long long q = ring_step(g, p, -k);
-      const long long D = wrap_gap(x - Xs[q], g.Lq);
+      const long long D = ring_gap(g, q, Xs[q], p, x);
       if (D > d.S) break;
       f(q, D);
     }
     for (long long k = 1; k < g.n; ++k) {
       const long long q = ring_step(g, p, k);
-      const long long D = wrap_gap(Xs[q] - x, g.Lq);
+      const long long D = ring_gap(g, p, x, q, Xs[q]);
       if (D > d.S) break;
       f(q, D);
     }
@@ -702,7 +702,7 @@ __device__ __forceinline__ long long walk_left(const Dev& d, const Ring& g, long
 // Tick distance from slot q up to slot p (p to the right of q).
 __device__ __forceinline__ long long gap(const Dev& d, const Ring& g, const long long* Xs,
                                          long long q, long long p) {
-  return d.periodic ? wrap_gap(Xs[p] - Xs[q], g.Lq) : Xs[p] - Xs[q];
+  return d.periodic ? ring_gap(g, q, Xs[q], p, Xs[p]) : Xs[p] - Xs[q];
 }
 
 template <int PR>
