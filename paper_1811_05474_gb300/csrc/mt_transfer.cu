@@ -449,16 +449,17 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
   if (valid) exact_range(d, Xs, x, jl, jr);
   const TileRanges t = tile_ranges(jl, jr, b0, b1, s_lohi);
   const unsigned int x32 = (unsigned int)x;
-  // SYM: P = w (1/r_p + 1/r_q) / 2 is formed as 2P = w (1/r_p + 1/r_q) and
-  // the sums are halved at the end; ROW: P = w / r_p (the staged 1/r_q is
-  // 0).  Halving is exact, so the result is the same as with P.
+  // SYM: P = w (1/(2 r_p) + 1/(2 r_q)), the halves exact; ROW: P = w / r_p (the
+  // staged 1/r_q is 0).  (Sums of 2 P overflow for masses beyond half of
+  // binary64's range, whose weighted means are finite.)
   const bool sym = d.norm != MT_NORM_ROW;
+  const T scale = sym ? T(0.5) : T(1);
   MV A{}, B{};
   T ip = T(0);
   if (valid) {
     A = MS::load(MA, p);
     B = MS::load(MB, p);
-    ip = load_rinv<mixw(PR)>(d, p);
+    ip = scale * load_rinv<mixw(PR)>(d, p);
   }
   // two accumulator sets (even and odd candidates) halve the dependent
   // chain of compensated additions
@@ -467,7 +468,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
     const int nc = (int)min((long long)kTileChunk, t.hi - c0);
     for (int i = threadIdx.x; i < nc; i += kThreads) {
       s_x[i] = (unsigned int)Xs[c0 + i];
-      s_r[i] = sym ? load_rinv<mixw(PR)>(d, c0 + i) : T(0);
+      s_r[i] = sym ? scale * load_rinv<mixw(PR)>(d, c0 + i) : T(0);
       s_a[i] = MS::load(MA, c0 + i);
       s_b[i] = MS::load(MB, c0 + i);
     }
@@ -477,9 +478,9 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
     const unsigned int qn = (unsigned int)(jr - jl);
     auto pair = [&](int j, typename MS::Acc& a, typename MS::Acc& b) {
       const T w = W::near(d, (int)(s_x[j] - x32), s_tab);
-      const T P2 = (unsigned int)(j - ql) < qn ? w * (ip + s_r[j]) : T(0);
-      MS::acc(a, P2, MS::diff(s_a[j], A));
-      MS::acc(b, P2, MS::diff(s_b[j], B));
+      const T P = (unsigned int)(j - ql) < qn ? w * (ip + s_r[j]) : T(0);
+      MS::acc(a, P, MS::diff(s_a[j], A));
+      MS::acc(b, P, MS::diff(s_b[j], B));
     };
     int j = j0;
     for (; j + 1 < j1; j += 2) {
@@ -491,10 +492,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
   }
   dA = acc_merge(dA, dA1);
   dB = acc_merge(dB, dB1);
-  if (sym) {
-    dA = acc_half(dA);
-    dB = acc_half(dB);
-  }
   if (valid) {
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
@@ -540,7 +537,11 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   if (valid) exact_range(d, Xs, x, jl, jr);
   const TileRanges t = tile_ranges(jl, jr, b0, b1, s_lohi);
   const unsigned int x32 = (unsigned int)x;
-  const bool sym = d.norm != MT_NORM_ROW;  // 2 P is formed, the sums are halved at the end
+  // SYM: the integer sums take 2 P and are halved; the binary64 sums take P
+  // (those of 2 P overflow for masses beyond half of binary64's range)
+  const bool sym = d.norm != MT_NORM_ROW;
+  const float p_scale = sym ? 0.5f : 1.0f;
+  const double half = sym ? 0.5 : 1.0;
   const unsigned long long Ab = valid ? MA[p] : 0, Bb = valid ? MB[p] : 0;
   const float ip = valid ? load_rinv<true>(d, p) : 0.0f;
   double dA = 0.0, dB = 0.0;
@@ -617,14 +618,14 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       qb.add(ab.y - fb, P);
     }
     if (l0 < l1) {
-      double ca = qa.value(EA), cb = qb.value(EB);
+      double ca = half * qa.value(EA), cb = half * qb.value(EB);
       // units: 2^(E - 1083) of the masses, 2^-29 of 2 P
       if (!fixa || !fixb) {
         double ga = 0.0, gb = 0.0;
         const double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
         for (int j = l0; j < l1; ++j) {
           const float P = W::near(d, (int)(s_xr[j].x - x32), nullptr) *
-                          (ip + __uint_as_float(s_xr[j].y));
+                          (ip + __uint_as_float(s_xr[j].y)) * p_scale;
           MS::acc(ga, P, MS::diff(MS::load(MA, c0 + j), A));
           MS::acc(gb, P, MS::diff(MS::load(MB, c0 + j), B));
         }
@@ -635,10 +636,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       dB += cb;
     }
     __syncthreads();
-  }
-  if (sym) {
-    dA = acc_half(dA);
-    dB = acc_half(dB);
   }
   if (valid) {
     double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
