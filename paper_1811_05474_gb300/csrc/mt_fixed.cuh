@@ -6,21 +6,33 @@
 // ordered pair and species pair hold it for ~76 cycles, while the ~30 integer
 // instructions here take ~8 issue cycles of the four schedulers.
 //
-// Masses become 61-bit integers in units of 2^(E - 1083), E the largest
-// biased exponent among the staged masses of the species; the 53-bit
-// significand of any mass of at least 2^-7 of the largest one is kept
-// exactly.  A smaller mass may lose bits below that unit; its last bit is then
-// set, which marks it.  Differences are exact, P's 24-bit significand times a
-// difference is exact in 96 bits, and the products are shifted by P's exponent
-// and added in 96 bits (unit 2^-29 of the masses'): one rounding, to binary64,
-// at the end, where the binary64 form rounds every difference and every term.
-// A row that holds a marked mass and no mass of at least 2^-2 of the largest
-// staged one is summed in binary64 instead (its result may be as small as
-// the unit lets through), and so is everything when E is out of range
-// (infinities, NaNs, masses near the ends of binary64's range).  Weights below
-// e^-6.9 (cutoffs far beyond the kernel's width) and realisations of more than
-// 2^20 particles (row sums that large could take P below 2^-30) keep the
-// binary64 form throughout (Dev::fix).
+// Masses become 61-bit integers in units of u = 2^(E - 1083), E the largest
+// biased exponent among the staged masses of the species.  A mass other than
+// zero is marked if it loses bits below u or lies more than 2^16 below the
+// largest: its last bit is set, and it is off by less than u.  (Small masses
+// that keep every bit are common: a reaction leaves differences of larger ones,
+// on their coarse grid.  Marking every mass below 2^-7 of the largest made the
+// one-kernel step 3-8 % slower.)  Differences are exact, P's 24-bit significand
+// times a difference is exact in 96 bits, and the products are shifted by P's
+// exponent and added in 96 bits (unit 2^-29 u): one rounding, to binary64, at
+// the end, where the binary64 form rounds every difference and every term.
+//   A row of c terms without a marked mass: its sum is off by less than
+// c 2^-29 u, its new mass M' = M + sum / 2 by half of that; its nonzero masses
+// are at least 2^44 u.
+//   A row with one: the marks make the sum wrong by less than 2 sum_j P u, M'
+// by sum_j P u ~ u.
+//   In the first tier a row with a marked mass is summed in binary64; without
+// one, M' is zero or at least 2^43 u P, P the largest of its nonzero neighbours'
+// (2^-20 at the least there), and off by c 2^-73 / P of itself.  In the dense
+// tiles a row is if its M' does not outweigh the error by 2^53 (FixAcc::keeps: u or,
+// with 2^20 terms, 2^-10 u).  So a sum that is kept costs M' no more than about
+// one rounding more.
+//   Everything is summed in binary64 when E is out of range (infinities, NaNs,
+// masses near the ends of binary64's range), where weights fall below e^-6.9
+// (cutoffs far beyond the kernel's width) and in systems that hold a
+// realisation of more than 2^20 particles (row sums that large could take P
+// below 2^-30; Dev::fix): N = 1.1 10^6 at one per unit length then takes ~1.1
+// times, at 200 per unit length ~3 times as long as with integers.
 #pragma once
 
 #include "mt_pair.cuh"
@@ -37,27 +49,16 @@ __device__ __forceinline__ int fix_exponent(unsigned long long bits) {
 __device__ __forceinline__ int fix_scale(int emax) { return emax == 0 ? 1023 : emax; }
 __device__ __forceinline__ bool fix_covers(int E) { return E >= 200 && E <= 2030; }
 
-// A mass in units of 2^(E - 1083); odd if bits were lost.
+// A mass in units of 2^(E - 1083); odd if it is marked.
 __device__ __forceinline__ long long to_fix(unsigned long long bits, int E) {
   const int e = fix_exponent(bits);
   const unsigned long long m =
       ((bits & ((1ULL << 52) - 1)) | ((unsigned long long)(e != 0) << 52)) << 8;
   const int sh = E - (e != 0 ? e : 1);
-  unsigned long long v = sh < 64 ? m >> (sh < 63 ? sh : 63) : 0;
-  if (sh > 7 && m != 0) {
-    const bool lost = sh >= 63 || (v << sh) != m || (v & 1);
-    v = (v & ~1ULL) | (lost ? 1 : 0);
-  }
+  unsigned long long v = m >> (sh < 63 ? sh : 63);
+  if (sh > 7 && m != 0) v |= sh > 16 || (v << sh) != m ? 1 : 0;
   return (long long)bits < 0 ? -(long long)v : (long long)v;
 }
-
-// Magnitude bits of a fixed mass's high word, to be ORed over a row: a mass
-// of at least 2^-2 of the largest has one of the bits 26 .. 28.
-__device__ __forceinline__ unsigned int fix_size(long long v) {
-  const int h = (int)(v >> 32);
-  return (unsigned int)(h ^ (h >> 31));
-}
-__device__ __forceinline__ bool fix_large(unsigned int size) { return (size >> 26) != 0; }
 
 // P (or 2 P; in [2^-30, 2]) as a 31-bit integer and a right shift: P = p 2^-29
 // after the shift.
@@ -83,6 +84,16 @@ struct FixAcc {
     asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
         : "+r"(a0), "+r"(a1), "+r"(a2)
         : "r"(y0), "r"(y1), "r"(y2));
+  }
+  // Whether the sum is kept: the new mass it gives, M' = mass + sum / 2^halvings,
+  // outweighs the error of a row with (marked) or without marked masses.  In
+  // units of 8 u, by integers: two binary64 instructions per chunk and species
+  // made the dense step 1.4 % slower.
+  __device__ __forceinline__ bool keeps(long long mass, int halvings, bool marked) const {
+    const long long next =
+        (mass >> 3) + ((long long)((unsigned long long)a2 << 32 | a1) >> halvings);
+    return ((next ^ (next >> 63)) >> (marked ? 50 : 40)) != 0 ||
+           (!marked && (mass | a0 | a1 | a2) == 0);
   }
   // The sum in binary64 (rounded to nearest even), masses in units of
   // 2^(E - 1083).

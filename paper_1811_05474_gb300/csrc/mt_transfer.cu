@@ -506,10 +506,10 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
 // pair at the paper's density); here a pair is ~55 integer and binary32
 // instructions, issue-bound.  Each chunk's masses, and the rows' own, are
 // converted with the largest exponent among them, and a chunk's sum is rounded
-// to binary64 once.  A lane whose neighbours in the chunk hold a marked mass
-// and no large one (fix_large; looked for only where the chunk holds marked
-// masses, first in blocks of 32 slots wholly inside its range) sums the chunk
-// in binary64.  N = 10^6 at 200 per unit length: 4.09 -> 1.09 ms (step 4.47 -> 1.43 ms).
+// to binary64 once.  A lane whose sum does not outweigh its error (FixAcc::keeps; the
+// marks of the whole chunk count) sums the chunk again, in binary64 (where two
+// reactants meet across a front, 10^5 particles: a quarter of the pass).  N = 10^6
+// at 200 per unit length: 4.09 -> 1.10 ms (step 4.47 -> 1.43 ms).
 template <bool TR>
 __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   chained();
@@ -519,9 +519,8 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   __shared__ uint2 s_xr[kTileChunk];       // low word of the position, 1 / r
   __shared__ longlong2 s_ab[kTileChunk];   // fixed masses
   __shared__ long long s_lohi[2];
-  __shared__ int s_e[kWarps][2];                       // largest exponents
-  __shared__ unsigned int s_size[2][kTileChunk / 32];  // fix_size over blocks of 32 slots
-  __shared__ int s_mark[2];                            // the chunk holds marked masses
+  __shared__ int s_e[kWarps][2];  // largest exponents
+  __shared__ int s_mark[2];       // the chunk holds marked masses
   const long long b0 = (long long)blockIdx.x * kThreads;
   const long long b1 = min(b0 + (long long)kThreads, d.n);
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -541,7 +540,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   // (those of 2 P overflow for masses beyond half of binary64's range)
   const bool sym = d.norm != MT_NORM_ROW;
   const float p_scale = sym ? 0.5f : 1.0f;
-  const double half = sym ? 0.5 : 1.0;
   const unsigned long long Ab = valid ? MA[p] : 0, Bb = valid ? MB[p] : 0;
   const float ip = valid ? load_rinv<true>(d, p) : 0.0f;
   double dA = 0.0, dB = 0.0;
@@ -580,12 +578,8 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       const int i = threadIdx.x + k * kThreads;
       const long long fa = to_fix(va[k], EA), fb = to_fix(vb[k], EB);
       s_ab[i] = make_longlong2(fa, fb);
-      const unsigned int za = __reduce_or_sync(0xffffffffu, fix_size(fa));
-      const unsigned int zb = __reduce_or_sync(0xffffffffu, fix_size(fb));
       const bool ma = __any_sync(0xffffffffu, fa & 1), mb = __any_sync(0xffffffffu, fb & 1);
       if (lane == 0) {
-        s_size[0][i / 32] = za;
-        s_size[1][i / 32] = zb;
         if (ma) s_mark[0] = 1;
         if (mb) s_mark[1] = 1;
       }
@@ -597,15 +591,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
     const long long fa = to_fix(Ab, EA), fb = to_fix(Bb, EB);
     // this lane's slots of the chunk
     const int l0 = (int)(max(jl, c0) - c0), l1 = (int)(min(jr, c0 + nc) - c0);
-    auto small = [&](int h, long long own) {
-      if (!s_mark[h] && !(own & 1)) return false;
-      unsigned int z = fix_size(own);
-      for (int b = (l0 + 31) / 32; b < l1 / 32; ++b) z |= s_size[h][b];
-      for (int j = l0; j < l1 && !fix_large(z); ++j) z |= fix_size(h ? s_ab[j].y : s_ab[j].x);
-      return !fix_large(z);
-    };
-    const bool fixa = fix_covers(EA) && !small(0, fa);
-    const bool fixb = fix_covers(EB) && !small(1, fb);
     FixAcc qa, qb;
 #pragma unroll 2
     for (int j = j0; j < j1; ++j) {
@@ -618,8 +603,11 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       qb.add(ab.y - fb, P);
     }
     if (l0 < l1) {
-      double ca = half * qa.value(EA), cb = half * qb.value(EB);
-      // units: 2^(E - 1083) of the masses, 2^-29 of 2 P
+      // (halved in the exponent, which is far from binary64's ends)
+      double ca = qa.value(EA - sym), cb = qb.value(EB - sym);
+      const int halvings = sym ? 2 : 1;
+      const bool fixa = fix_covers(EA) && qa.keeps(fa, halvings, s_mark[0] || (fa & 1));
+      const bool fixb = fix_covers(EB) && qb.keeps(fb, halvings, s_mark[1] || (fb & 1));
       if (!fixa || !fixb) {
         double ga = 0.0, gb = 0.0;
         const double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
