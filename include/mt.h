@@ -188,7 +188,8 @@ mt_status mt_batch_create(const mt_params* p, const mt_batch* b, void* workspace
                           size_t workspace_bytes, void* stream, mt_handle** out);
 
 /* Autotuner for the 1-d cell path: times `steps` steps (after `warmup`
- * steps, the first of which captures the CUDA graph) of each candidate cell
+ * steps, which capture the CUDA graph; both counts are rounded up to whole
+ * graphs where a long mt_run replays graphs of several steps) of each candidate cell
  * width (cell_shift c - 1 .. c + 2 around the resolver's choice c) and
  * segment size (seg_target: the resolver's choice, 256, 512, 1024) on the
  * inputs x, A, B (as mt_upload takes them) and returns in *best the resolved
@@ -340,7 +341,11 @@ mt_status mt_set_noise(mt_handle* h, const float* xi_device);
 mt_status mt_step(mt_handle* h);
 
 /* Enqueue nsteps time steps.  With the built-in generator the steps are
- * replayed from a CUDA graph captured on the first call. */
+ * replayed from CUDA graphs.  A graph is captured (0.1 to 1 ms of host work)
+ * by the first call that needs it: one of a single step or, in the 1-d
+ * one-kernel step of systems below a wave of segments whose binary64 masses
+ * are not observed, one of 12 steps for the multiples of 12 and one of a
+ * single step for the rest.  So a run is timed after one of the same length. */
 mt_status mt_run(mt_handle* h, int64_t nsteps);
 
 /* Wait for the handle's stream and report device-side errors. */

@@ -465,6 +465,16 @@ struct mt_handle {
   int ev_count = 0;  // kernels marked in the last profiled step
 };
 
+namespace mt {
+// Steps of the graphs that a long mt_run replays.  With observables of binary64
+// masses the one-step graphs are the faster form: they run a step's observables
+// beside the next step (N = 46773 MT_FP64: 44 us per step against 51 in a graph
+// of several steps).
+int graph_steps(const mt_handle* h) {
+  return h->D.fused && !h->dev.use_pred && !h->obs_defer ? kMultiSteps : 1;
+}
+}  // namespace mt
+
 namespace {
 
 bool capturable(cudaStream_t s) {
@@ -1117,10 +1127,7 @@ mt_status mt_run(mt_handle* h, int64_t nsteps) {
     return MT_OK;
   }
   int64_t left = nsteps;
-  // With observables of binary64 masses the one-step graphs are the faster
-  // form: they run a step's observables beside the next step (N = 46773
-  // MT_FP64: 44 us per step against 51 in a graph of several steps).
-  if (h->D.fused && !h->dev.use_pred && !h->obs_defer && left >= kMultiSteps) {
+  if (mt::graph_steps(h) == kMultiSteps && left >= kMultiSteps) {
     if (!h->multi) {
       const mt_status s = build_multi(h);
       if (s != MT_OK) return s;
