@@ -20,8 +20,28 @@
 // and a prefix count), and a full list is worked off 32 entries at a time with
 // the exact 64-bit test and the weight.  Row sums in binary32 add the list's
 // nonzero weights one by one in the order of j, the order (and the bits) of
-// a plain loop over j; binary64 sums and the flux sums use lane partials and
+// a plain loop over j (but for direct tiles); binary64 sums and the flux sums use lane partials and
 // a fixed shuffle tree.
+//
+// Where much of the matrix is nonzero (a dense system, particles piled at one
+// place, in whatever order they are numbered) a list costs more than the pairs:
+// a group of 32 candidates takes ~60 warp instructions and, in binary32 row
+// sums, 32 dependent additions.  With binary32 weights a CTA that met more than
+// a given share of its pairs in one tile therefore takes the next one directly
+// (ap_direct): a lane per row and share of the columns, every weight evaluated,
+// until a tile holds fewer again.  (Binary64 weights outweigh their list: 1.9
+// times as long directly with a quarter of all pairs in reach, 0.83 with all.)
+// The first tile of more than two is a short one, so that little is listed before the
+// first choice.  The shares are where the two forms take as long, at N = 2 10^4
+// and 5 10^4, one per unit length on a part of the domain:
+//   row sums            directly 0.86 ms and 2.9 ms; by lists 1.8 and 4.7 with
+//                       1/21 and 1/27 of the pairs in reach: 1/32
+//   DF32's exchange     2.1 and 7.9; 2.1 with 1/14, 7.9 with 1/11: 1/8
+//   MIXED's exchange    4.5 and 20.5; 4.6 with 1/4, 14.7 with 1/4: 1/4
+// N = 2 10^4, all in reach: 25.5 ms -> 6.5 ms (MIXED), 19.9 -> 3.2 (DF32); a thread
+// per row, which systems with more than 1/4 of the pairs in reach by their domain
+// took before: 10.5 and 4.0 ms, and N = 5000 on 50 units 2.35 and 1.01 ms -> 0.43
+// and 0.24.
 //
 // Measured, one step: N = 10^3 binary64 full matrix 3.0 ms -> 35 us, N = 10^5
 // binary32 weights 22.2 ms -> 2.6 ms (a thread per row and an exponential per
@@ -38,6 +58,12 @@ constexpr int kApTile = 2048;   // j-particles staged per tile
 constexpr int kApThreads = 128;
 constexpr int kApWarps = kApThreads / 32;
 constexpr int kApCap = 64;      // list entries per row
+constexpr int kApFirst = 256;   // j-particles in the first tile of more than two
+// The next tile is taken directly if more than 1 / kDense of the last one's
+// pairs had a weight (binary32 weights).
+constexpr int dense(int precision, bool exchange) {
+  return !exchange ? 32 : precision == MT_MIXED_DF32 ? 8 : 4;
+}
 
 struct ApGrid {
   int sh;         // coarse coordinate: X >> sh, below 2^24
@@ -60,6 +86,93 @@ struct ApRow {
   typename Mass<PR>::Acc da[EX ? R : 1], db[EX ? R : 1];
 };
 
+// One tile directly: columns [j0, j0 + nt) staged exactly, kApThreads at a time
+// (stage: 40 bytes each), lane l taking row l % R and every (32 / R)-th of them;
+// the lanes' sums join the row's at the end.  Every thread of the CTA calls it
+// (nr = 0: a warp without rows).  Returns the lane's number of nonzero weights.
+template <int PR, int DIM, int R, bool EX, bool PER>
+__device__ __forceinline__ int ap_direct(const Dev& d, const ApGrid& g, long long j0, int nt,
+                                         long long row0, int nr, unsigned char* stage,
+                                         ApRow<PR, R, EX>& s, const long long* X,
+                                         const unsigned long long* MA,
+                                         const unsigned long long* MB) {
+  using W = Weight<mixw(PR), DIM>;
+  using T = typename W::T;
+  using MS = Mass<PR>;
+  using MV = typename MS::V;
+  long long* sx = reinterpret_cast<long long*>(stage);
+  long long* sy = sx + kApThreads;
+  MV* sa = reinterpret_cast<MV*>(sy + kApThreads);
+  MV* sb = sa + kApThreads;
+  T* sr = reinterpret_cast<T*>(sb + kApThreads);
+  const int lane = threadIdx.x & 31, r = lane % R;
+  const bool mine = r < nr;
+  const long long p = row0 + r;
+  const long long x = mine ? X[p] : 0, y = mine && DIM == 2 ? X[d.n + p] : 0;
+  MV A{}, B{};
+  T ip = T(0);
+  if (EX && mine) {
+    A = MS::load(MA, p);
+    B = MS::load(MB, p);
+    ip = load_rinv<mixw(PR)>(d, p);
+  }
+  T sum = T(0);
+  typename MS::Acc a{}, b{};
+  int found = 0;
+  for (int c0 = 0; c0 < nt; c0 += kApThreads) {
+    const int nc = min(nt - c0, kApThreads);
+    __syncthreads();
+    if ((int)threadIdx.x < nc) {
+      const int i = threadIdx.x;
+      const long long j = j0 + c0 + i;
+      sx[i] = X[j];
+      if (DIM == 2) sy[i] = X[d.n + j];
+      if (EX) {
+        sa[i] = MS::load(MA, j);
+        sb[i] = MS::load(MB, j);
+        sr[i] = load_rinv<mixw(PR)>(d, j);
+      }
+    }
+    __syncthreads();
+    for (int i = lane / R; mine && i < nc; i += 32 / R) {
+      long long dx = sx[i] - x, dy = DIM == 2 ? sy[i] - y : 0;
+      if (PER) {
+        dx = min_image(dx, d.Lq[0]);
+        if (DIM == 2) dy = min_image(dy, d.Lq[1]);
+      }
+      if (g.cut && !in_range2(dx, dy, d.S)) continue;
+      const T w = W::eval(d, dx, dy);
+      if (w == T(0)) continue;
+      ++found;
+      if (!EX) {
+        sum += w;
+      } else if (j0 + c0 + i != p) {
+        const T P = normalised<T>(d.norm, w, ip, sr[i]);
+        MS::acc(a, P, MS::diff(sa[i], A));
+        MS::acc(b, P, MS::diff(sb[i], B));
+      }
+    }
+  }
+  __syncwarp();
+  if constexpr (EX) {
+#pragma unroll
+    for (int o = 16; o >= R; o >>= 1) {
+      a = acc_merge(a, acc_shfl_xor(a, o));
+      b = acc_merge(b, acc_shfl_xor(b, o));
+    }
+    if (lane < nr) {
+      s.da[lane] = acc_merge(s.da[lane], a);
+      s.db[lane] = acc_merge(s.db[lane], b);
+    }
+  } else {
+#pragma unroll
+    for (int o = 16; o >= R; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane < nr) s.r[lane] += sum;
+  }
+  __syncwarp();
+  return found;
+}
+
 // PER: periodic walls.  EX = false: row sums.  EX = true: exchange of A and B and the end of the
 // step (sp = 0), or of the extra species sp, sp + 1.
 template <int PR, int DIM, int R, bool EX, bool PER>
@@ -68,7 +181,9 @@ __global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_
   using T = typename W::T;
   using MS = Mass<PR>;
   using MV = typename MS::V;
-  __shared__ float s_cx[kApTile];
+  __shared__ __align__(16) float s_cx[kApTile];  // (ap_direct: its stage)
+  static_assert(kApTile * sizeof(float) >= kApThreads * 40, "ap_direct's stage");
+  __shared__ int s_found[2];  // pairs with a weight (candidates) in the last tile
   __shared__ float s_cy[DIM == 2 ? kApTile : 1];
   extern __shared__ __align__(16) unsigned char s_rows[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -169,16 +284,41 @@ __global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_
     __syncwarp();
     if (lane == r) mycnt = 0;
   };
-  for (long long j0 = 0; j0 < n; j0 += kApTile) {
+  // tiles of kApTile, the first of more than two shorter
+  int nt = mixw(PR) && n > 2 * kApTile ? kApFirst : (int)min((long long)kApTile, n);
+  const int cta_rows = (int)min((long long)(kApWarps * R),
+                                n - (long long)blockIdx.x * (kApWarps * R));
+  int found = 0, par = 0;  // this warp's pairs with a weight in the tile
+  bool direct = false;
+  if (threadIdx.x < 2) s_found[threadIdx.x] = 0;
+  for (long long j0 = 0; j0 < n;) {
+    if (mixw(PR) && j0 > 0) {
+      if (lane == 0 && found) atomicAdd(&s_found[par], found);
+      __syncthreads();
+      direct = s_found[par] > cta_rows * nt / dense(PR, EX);
+      par ^= 1;
+      found = 0;
+    }
+    if (j0 > 0) nt = (int)min((long long)kApTile, n - j0);
     __syncthreads();
+    if constexpr (mixw(PR)) {
+      if (threadIdx.x == 0) s_found[par ^ 1] = 0;
+      if (direct) {
+        found = __reduce_add_sync(0xffffffffu, ap_direct<PR, DIM, R, EX, PER>(
+            d, g, j0, nt, row0, nr, reinterpret_cast<unsigned char*>(s_cx), s, X, MA, MB));
+        j0 += nt;
+        continue;
+      }
+    }
     for (int i = threadIdx.x; i < kApTile; i += kApThreads) {
       const long long j = j0 + i;
       s_cx[i] = j < n ? coarse(0, j) : 0.0f;
       if (DIM == 2) s_cy[i] = j < n ? coarse(1, j) : 0.0f;
     }
     __syncthreads();
-    const int nt = (int)min((long long)kApTile, n - j0);
+    j0 += nt;
     if (nr == 0) continue;  // a warp without rows only stages
+    const long long jt = j0 - nt;
 #pragma unroll 2
     for (int i0 = 0; i0 < nt; i0 += 32) {
       const float cx = s_cx[i0 + lane], cy = DIM == 2 ? s_cy[i0 + lane] : 0.0f;
@@ -191,8 +331,9 @@ __global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_
           flush(0);
           cnt1 = 0;
         }
-        if (c) s.list[0][cnt1 + __popc(m & ((1u << lane) - 1u))] = (int)(j0 + i0 + lane);
+        if (c) s.list[0][cnt1 + __popc(m & ((1u << lane) - 1u))] = (int)(jt + i0 + lane);
         cnt1 += __popc(m);
+        if (mixw(PR)) found += __popc(m);
         continue;
       }
       float m = 3.0e38f;
@@ -215,8 +356,9 @@ __global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_
           flush(r);
           at = 0;
         }
-        if (c) s.list[r][at + __popc(m & ((1u << lane) - 1u))] = (int)(j0 + i0 + lane);
+        if (c) s.list[r][at + __popc(m & ((1u << lane) - 1u))] = (int)(jt + i0 + lane);
         if (lane == r) mycnt = at + __popc(m);
+        if (mixw(PR)) found += __popc(m);
       }
     }
   }
@@ -267,31 +409,22 @@ static cudaError_t launch_pr(const Dev& d, const ApGrid& g, int sp, cudaStream_t
   return d.dim == 1 ? launch_rows<PR, 1, EX>(d, g, sp, s) : launch_rows<PR, 2, EX>(d, g, sp, s);
 }
 
-// The scan's parameters; false where the list does not pay: binary32 weights
-// (whose row sums add the list's entries one by one) with more than a quarter
-// of all pairs in reach of one another, e.g. the paper's 50-unit domain, where
-// a thread per row is faster (binary64 weights always take the list: their
-// arithmetic outweighs it).
-static bool ap_grid(const Dev& d, bool cut, int precision, ApGrid* g) {
+// The scan's parameters.
+static ApGrid ap_grid(const Dev& d, bool cut, int precision) {
+  ApGrid g;
   const double a = precision == MT_FP64 ? d.inv8 * d.scale * d.scale : (double)d.inv8f;
   double Z = a > 0.0 ? sqrt((precision == MT_FP64 ? 746.0 : 110.0) / a) * (1.0 + 1e-6) + 2.0 : 9e18;
   if (cut && (double)d.S < Z) Z = (double)d.S;
-  double reach = 1.0;
-  long long Lmax = 0;
-  for (int k = 0; k < d.dim; ++k) {
-    const double f = 2.0 * Z / ((double)d.Lq[k] + 1.0);
-    reach *= f < 1.0 ? f : 1.0;
-    Lmax = d.Lq[k] > Lmax ? d.Lq[k] : Lmax;
-  }
-  if (precision != MT_FP64 && reach > 0.25) return false;
-  g->cut = cut ? 1 : 0;
-  g->sh = 0;
-  while ((Lmax >> g->sh) >= (1LL << 24)) ++g->sh;
+  long long Lmax = d.Lq[0];
+  if (d.dim == 2 && d.Lq[1] > Lmax) Lmax = d.Lq[1];
+  g.cut = cut ? 1 : 0;
+  g.sh = 0;
+  while ((Lmax >> g.sh) >= (1LL << 24)) ++g.sh;
   // rounding of both coordinates, and of the coarse half length and of its
   // differences (half a unit each): two more units
-  g->zc = (float)(std::floor(std::ldexp(Z < (double)Lmax ? Z : (double)Lmax, -g->sh)) + 3.0);
-  for (int k = 0; k < 2; ++k) g->half[k] = (float)std::ldexp((double)d.Lq[k], -g->sh - 1);
-  return true;
+  g.zc = (float)(std::floor(std::ldexp(Z < (double)Lmax ? Z : (double)Lmax, -g.sh)) + 3.0);
+  for (int k = 0; k < 2; ++k) g.half[k] = (float)std::ldexp((double)d.Lq[k], -g.sh - 1);
+  return g;
 }
 
 template <int PR>
@@ -306,14 +439,11 @@ static cudaError_t allpairs_t(const Dev& d, const ApGrid& g, cudaStream_t s, Mar
   return e == cudaSuccess ? launch_pr<PR, true>(d, g, 0, s) : e;
 }
 
-bool launch_allpairs(const Dev& d, bool cut, int precision, cudaStream_t s, Marker& mk,
-                     cudaError_t* e) {
-  ApGrid g;
-  if (!ap_grid(d, cut, precision, &g)) return false;
-  *e = precision == MT_MIXED        ? allpairs_t<MT_MIXED>(d, g, s, mk)
-       : precision == MT_MIXED_DF32 ? allpairs_t<MT_MIXED_DF32>(d, g, s, mk)
-                                    : allpairs_t<MT_FP64>(d, g, s, mk);
-  return true;
+cudaError_t launch_allpairs(const Dev& d, bool cut, int precision, cudaStream_t s, Marker& mk) {
+  const ApGrid g = ap_grid(d, cut, precision);
+  if (precision == MT_MIXED) return allpairs_t<MT_MIXED>(d, g, s, mk);
+  if (precision == MT_MIXED_DF32) return allpairs_t<MT_MIXED_DF32>(d, g, s, mk);
+  return allpairs_t<MT_FP64>(d, g, s, mk);
 }
 
 }  // namespace mt

@@ -14,7 +14,6 @@ constexpr int kScanItems = 16;         // cell counts per thread in the scan
 constexpr int kScanTile = kThreads * kScanItems;
 constexpr int kSmallCell = 32;         // cells up to this size sort in one thread
 constexpr int kBigSortCap = 2048;      // cells up to this size sort in shared memory
-constexpr int kBruteTile = 256;        // j-particles staged per tile, brute force
 constexpr long long kSpinLimit = 1LL << 22;  // bounded waits (scan look-back)
 constexpr int kObsChunk = 4096;  // slots per observables chunk (16 per thread)
 constexpr double kTileMinNeighbours = 32.0;  // mean neighbours a side for tiled passes
@@ -534,10 +533,8 @@ cudaError_t launch_move(const Dev& d, bool move, bool hist, cudaStream_t s);
 cudaError_t launch_sort(const Dev& d, cudaStream_t s, Marker& mk);  // scan, scatter, cell sort
 cudaError_t launch_permute(const Dev& d, cudaStream_t s);  // gather id/masses after sort, flip
 cudaError_t launch_transfer(const Dev& d, int search, int precision, cudaStream_t s, Marker& mk);
-// brute force and full matrix by the scan with candidate lists (mt_allpairs.cu);
-// false, with nothing enqueued, where a thread per row is the faster form
-bool launch_allpairs(const Dev& d, bool cut, int precision, cudaStream_t s, Marker& mk,
-                     cudaError_t* e);
+// brute force (cut) and full matrix (mt_allpairs.cu)
+cudaError_t launch_allpairs(const Dev& d, bool cut, int precision, cudaStream_t s, Marker& mk);
 // after a step: the observables row of every realisation
 cudaError_t launch_obs(const Dev& d, int precision, cudaStream_t s);
 // the fused path's graph: snapshot the state's buffer and step, then (beside

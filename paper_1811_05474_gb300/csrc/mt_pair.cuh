@@ -454,6 +454,12 @@ __device__ __forceinline__ kahan acc_merge(kahan a, kahan b) {
   const df e = two_sum(a.s, b.s);
   return {e.hi, __fadd_rn(__fadd_rn(a.c, b.c), e.lo)};
 }
+__device__ __forceinline__ double acc_shfl_xor(double v, int o) {
+  return __shfl_xor_sync(0xffffffffu, v, o);
+}
+__device__ __forceinline__ kahan acc_shfl_xor(kahan v, int o) {
+  return {__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o)};
+}
 __device__ __forceinline__ kahan acc_warp_sum(kahan v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

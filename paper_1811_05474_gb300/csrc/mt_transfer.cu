@@ -10,8 +10,8 @@
 //         <= Smax; each thread walks left and right until it leaves range.
 //   cell2 (2-d cell list) candidates are the 3 x 3 block of cells around the
 //         particle's cell (cell width > Smax), contiguous per row.
-//   brute all n particles in shared-memory tiles, with (BRUTE) or without
-//         (FULL, the paper's full-matrix reference) the cutoff test.
+//   all pairs, with (BRUTE) or without (FULL, the paper's full-matrix
+//         reference) the cutoff: mt_allpairs.cu.
 // Precision: mixw(PR) = false is IEEE binary64 throughout; mixw(PR) = true forms
 // weights and normalised weights in binary32 and updates the double-binary32
 // masses with compensated additions.
@@ -304,11 +304,6 @@ __global__ void __launch_bounds__(kThreads) k_exchange_walk(Dev d) {
     MS::store(Mn, off(2 * k) + p, m[2 * k]);
     if (2 * k + 1 < d.nspec) MS::store(Mn, off(2 * k + 1) + p, m[2 * k + 1]);
   }
-}
-
-// |dx| <= S in one unsigned comparison (1-d)
-__device__ __forceinline__ bool within1(long long dx, long long S) {
-  return (unsigned long long)(dx + S) <= (unsigned long long)(2 * S);
 }
 
 // ======================================================= 1-d dense tiles ==
@@ -990,119 +985,6 @@ __global__ void k_finish(Dev d, int flip_x, int flip_m) {
   c->mcur ^= flip_m;
 }
 
-// ============================================================ brute force ==
-// All pairs, j-particles staged through shared memory in tiles.  Particles
-// keep their caller order (no sort); masses ping-pong between buffers.
-
-template <int PR, bool CUT, int DIM>
-__global__ void __launch_bounds__(kThreads) k_rowsum_brute(Dev d) {
-  using W = Weight<mixw(PR), DIM>;
-  using T = typename W::T;
-  __shared__ long long s_x[kBruteTile];
-  __shared__ long long s_y[DIM == 2 ? kBruteTile : 1];
-  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = p < d.n;
-  const long long* X = d.X[d.ctrl->xcur];
-  const long long x = valid ? X[p] : 0;
-  const long long y = (valid && DIM == 2) ? X[d.n + p] : 0;
-  T r = T(0);
-  for (long long j0 = 0; j0 < d.n; j0 += kBruteTile) {
-    const long long j = j0 + threadIdx.x;
-    if (j < d.n) {
-      s_x[threadIdx.x] = X[j];
-      if (DIM == 2) s_y[threadIdx.x] = X[d.n + j];
-    }
-    __syncthreads();
-    const int jn = (int)min((long long)kBruteTile, d.n - j0);
-    if (valid) {
-      for (int jj = 0; jj < jn; ++jj) {
-        long long dx = s_x[jj] - x;
-        long long dy = DIM == 2 ? s_y[jj] - y : 0;
-        if (d.periodic) {
-          dx = min_image(dx, d.Lq[0]);
-          if (DIM == 2) dy = min_image(dy, d.Lq[1]);
-        }
-        if (CUT) {
-          if (DIM == 1 ? !within1(dx, d.S) : !in_range2(dx, dy, d.S)) continue;
-        }
-        r += W::eval(d, dx, dy);
-      }
-    }
-    __syncthreads();
-  }
-  if (valid) store_rinv<mixw(PR)>(d, p, r);
-}
-
-template <int PR, bool CUT, int DIM, bool TR>
-__global__ void __launch_bounds__(kThreads) k_exchange_brute(Dev d, int sp) {
-  using W = Weight<mixw(PR), DIM>;
-  using T = typename W::T;
-  using MS = Mass<PR>;
-  using MV = typename MS::V;
-  __shared__ long long s_x[kBruteTile];
-  __shared__ long long s_y[DIM == 2 ? kBruteTile : 1];
-  __shared__ T s_ri[kBruteTile];
-  __shared__ MV s_a[kBruteTile];
-  __shared__ MV s_b[kBruteTile];
-  const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = p < d.n;
-  const int mc = d.ctrl->mcur;
-  const long long* X = d.X[d.ctrl->xcur];
-  const SpeciesPair sq = species_pair<TR>(d, sp);
-  const unsigned long long* MA = d.M[mc] + sq.oa;
-  const unsigned long long* MB = d.M[mc] + sq.ob;
-  const long long x = valid ? X[p] : 0;
-  const long long y = (valid && DIM == 2) ? X[d.n + p] : 0;
-  MV A{}, B{};
-  T ip = T(0);
-  if (valid) {
-    A = MS::load(MA, p);
-    B = MS::load(MB, p);
-    ip = load_rinv<mixw(PR)>(d, p);
-  }
-  typename MS::Acc dA{}, dB{};
-  for (long long j0 = 0; j0 < d.n; j0 += kBruteTile) {
-    const long long j = j0 + threadIdx.x;
-    if (j < d.n) {
-      s_x[threadIdx.x] = X[j];
-      if (DIM == 2) s_y[threadIdx.x] = X[d.n + j];
-      s_ri[threadIdx.x] = load_rinv<mixw(PR)>(d, j);
-      s_a[threadIdx.x] = MS::load(MA, j);
-      s_b[threadIdx.x] = MS::load(MB, j);
-    }
-    __syncthreads();
-    const int jn = (int)min((long long)kBruteTile, d.n - j0);
-    if (valid) {
-      for (int jj = 0; jj < jn; ++jj) {
-        if (j0 + jj == p) continue;
-        long long dx = s_x[jj] - x;
-        long long dy = DIM == 2 ? s_y[jj] - y : 0;
-        if (d.periodic) {
-          dx = min_image(dx, d.Lq[0]);
-          if (DIM == 2) dy = min_image(dy, d.Lq[1]);
-        }
-        if (CUT) {
-          if (DIM == 1 ? !within1(dx, d.S) : !in_range2(dx, dy, d.S)) continue;
-        }
-        const T w = W::eval(d, dx, dy);
-        // a weight that underflowed to zero adds exact zeros: skip the
-        // flux arithmetic (the full matrix still evaluates every weight)
-        if (w == T(0)) continue;
-        const T P = normalised<T>(d.norm, w, ip, s_ri[jj]);
-        MS::acc(dA, P, MS::diff(s_a[jj], A));
-        MS::acc(dB, P, MS::diff(s_b[jj], B));
-      }
-    }
-    __syncthreads();
-  }
-  if (valid) {
-    MS::update(A, B, dA, dB, TR ? 0 : d.react);
-    MS::store(d.M[mc ^ 1] + sq.oa, p, A);
-    if (sq.store_b) MS::store(d.M[mc ^ 1] + sq.ob, p, B);
-  }
-  if (!TR) finish_step(d, 0, 1);
-}
-
 // Species 2 and up into the sorted slots (the row-sum pass moved A and B).
 __global__ void __launch_bounds__(kThreads) k_gather_species(Dev d) {
   const long long p = (long long)blockIdx.x * kThreads + threadIdx.x;
@@ -1123,22 +1005,6 @@ static void cell2_passes(const Dev& d, unsigned int g, cudaStream_t s, Marker& m
   mk("exchange_cell2", s);
   launch_chained(k_exchange_cell2<PR, false, PER>, g, kThreads, 0, s, d, 0);
   launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
-}
-
-template <int PR, bool TR>
-static void launch_exchange_brute(const Dev& d, bool cut, unsigned int g, cudaStream_t s,
-                                  int sp) {
-  if (cut) {
-    if (d.dim == 1)
-      k_exchange_brute<PR, true, 1, TR><<<g, kThreads, 0, s>>>(d, sp);
-    else
-      k_exchange_brute<PR, true, 2, TR><<<g, kThreads, 0, s>>>(d, sp);
-  } else {
-    if (d.dim == 1)
-      k_exchange_brute<PR, false, 1, TR><<<g, kThreads, 0, s>>>(d, sp);
-    else
-      k_exchange_brute<PR, false, 2, TR><<<g, kThreads, 0, s>>>(d, sp);
-  }
 }
 
 // The extra species' passes (pairs 2-3, 4-5, ...) run between the row sums
@@ -1194,42 +1060,11 @@ static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
   }
 }
 
-// All pairs, a thread per row: binary32 weights in systems where much of the
-// matrix is nonzero (launch_allpairs takes the others).
-template <int PR>
-static void brute_t(const Dev& d, bool cut, cudaStream_t s, Marker& mk) {
-  const unsigned int g = (unsigned int)((d.n + kThreads - 1) / kThreads);
-  mk(cut ? "rowsum_brute" : "rowsum_full", s);
-  if (cut) {
-    if (d.dim == 1)
-      k_rowsum_brute<PR, true, 1><<<g, kThreads, 0, s>>>(d);
-    else
-      k_rowsum_brute<PR, true, 2><<<g, kThreads, 0, s>>>(d);
-  } else {
-    if (d.dim == 1)
-      k_rowsum_brute<PR, false, 1><<<g, kThreads, 0, s>>>(d);
-    else
-      k_rowsum_brute<PR, false, 2><<<g, kThreads, 0, s>>>(d);
-  }
-  for (int sp = 2; sp < d.nspec; sp += 2) {
-    mk(cut ? "exchange_brute_species" : "exchange_full_species", s);
-    launch_exchange_brute<PR, true>(d, cut, g, s, sp);
-  }
-  mk(cut ? "exchange_brute" : "exchange_full", s);
-  launch_exchange_brute<PR, false>(d, cut, g, s, 0);
-}
-
 cudaError_t launch_transfer(const Dev& d, int search, int precision, cudaStream_t s,
                             Marker& mk) {
-  if (search != MT_SEARCH_CELL) {
-    const bool cut = search == MT_SEARCH_BRUTE;
-    cudaError_t e = cudaSuccess;
-    if (launch_allpairs(d, cut, precision, s, mk, &e)) return e;
-    if (precision == MT_MIXED)
-      brute_t<MT_MIXED>(d, cut, s, mk);
-    else
-      brute_t<MT_MIXED_DF32>(d, cut, s, mk);
-  } else if (precision == MT_MIXED) {
+  if (search != MT_SEARCH_CELL)
+    return launch_allpairs(d, search == MT_SEARCH_BRUTE, precision, s, mk);
+  if (precision == MT_MIXED) {
     transfer_t<MT_MIXED>(d, s, mk);
   } else if (precision == MT_MIXED_DF32) {
     transfer_t<MT_MIXED_DF32>(d, s, mk);
