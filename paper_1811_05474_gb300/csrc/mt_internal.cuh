@@ -482,13 +482,22 @@ __device__ __forceinline__ void f64_store(unsigned long long* M, long long i, do
 // way calls chained() before it touches memory.  (Without the attribute both
 // calls do nothing.)  Only grids of up to kChainedCtas: the CTAs of a larger
 // kernel's successor would hold its multiprocessors' room while they wait
-// (mixed requests on several streams: 2.6 % slower).
+// (mixed requests on several streams: 2.6 % slower).  A chained kernel's CTAs
+// are placed where the kernel before it leaves room first, not evenly: a few
+// multiprocessors take several while others stay empty, which a kernel of a few
+// microseconds does not show and one whose CTAs run long pays for.  So the dense
+// tiles' passes are never chained (chained behind the sort's kernels, 136 per unit
+// length: N = 30000 MT_FP64 513 -> 1171 us per step, N = 40208 MT_MIXED_DF32
+// 133 -> 216; not chained, MT_MIXED loses 2 of 109 us), and the 2-d passes up to
+// kChainedCells (one per unit of area: N = 60000 MT_FP64 103 -> 126 us chained,
+// MT_MIXED 66 -> 73; N = 52000 1 to 2 % faster).
 constexpr unsigned int kChainedCtas = 304;
+constexpr unsigned int kChainedCells = 228;
 __device__ __forceinline__ void chained() {
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
 }
-template <class... P, class... A>
+template <unsigned int MOST = kChainedCtas, class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), unsigned int grid, unsigned int block, size_t smem,
                            cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
@@ -500,7 +509,7 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned int grid, unsigned int
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = grid <= kChainedCtas ? 1 : 0;
+  cfg.numAttrs = grid <= MOST ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 

@@ -633,11 +633,11 @@ template <int PR, bool TR>
 static void launch_exchange_tile(const Dev& d, unsigned int g, cudaStream_t s, int sp) {
   if constexpr (PR == MT_MIXED) {
     if (d.fix) {
-      launch_chained(k_exchange_tile_fix<TR>, g, kThreads, 0, s, d, sp);
+      k_exchange_tile_fix<TR><<<g, kThreads, 0, s>>>(d, sp);
       return;
     }
   }
-  launch_chained(k_exchange_tile<PR, TR>, g, kThreads, 0, s, d, sp);
+  k_exchange_tile<PR, TR><<<g, kThreads, 0, s>>>(d, sp);
 }
 
 // ================================================== 1-d SPaM (stored P) ==
@@ -997,13 +997,13 @@ __global__ void __launch_bounds__(kThreads) k_gather_species(Dev d) {
 template <int PR, bool PER>
 static void cell2_passes(const Dev& d, unsigned int g, cudaStream_t s, Marker& mk) {
   mk("rowsum_cell2", s);
-  launch_chained(k_rowsum_cell2<PR, PER>, g, kThreads, 0, s, d);
+  launch_chained<kChainedCells>(k_rowsum_cell2<PR, PER>, g, kThreads, 0, s, d);
   for (int sp = 2; sp < d.nspec; sp += 2) {
     mk("exchange_cell2_species", s);
-    launch_chained(k_exchange_cell2<PR, true, PER>, g, kThreads, 0, s, d, sp);
+    launch_chained<kChainedCells>(k_exchange_cell2<PR, true, PER>, g, kThreads, 0, s, d, sp);
   }
   mk("exchange_cell2", s);
-  launch_chained(k_exchange_cell2<PR, false, PER>, g, kThreads, 0, s, d, 0);
+  launch_chained<kChainedCells>(k_exchange_cell2<PR, false, PER>, g, kThreads, 0, s, d, 0);
   launch_chained(k_finish, 1, 1, 0, s, d, 1, 0);
 }
 
@@ -1029,7 +1029,7 @@ static void transfer_t(const Dev& d, cudaStream_t s, Marker& mk) {
     k_band_exchange<PR, false><<<g, kThreads, 0, s>>>(d, 0);
   } else if (d.dim == 1 && d.tile) {
     mk("rowsum_tile", s);
-    launch_chained(k_rowsum_tile<PR>, g, kThreads, 0, s, d);
+    k_rowsum_tile<PR><<<g, kThreads, 0, s>>>(d);
     if (d.nspec > 2) {
       mk("gather_species", s);
       k_gather_species<<<g, kThreads, 0, s>>>(d);
