@@ -817,19 +817,29 @@ constexpr int kNone = -1, kMany = -2;
 // cell (reflecting walls), or the wrapped cell spans (PER, minimum-image
 // separations).  (The lanes of a warp meet themselves in different
 // iterations: with p among the pairs, nearly every iteration evaluated a
-// weight.)
-template <bool PER, class F, class G>
+// weight.)  AHEAD: a candidate's coordinates are loaded while the one before it
+// is tested, since a warp with many candidates (a pile) waits for them: 10^4
+// particles, most in a few cells, MT_MIXED 1057 -> 873 us per step (with the three
+// runs' loops before: 931), and 30000 at one per unit of area 58 -> 54;
+// MT_MIXED_DF32's exchange, which has no registers left for it, does without (10^6
+// at one per unit of area: 293 against 282 us).
+template <bool PER, bool AHEAD, class F, class G>
 __device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, int p, long long x,
                                             long long y, F&& f, G&& self) {
   if (PER) {
     cells2_visit(d, x, y, [&](int q0, int q1) {
+      long long xn = q0 < q1 ? Xs[q0] : 0, yn = q0 < q1 ? Xs[d.n + q0] : 0;
       for (int q = q0; q < q1; ++q) {
+        const long long dx = min_image(xn - x, d.Lq[0]);
+        const long long dy = min_image(yn - y, d.Lq[1]);
+        if (q + 1 < q1) {
+          xn = Xs[q + 1];
+          yn = Xs[d.n + q + 1];
+        }
         if (q == p) {
           self();
           continue;
         }
-        const long long dx = min_image(Xs[q] - x, d.Lq[0]);
-        const long long dy = min_image(Xs[d.n + q] - y, d.Lq[1]);
         if (in_range2(dx, dy, d.S)) f(q, dx, dy);
       }
     });
@@ -854,15 +864,28 @@ __device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, i
   const unsigned long long x0 = (unsigned long long)(x - d.S), y0 = (unsigned long long)(y - d.S);
   const unsigned int S2 = 2u * (unsigned int)d.S;
   const long long* Ys = Xs + d.n;
+  auto slot = [&](int t) { return t + (t < n0 ? a[0] : t < n1 ? o1 : o2); };
+  int next = n2 > 0 ? slot(0) : 0;
+  long long xn = n2 > 0 ? Xs[next] : 0, yn = n2 > 0 ? Ys[next] : 0;
 #pragma unroll 2
   for (int t = 0; t < n2; ++t) {
-    const int q = t + (t < n0 ? a[0] : t < n1 ? o1 : o2);
+    if (!AHEAD) {
+      next = slot(t);
+      xn = Xs[next];
+      yn = Ys[next];
+    }
+    const int q = next;
+    const unsigned long long ux = (unsigned long long)xn - x0;
+    const unsigned long long uy = (unsigned long long)yn - y0;
+    if (AHEAD && t + 1 < n2) {
+      next = slot(t + 1);
+      xn = Xs[next];
+      yn = Ys[next];
+    }
     if (q == p) {
       self();
       continue;
     }
-    const unsigned long long ux = (unsigned long long)Xs[q] - x0;
-    const unsigned long long uy = (unsigned long long)Ys[q] - y0;
     if ((unsigned int)(ux >> 32) | (unsigned int)(uy >> 32)) continue;
     if ((unsigned int)ux > S2 || (unsigned int)uy > S2) continue;
     const int dx = (int)((unsigned int)ux - (unsigned int)d.S);
@@ -890,7 +913,7 @@ __global__ void __launch_bounds__(kThreads) k_rowsum_cell2(Dev d) {
     const long long* Xs = d.X[xc ^ 1];
     T r = T(0);
     int found = 0;
-    cell2_visit<PER>(
+    cell2_visit<PER, true>(
         d, Xs, (int)p, Xs[p], Xs[d.n + p],
         [&](int q, long long dx, long long dy) {
           r += W::near2(d, dx, dy, s_tab);
@@ -968,7 +991,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
     }
     pair(nb, dx, dy);
   } else {
-    cell2_visit<PER>(d, Xs, (int)p, x, y, pair, [] {});
+    cell2_visit<PER, PR != MT_MIXED_DF32>(d, Xs, (int)p, x, y, pair, [] {});
   }
   MS::update(A, B, dA, dB, TR ? 0 : d.react);
   store(p, A, B);
