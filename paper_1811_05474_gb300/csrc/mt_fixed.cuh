@@ -60,6 +60,11 @@ __device__ __forceinline__ long long to_fix(unsigned long long bits, int E) {
   return (long long)bits < 0 ? -(long long)v : (long long)v;
 }
 
+// 1: marked, 2: negative.
+__device__ __forceinline__ int fix_flags(long long v) {
+  return (int)(v & 1) | (v < 0 ? 2 : 0);
+}
+
 // P (or 2 P; in [2^-30, 2]) as a 31-bit integer and a right shift: P = p 2^-29
 // after the shift.
 struct FixP {
@@ -86,14 +91,16 @@ struct FixAcc {
         : "r"(y0), "r"(y1), "r"(y2));
   }
   // Whether the sum is kept: the new mass it gives, M' = mass + sum / 2^halvings,
-  // outweighs the error of a row with (marked) or without marked masses.  In
-  // units of 8 u, by integers: two binary64 instructions per chunk and species
-  // made the dense step 1.4 % slower.
-  __device__ __forceinline__ bool keeps(long long mass, int halvings, bool marked) const {
+  // outweighs the error of a row with (flags & 1) or without marked masses; or
+  // both are zero, which without marked or negative masses, or (one: a P times
+  // u is at least one unit of the sum) without negative ones, says that every
+  // mass of the row is.  In units of 8 u, by integers: two binary64
+  // instructions per chunk and species made the dense step 1.4 % slower.
+  __device__ __forceinline__ bool keeps(long long mass, int halvings, int flags, bool one) const {
     const long long next =
         (mass >> 3) + ((long long)((unsigned long long)a2 << 32 | a1) >> halvings);
-    return ((next ^ (next >> 63)) >> (marked ? 50 : 40)) != 0 ||
-           (!marked && (mass | a0 | a1 | a2) == 0);
+    if (((next ^ (next >> 63)) >> (flags & 1 ? 50 : 40)) != 0) return true;
+    return (mass | a0 | a1 | a2) == 0 && (flags == 0 || (flags == 1 && one));
   }
   // The sum in binary64 (rounded to nearest even), masses in units of
   // 2^(E - 1083).

@@ -502,9 +502,12 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
 // instructions, issue-bound.  Each chunk's masses, and the rows' own, are
 // converted with the largest exponent among them, and a chunk's sum is rounded
 // to binary64 once.  A lane whose sum does not outweigh its error (FixAcc::keeps; the
-// marks of the whole chunk count) sums the chunk again, in binary64 (where two
-// reactants meet across a front, 10^5 particles: a quarter of the pass).  N = 10^6
-// at 200 per unit length: 4.09 -> 1.10 ms (step 4.47 -> 1.43 ms).
+// marks of the whole chunk count) sums the chunk again, in binary64, which holds
+// the binary64 pipe of the multiprocessor a front lies on: a species at a time,
+// since in the tail of one the other is large (27 realisations of 5000, two
+// segregated components, eighth step: 309 us with both, 196 so; unrolled four
+// times 188, but 0.6 % more for the systems that have no such row).  N = 10^6 at
+// 200 per unit length: 4.09 -> 1.10 ms (step 4.47 -> 1.43 ms).
 template <bool TR>
 __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   chained();
@@ -515,7 +518,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
   __shared__ longlong2 s_ab[kTileChunk];   // fixed masses
   __shared__ long long s_lohi[2];
   __shared__ int s_e[kWarps][2];  // largest exponents
-  __shared__ int s_mark[2];       // the chunk holds marked masses
+  __shared__ int s_mark[2];       // fix_flags of the chunk's masses
   const long long b0 = (long long)blockIdx.x * kThreads;
   const long long b1 = min(b0 + (long long)kThreads, d.n);
   const int xc = d.ctrl->xcur, mc = d.ctrl->mcur;
@@ -573,10 +576,11 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       const int i = threadIdx.x + k * kThreads;
       const long long fa = to_fix(va[k], EA), fb = to_fix(vb[k], EB);
       s_ab[i] = make_longlong2(fa, fb);
-      const bool ma = __any_sync(0xffffffffu, fa & 1), mb = __any_sync(0xffffffffu, fb & 1);
+      const int ma = __reduce_or_sync(0xffffffffu, fix_flags(fa));
+      const int mb = __reduce_or_sync(0xffffffffu, fix_flags(fb));
       if (lane == 0) {
-        if (ma) s_mark[0] = 1;
-        if (mb) s_mark[1] = 1;
+        if (ma) atomicOr(&s_mark[0], ma);
+        if (mb) atomicOr(&s_mark[1], mb);
       }
     }
     __syncthreads();
@@ -601,20 +605,22 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
       // (halved in the exponent, which is far from binary64's ends)
       double ca = qa.value(EA - sym), cb = qb.value(EB - sym);
       const int halvings = sym ? 2 : 1;
-      const bool fixa = fix_covers(EA) && qa.keeps(fa, halvings, s_mark[0] || (fa & 1));
-      const bool fixb = fix_covers(EB) && qb.keeps(fb, halvings, s_mark[1] || (fb & 1));
-      if (!fixa || !fixb) {
-        double ga = 0.0, gb = 0.0;
-        const double A = __longlong_as_double((long long)Ab), B = __longlong_as_double((long long)Bb);
+      const bool one = ip >= 0x1p-19f;
+      const bool fixa = fix_covers(EA) && qa.keeps(fa, halvings, s_mark[0] | fix_flags(fa), one);
+      const bool fixb = fix_covers(EB) && qb.keeps(fb, halvings, s_mark[1] | fix_flags(fb), one);
+      // (a species at a time: in a tail of one the other is large)
+      auto again = [&](const unsigned long long* M, double own) {
+        double sum = 0.0;
+#pragma unroll 1
         for (int j = l0; j < l1; ++j) {
           const float P = W::near(d, (int)(s_xr[j].x - x32), nullptr) *
                           (ip + __uint_as_float(s_xr[j].y)) * p_scale;
-          MS::acc(ga, P, MS::diff(MS::load(MA, c0 + j), A));
-          MS::acc(gb, P, MS::diff(MS::load(MB, c0 + j), B));
+          MS::acc(sum, P, MS::diff(MS::load(M, c0 + j), own));
         }
-        ca = fixa ? ca : ga;
-        cb = fixb ? cb : gb;
-      }
+        return sum;
+      };
+      if (!fixa) ca = again(MA, __longlong_as_double((long long)Ab));
+      if (!fixb) cb = again(MB, __longlong_as_double((long long)Bb));
       dA += ca;
       dB += cb;
     }
