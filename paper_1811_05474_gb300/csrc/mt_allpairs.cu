@@ -29,10 +29,10 @@
 // sums, 32 dependent additions.  With binary32 weights a CTA that met more than
 // a given share of its pairs in one tile therefore takes the next one directly
 // (ap_direct): a lane per row and share of the columns, every weight evaluated,
-// until a tile holds fewer again.  (Binary64 weights outweigh their list: 1.9
+// until a tile holds fewer again.  (Binary64 weights outweigh their list: 1.5
 // times as long directly with a quarter of all pairs in reach, 0.83 with all.)
-// The first tile of more than two is a short one, so that little is listed before the
-// first choice.  The shares are where the two forms take as long, at N = 2 10^4
+// The first tile of more than two is a short one, so that little is listed
+// before the first choice.  The shares are where the two forms take as long, at N = 2 10^4
 // and 5 10^4, one per unit length on a part of the domain:
 //   row sums            directly 0.86 ms and 2.9 ms; by lists 1.8 and 4.7 with
 //                       1/21 and 1/27 of the pairs in reach: 1/32
@@ -59,8 +59,8 @@ constexpr int kApThreads = 128;
 constexpr int kApWarps = kApThreads / 32;
 constexpr int kApCap = 64;      // list entries per row
 constexpr int kApFirst = 256;   // j-particles in the first tile of more than two
-// The next tile is taken directly if more than 1 / kDense of the last one's
-// pairs had a weight (binary32 weights).
+// The next tile is taken directly if more than this share of the last one's
+// pairs (its inverse) had a weight (binary32 weights).
 constexpr int dense(int precision, bool exchange) {
   return !exchange ? 32 : precision == MT_MIXED_DF32 ? 8 : 4;
 }
@@ -310,7 +310,8 @@ __global__ void __launch_bounds__(kApThreads, R < 16 ? 10 : DIM == 1 ? 8 : 6) k_
         continue;
       }
     }
-    for (int i = threadIdx.x; i < kApTile; i += kApThreads) {
+    // (the last group of 32 is filled up)
+    for (int i = threadIdx.x; i < ((nt + 31) & ~31); i += kApThreads) {
       const long long j = j0 + i;
       s_cx[i] = j < n ? coarse(0, j) : 0.0f;
       if (DIM == 2) s_cy[i] = j < n ? coarse(1, j) : 0.0f;
