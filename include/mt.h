@@ -321,7 +321,8 @@ mt_status mt_read_species(mt_handle* h, int32_t s, double* M, int32_t mem);
  * handle then continues exactly as the saved one would have (the
  * counter-based random walk is keyed by the step counter, which the state
  * holds), bit for bit on the same device kind.  The handle's own noise
- * source (mt_set_noise) replaces the saved one.  Errors: MT_ERR_STATE
+ * source (mt_set_noise) replaces the saved one.  Files of both format
+ * versions load (1 held two workspace regions more).  Errors: MT_ERR_STATE
  * (mt_save before mt_upload); MT_ERR_INVALID (unreadable or foreign file, or
  * a handle with other resolved parameters or realisations; the device state
  * is then unchanged). */

@@ -65,7 +65,7 @@ struct Derived {
   std::vector<int> ochunk;  // first slot of each observables chunk (+ n)
   std::vector<int> ochr;    // realisation of each chunk
   // workspace offsets
-  size_t o_ctrl, o_X[2], o_id[2], o_M[2], o_src, o_rinv, o_count, o_start, o_cursor,
+  size_t o_ctrl, o_X[2], o_id[2], o_M[2], o_src, o_rinv, o_count, o_start,
       o_status, o_big, o_obs, o_fstart[2], o_cb[2], o_ovlist, o_pred[2], o_rt, o_sslot,
       o_sreal, o_ochunk, o_opart, o_ochr, o_ocnt, o_cnt, o_band, total;
   long long band = 0;  // SPaM band entries per particle (0: off)
@@ -391,16 +391,12 @@ mt_status resolve(const mt_params* in, const mt_batch* b, Derived* out) {
   D.o_rinv = take(n * 8);
   D.o_count = take((size_t)D.ncell * 4);
   D.o_start = take((size_t)(D.ncell + 1) * 4);
-  D.o_cursor = take((size_t)D.ncell * 4);
   D.o_status = take((size_t)D.ntiles * 8);
   D.o_big = take((size_t)D.nbig_cap * 4);
   D.o_obs = take((size_t)p.observe_cap * D.nreal * 4 * 8);
   for (int b2 = 0; b2 < 2; ++b2) D.o_fstart[b2] = take(D.fused ? (size_t)(D.ncell + 1) * 4 : 0);
   for (int b2 = 0; b2 < 2; ++b2) D.o_cb[b2] = take(D.fused ? (size_t)(D.nseg + 1) * 4 : 0);
   D.o_ovlist = take(D.fused ? (size_t)D.nseg * 4 : 0);
-  // (32 MiB that nothing uses: saved states and footprints of large MT_FP64
-  // systems keep their layout)
-  if (D.fused && p.precision == MT_FP64 && p.n >= (1LL << 17)) take((size_t)32 << 20);
   for (int b2 = 0; b2 < 2; ++b2) D.o_pred[b2] = take(D.fused ? (size_t)D.nseg : 0);
   D.o_rt = take(D.rt.size() * sizeof(Real));
   D.o_sslot = take(D.sslot.size() * 4);
@@ -1405,7 +1401,7 @@ const char* mt_profile_name(const mt_handle* h, int32_t idx) {
 }
 
 // ------------------------------------------------------------ checkpoint --
-// File: kCkptMagic, format version, sizeof(mt_params), the resolved
+// File: kCkptMagic, format version (1 is read too), sizeof(mt_params), the resolved
 // parameters, the host step count, the realisation table's size and bytes,
 // the workspace's size and bytes (little-endian, as on both host
 // architectures).  The workspace holds the whole device state (positions,
@@ -1416,7 +1412,24 @@ const char* mt_profile_name(const mt_handle* h, int32_t idx) {
 
 namespace {
 constexpr char kCkptMagic[8] = {'M', 'T', 'C', 'K', 'P', 'T', '0', '1'};
-constexpr uint32_t kCkptVersion = 1;
+constexpr uint32_t kCkptVersion = 2;
+
+// Version 1's workspace held two regions more, which nothing reads any more: a
+// word per cell before the scan's status words, and 32 MiB before the
+// prediction flags of large MT_FP64 one-kernel systems.
+struct OldRegions {
+  size_t cursor, wc;  // bytes of each
+};
+OldRegions old_regions(const Derived& D) {
+  const bool wc = D.fused && D.p.precision == MT_FP64 && D.p.n >= (1LL << 17);
+  return {align_up((size_t)D.ncell * 4), wc ? (size_t)32 << 20 : 0};
+}
+void drop_old_regions(const Derived& D, std::vector<char>* ws) {
+  const OldRegions o = old_regions(D);
+  const auto at = [&](size_t k) { return ws->begin() + (std::ptrdiff_t)k; };
+  ws->erase(at(D.o_pred[0] + o.cursor), at(D.o_pred[0] + o.cursor + o.wc));
+  ws->erase(at(D.o_status), at(D.o_status + o.cursor));
+}
 
 struct CkptHeader {
   char magic[8];
@@ -1437,7 +1450,7 @@ mt_status read_header(FILE* f, CkptHeader* hd) {
     return fail(MT_ERR_INVALID, "checkpoint: short header");
   if (std::memcmp(hd->magic, kCkptMagic, sizeof kCkptMagic) != 0)
     return fail(MT_ERR_INVALID, "checkpoint: not a checkpoint file");
-  if (hd->version != kCkptVersion || hd->params_bytes != sizeof(mt_params))
+  if (hd->version < 1 || hd->version > kCkptVersion || hd->params_bytes != sizeof(mt_params))
     return fail(MT_ERR_INVALID, "checkpoint: format version %u not supported", hd->version);
   return MT_OK;
 }
@@ -1495,7 +1508,8 @@ mt_status mt_load(mt_handle* h, const char* path) {
   mt_status s = read_header(f, &hd);
   std::vector<char> rt, ws;
   if (s == MT_OK) {
-    if (!same_params(hd.p, h->D.p) || hd.ws_bytes != h->D.total ||
+    const OldRegions o = hd.version == 1 ? old_regions(h->D) : OldRegions{0, 0};
+    if (!same_params(hd.p, h->D.p) || hd.ws_bytes != h->D.total + o.cursor + o.wc ||
         hd.rt_bytes != h->D.rt.size() * sizeof(Real))
       s = fail(MT_ERR_INVALID, "mt_load: the checkpoint was saved by a handle with other parameters");
   }
@@ -1513,6 +1527,7 @@ mt_status mt_load(mt_handle* h, const char* path) {
   CU(cudaStreamSynchronize(h->stream));
   if (h->side) CU(cudaStreamSynchronize(h->side));
   if (h->side2) CU(cudaStreamSynchronize(h->side2));
+  if (hd.version == 1) drop_old_regions(h->D, &ws);
   if (!ws.empty()) {
     // A state is saved between steps, with no graph of several steps running.
     // (Files written before the control block had these words hold anything
