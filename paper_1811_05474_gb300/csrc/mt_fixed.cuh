@@ -19,14 +19,14 @@
 //   A row of c terms without a marked mass: its sum is off by less than
 // c 2^-29 u, its new mass M' = M + sum / 2 by half of that; its nonzero masses
 // are at least 2^44 u.
-//   A row with one: the marks make the sum wrong by less than 2 sum_j P u, M'
-// by sum_j P u ~ u.
-//   In the first tier a row with a marked mass is summed in binary64; without
-// one, M' is zero or at least 2^43 u P, P the largest of its nonzero neighbours'
-// (2^-20 at the least there), and off by c 2^-73 / P of itself.  In the dense
-// tiles a row is if its M' does not outweigh the error by 2^53 (FixAcc::keeps: u or,
-// with 2^20 terms, 2^-10 u).  So a sum that is kept costs M' no more than about
-// one rounding more.
+//   A row with one: the marks would make the sum wrong by up to 2 sum_j P u.  In
+// the first tier such a row is summed in binary64 (without one, M' is zero or at
+// least 2^43 u P, P the largest of its nonzero neighbours', 2^-20 at the least
+// there, and off by c 2^-73 / P of itself).  In the dense tiles the marked masses'
+// rests (fix_rest) are summed beside it in binary32: of 512 terms, a chunk, within
+// 2^9 2^-24 sum_j P u, so M' is off by 2^-15 u, and a row whose M' is not at least
+// 2^38 u (FixAcc::keeps) is summed in binary64.  So a sum that is kept costs M' no
+// more than about one rounding more.
 //   Everything is summed in binary64 when E is out of range (infinities, NaNs,
 // masses near the ends of binary64's range), where weights fall below e^-6.9
 // (cutoffs far beyond the kernel's width) and in systems that hold a
@@ -60,6 +60,23 @@ __device__ __forceinline__ long long to_fix(unsigned long long bits, int E) {
   return (long long)bits < 0 ? -(long long)v : (long long)v;
 }
 
+// What a marked mass is off by, M / u - to_fix (between -1 and 1; binary32).
+__device__ __forceinline__ float fix_rest(unsigned long long bits, int E) {
+  const int e = fix_exponent(bits);
+  const unsigned long long m =
+      ((bits & ((1ULL << 52) - 1)) | ((unsigned long long)(e != 0) << 52)) << 8;
+  const int sh = E - (e != 0 ? e : 1);
+  if (sh <= 7 || m == 0) return 0.0f;
+  const unsigned long long v = m >> (sh < 63 ? sh : 63);
+  float f = 0.0f;  // the bits below u
+  if (sh < 64)
+    f = __uint2float_rn((unsigned int)(m << (64 - sh) >> 32)) * 0x1p-32f;
+  else if (sh < 150)
+    f = __uint2float_rn((unsigned int)(m >> 32)) * __int_as_float((159 - sh) << 23);
+  if ((v & 1) == 0 && (sh > 16 || (v << sh) != m)) f -= 1.0f;
+  return (long long)bits < 0 ? -f : f;
+}
+
 // 1: marked, 2: negative.
 __device__ __forceinline__ int fix_flags(long long v) {
   return (int)(v & 1) | (v < 0 ? 2 : 0);
@@ -90,16 +107,25 @@ struct FixAcc {
         : "+r"(a0), "+r"(a1), "+r"(a2)
         : "r"(y0), "r"(y1), "r"(y2));
   }
-  // Whether the sum is kept: the new mass it gives, M' = mass + sum / 2^halvings,
-  // outweighs the error of a row with (flags & 1) or without marked masses; or
-  // both are zero, which without marked or negative masses, or (one: a P times
-  // u is at least one unit of the sum) without negative ones, says that every
-  // mass of the row is.  In units of 8 u, by integers: two binary64
-  // instructions per chunk and species made the dense step 1.4 % slower.
+  // Adds a binary32 sum of P times rests (fix_rest), in units of u.
+  __device__ __forceinline__ void add_rest(float rest) {
+    const long long r = __float2ll_rn(rest * 0x1p29f);
+    const unsigned int x0 = (unsigned int)r, x1 = (unsigned int)(r >> 32);
+    const unsigned int x2 = (unsigned int)(r >> 63);
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(a0), "+r"(a1), "+r"(a2)
+        : "r"(x0), "r"(x1), "r"(x2));
+  }
+  // Whether the sum of up to 512 terms and their rests is kept: the new mass it
+  // gives, M' = mass + sum / 2^halvings, is at least 2^38 u; or both are zero,
+  // which without marked or negative masses, or (one: a P times u is at least one
+  // unit of the sum) without negative ones, says that every mass of the row is.
+  // In units of 8 u, by integers: two binary64 instructions per chunk and species
+  // made the dense step 1.4 % slower.
   __device__ __forceinline__ bool keeps(long long mass, int halvings, int flags, bool one) const {
     const long long next =
         (mass >> 3) + ((long long)((unsigned long long)a2 << 32 | a1) >> halvings);
-    if (((next ^ (next >> 63)) >> (flags & 1 ? 50 : 40)) != 0) return true;
+    if (((next ^ (next >> 63)) >> 35) != 0) return true;
     return (mass | a0 | a1 | a2) == 0 && (flags == 0 || (flags == 1 && one));
   }
   // The sum in binary64 (rounded to nearest even), masses in units of

@@ -501,21 +501,22 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile(Dev d, int sp) {
 // pair at the paper's density); here a pair is ~55 integer and binary32
 // instructions, issue-bound.  Each chunk's masses, and the rows' own, are
 // converted with the largest exponent among them, and a chunk's sum is rounded
-// to binary64 once.  A lane whose sum does not outweigh its error (FixAcc::keeps; the
-// marks of the whole chunk count) sums the chunk again, in binary64, which holds
-// the binary64 pipe of the multiprocessor a front lies on: a species at a time,
-// since in the tail of one the other is large (27 realisations of 5000, two
-// segregated components, eighth step: 309 us with both, 196 so; unrolled four
-// times 188, but 0.6 % more for the systems that have no such row).  N = 10^6 at
-// 200 per unit length: 4.09 -> 1.10 ms (step 4.47 -> 1.43 ms).
+// to binary64 once.  Where the chunk, or a row, has marked masses, their rests are
+// summed too, in binary32 (six instructions more).  A lane whose sum still does
+// not outweigh its error (FixAcc::keeps: deep in a front's tail) sums the chunk
+// again, in binary64, a species at a time.  N = 10^6 at 200 per unit length: 4.09 ->
+// 1.09 ms (step 4.47 -> 1.42 ms); 27 realisations of 5000, two segregated
+// components, eighth step: 162 us (without rests, rows of small masses in
+// binary64: 196).
 template <bool TR>
-__global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
+__global__ void __launch_bounds__(kThreads, 4) k_exchange_tile_fix(Dev d, int sp) {
   chained();
   using W = Weight<true, 1>;
   using MS = Mass<MT_MIXED>;
   constexpr int kWarps = kThreads / 32, kPer = kTileChunk / kThreads;
   __shared__ uint2 s_xr[kTileChunk];       // low word of the position, 1 / r
   __shared__ longlong2 s_ab[kTileChunk];   // fixed masses
+  __shared__ float2 s_rest[kTileChunk];    // their rests, where the chunk has marked masses
   __shared__ long long s_lohi[2];
   __shared__ int s_e[kWarps][2];  // largest exponents
   __shared__ int s_mark[2];       // fix_flags of the chunk's masses
@@ -583,23 +584,58 @@ __global__ void __launch_bounds__(kThreads) k_exchange_tile_fix(Dev d, int sp) {
         if (mb) atomicOr(&s_mark[1], mb);
       }
     }
-    __syncthreads();
+    const long long fa = to_fix(Ab, EA), fb = to_fix(Bb, EB);
+    // (every lane stages the rests if any has a marked mass: its own may lie in
+    // another chunk)
+    const bool rests = __syncthreads_or(((s_mark[0] | s_mark[1]) & 1) || ((fa | fb) & 1));
+    if (rests) {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int i = threadIdx.x + k * kThreads;
+        s_rest[i] = i < nc ? make_float2(fix_rest(MA[c0 + i], EA), fix_rest(MB[c0 + i], EB))
+                           : make_float2(0.0f, 0.0f);
+      }
+      __syncthreads();
+    }
     const int j0 = (int)(max(t.wlo, c0) - c0), j1 = (int)(min(t.whi, c0 + nc) - c0);
     const int ql = (int)(jl - c0);
     const unsigned int qn = (unsigned int)(jr - jl);
-    const long long fa = to_fix(Ab, EA), fb = to_fix(Bb, EB);
     // this lane's slots of the chunk
     const int l0 = (int)(max(jl, c0) - c0), l1 = (int)(min(jr, c0 + nc) - c0);
     FixAcc qa, qb;
+    if (!rests) {
 #pragma unroll 2
-    for (int j = j0; j < j1; ++j) {
-      const uint2 xr = s_xr[j];
-      const longlong2 ab = s_ab[j];
-      const float w = W::near(d, (int)(xr.x - x32), nullptr);
-      FixP P = fix_p(w * (ip + __uint_as_float(xr.y)));
-      if ((unsigned int)(j - ql) >= qn) P.p = 0;
-      qa.add(ab.x - fa, P);
-      qb.add(ab.y - fb, P);
+      for (int j = j0; j < j1; ++j) {
+        const uint2 xr = s_xr[j];
+        const longlong2 ab = s_ab[j];
+        const float w = W::near(d, (int)(xr.x - x32), nullptr);
+        FixP P = fix_p(w * (ip + __uint_as_float(xr.y)));
+        if ((unsigned int)(j - ql) >= qn) P.p = 0;
+        qa.add(ab.x - fa, P);
+        qb.add(ab.y - fb, P);
+      }
+    } else {
+      const float ra = fix_rest(Ab, EA), rb = fix_rest(Bb, EB);
+      float sa = 0.0f, sb = 0.0f;
+#pragma unroll 2
+      for (int j = j0; j < j1; ++j) {
+        const uint2 xr = s_xr[j];
+        const longlong2 ab = s_ab[j];
+        const float2 rest = s_rest[j];
+        const float w = W::near(d, (int)(xr.x - x32), nullptr);
+        float Pf = w * (ip + __uint_as_float(xr.y));
+        FixP P = fix_p(Pf);
+        if ((unsigned int)(j - ql) >= qn) {
+          P.p = 0;
+          Pf = 0.0f;
+        }
+        qa.add(ab.x - fa, P);
+        qb.add(ab.y - fb, P);
+        sa = __fmaf_rn(Pf, rest.x - ra, sa);
+        sb = __fmaf_rn(Pf, rest.y - rb, sb);
+      }
+      qa.add_rest(sa);
+      qb.add_rest(sb);
     }
     if (l0 < l1) {
       // (halved in the exponent, which is far from binary64's ends)

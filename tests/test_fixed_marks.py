@@ -23,14 +23,46 @@ def to_fix(b, E):
     return -v if b >> 63 else v
 
 
+def fix_rest(b, E):
+    e = exponent(b)
+    m = ((b & (2 ** 52 - 1)) | ((1 if e else 0) << 52)) << 8
+    sh = E - (e if e else 1)
+    if sh <= 7 or not m:
+        return np.float32(0.0)
+    v, f = m >> min(sh, 63), np.float32(0.0)
+    if sh < 64:
+        f = np.float32(m << (64 - sh) >> 32 & 0xFFFFFFFF) * np.float32(2.0 ** -32)
+    elif sh < 150:
+        f = np.float32(m >> 32) * np.float32(2.0 ** (32 - sh))
+    if not v & 1 and (sh > 16 or v << sh != m):
+        f -= np.float32(1.0)
+    return -f if b >> 63 else f
+
+
+@pytest.mark.parametrize("E", [1023, 1400])
+def test_rests(E):
+    """A mass is its integer and its rest, to 2^-24 of the unit."""
+    rng = random.Random(2)
+    u = Fraction(2) ** (E - 1083)
+    for _ in range(4000):
+        x = math.ldexp(rng.choice([rng.random(), rng.randrange(1, 64) / 64.0]),
+                       E - 1022 - rng.randrange(0, 100)) * rng.choice([1, -1])
+        b = bits(x)
+        if exponent(b) > E:
+            continue
+        rest = fix_rest(b, E)
+        assert abs(rest) <= 1.0
+        assert abs(Fraction(x) / u - to_fix(b, E) - Fraction(float(rest))) <= Fraction(2) ** -24
+
+
 @pytest.mark.parametrize("kind", ["edge", "decades", "signed", "clean", "smooth", "zeros"])
 def test_kept_rows_are_as_exact_as_one_rounding(kind):
     """Rows of up to 200 neighbours with a large mass at the cutoff's edge, with
     masses over 30 decades, of both signs, with few significant bits, and nearly
-    equal ones: where the integer sum is kept, the new mass M' is within its
-    marks' error (sum of P <= 1: 2^-53 M') and the terms' (2^-30 of a unit each),
-    which together are at most 2^-53 M' (1 + 2^-10), and the sum's and the update's
-    rounding (2^-53 each of |M'| and the sum)."""
+    equal ones: where the integer sum is kept, the new mass M' is within its rests'
+    error (2^-15 of a unit for up to 512 terms) and the terms' (2^-30 of one each),
+    together at most 2^-53 M' (1 + 2^-5), and the sum's and the update's rounding
+    (2^-53 each of |M'| and the sum)."""
     rng = random.Random(7)
     kept = 0
     for _ in range(400):
@@ -55,20 +87,22 @@ def test_kept_rows_are_as_exact_as_one_rounding(kind):
         top = 1.0 if rng.random() < 0.5 else max(abs(m) for m in M)  # another staged mass
         E = exponent(bits(max(top, max(abs(m) for m in M)))) or 1023
         f = [to_fix(bits(m), E) for m in M]
-        acc = 0
+        rest = [fix_rest(bits(m), E) for m in M]
+        acc, sum_rest = 0, np.float32(0.0)
         for i in range(c):
             p, s = fix_p(P[i])
             acc = wrap96(acc + ((f[i + 1] - f[0]) * p >> s))
+            sum_rest = np.float32(P[i] * float(rest[i + 1] - rest[0]) + float(sum_rest))
+        acc = wrap96(acc + round(float(sum_rest) * 2.0 ** 29))
         exact = sum(Fraction(P[i]) * (Fraction(M[i + 1]) - Fraction(M[0])) for i in range(c))
         total = value(acc, E)
         new = M[0] + 0.5 * total
-        marked = any(v & 1 for v in f)
         size = abs((f[0] >> 3) + (acc >> 33))  # |M'| in units of 8 u
         zero = f[0] == 0 and acc == 0 and min(f) >= 0  # (P is at least 2^-18 here)
-        if size < 2 ** (50 if marked else 40) and not zero:
+        if size < 2 ** 35 and not zero:
             continue  # summed in binary64
         kept += 1
-        bound = Fraction(2) ** -53 * (2 * abs(Fraction(new)) + abs(exact)) * Fraction(1001, 1000)
+        bound = Fraction(2) ** -53 * (2 * abs(Fraction(new)) + abs(exact)) * Fraction(33, 32)
         assert abs(Fraction(new) - (Fraction(M[0]) + exact / 2)) <= bound
     assert kept > 20
 
