@@ -721,10 +721,11 @@ __device__ __forceinline__ long long walk_left(const Dev& d, const Ring& g, long
   return d.periodic ? g.n - 1 : p;
 }
 
-// Tick distance from slot q up to slot p (p to the right of q).
-__device__ __forceinline__ long long gap(const Dev& d, const Ring& g, const long long* Xs,
-                                         long long q, long long p) {
-  return d.periodic ? ring_gap(g, q, Xs[q], p, Xs[p]) : Xs[p] - Xs[q];
+// Tick distance from slot q up to slot p (p to the right of q; reflecting walls:
+// a higher slot).
+__device__ __forceinline__ long long gap(const Ring& g, const long long* Xs, long long q,
+                                         long long p) {
+  return ring_gap(g, q, Xs[q], p, Xs[p]);
 }
 
 template <int PR>
@@ -745,7 +746,7 @@ __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
   long long k = 1;
   const long long kr = walk_right(d, g, p);
   for (; k <= kr; ++k) {
-    const long long D = gap(d, g, Xs, p, ring(d, g, p, k));
+    const long long D = gap(g, Xs, p, ring(d, g, p, k));
     if (D > d.S) break;
     const T w = W::near(d, D, s_tab);
     if (k <= d.band_cap) band[band_at(d, p, k)] = w;
@@ -754,7 +755,7 @@ __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
   d.cnt[p] = (int)(k - 1);
   const long long kl = walk_left(d, g, p);
   for (k = 1; k <= kl; ++k)
-    if (gap(d, g, Xs, ring(d, g, p, -k), p) > d.S) break;
+    if (gap(g, Xs, ring(d, g, p, -k), p) > d.S) break;
   d.cnt[d.n + p] = (int)(k - 1);
   static_cast<T*>(d.rinv)[p] = r.value();  // right part of r_p, completed by band_rowsum
   d.id[xc ^ 1][p] = d.id[xc][s];
@@ -781,7 +782,7 @@ __global__ void __launch_bounds__(kThreads) k_band_rowsum(Dev d) {
   for (int k = 1; k <= kb; ++k) r.add(band[band_at(d, ring(d, g, p, -k), k)]);
   if (kl > kb) {
     const long long* Xs = d.X[xc ^ 1];
-    for (int k = kb + 1; k <= kl; ++k) r.add(W::near(d, gap(d, g, Xs, ring(d, g, p, -k), p), s_tab));
+    for (int k = kb + 1; k <= kl; ++k) r.add(W::near(d, gap(g, Xs, ring(d, g, p, -k), p), s_tab));
   }
   store_rinv<mixw(PR)>(d, p, r.value());
 }
@@ -825,13 +826,13 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
     }
     for (int k = bl + 1; k <= kl; ++k) {
       const long long q = ring(d, g, p, -k);
-      pair(q, W::near(d, gap(d, g, Xs, q, p), s_tab));
+      pair(q, W::near(d, gap(g, Xs, q, p), s_tab));
     }
 #pragma unroll 2
     for (int k = 1; k <= br; ++k) pair(ring(d, g, p, k), band[band_at(d, p, k)]);
     for (int k = br + 1; k <= kr; ++k) {
       const long long q = ring(d, g, p, k);
-      pair(q, W::near(d, gap(d, g, Xs, p, q), s_tab));
+      pair(q, W::near(d, gap(g, Xs, p, q), s_tab));
     }
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
