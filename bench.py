@@ -122,7 +122,7 @@ def parse():
     ap.add_argument("--ncu", action="store_true",
                     help="profiling mode: upload, W graph steps, then K direct steps, nothing else")
     ap.add_argument("--n", type=int, default=N, help="particles (profiling mode only)")
-    ap.add_argument("--ncu-search", default="cell", choices=["cell", "full", "dense", "dense_spam"],
+    ap.add_argument("--ncu-search", default="cell", choices=["cell", "cell2d", "full", "full50", "dense", "dense_spam"],
                     help="profiling mode: the cell list (headline), the full matrix, or the "
                          "paper's density on the fly or in the SPaM form")
     ap.add_argument("--no-batch", action="store_true", help="skip the batched-ensemble object")
@@ -720,10 +720,11 @@ def species_run(local: int, steps: int = 50, counts=(2, 3, 4, 6, 8)):
 
 def brute_run(local: int, n: int = 100000, steps: int = 2, sm_mhz: float | None = None):
     """The all-pairs forms at the N = 1e5 workload's shape (1-d, [0, 1e5],
-    MIXED): the full matrix (every pair whose weight does not underflow, the
-    paper's reference) and the cutoff brute force (every pair tested).  Per
-    pass: kernel time, pairs per second, and for the full matrix the pairs
-    tested per second against the issue rate."""
+    MIXED): the full matrix (the paper's reference) and the cutoff brute force.
+    Both test every ordered pair's separation, in each of the two passes, and
+    evaluate the weights of the pairs that can have one (no cutoff: that do not
+    underflow).  Per pass: kernel time, and for the full matrix the pairs tested
+    per second against the issue rate."""
     import torch
 
     from paper_1811_05474_gb300 import mt, synth
@@ -755,12 +756,10 @@ def brute_run(local: int, n: int = 100000, steps: int = 2, sm_mhz: float | None 
         pairs = float(n) * n
         rk, xk = ("rowsum_full", "exchange_full") if search == mt.MT_SEARCH_FULL else \
                  ("rowsum_brute", "exchange_brute")
-        r = {"ms_per_step": ms, "pair_evaluations_per_step": 2 * pairs,
-             "pairs_per_s": 2 * pairs / (ms * 1e-3),
+        r = {"ms_per_step": ms, "pair_tests_per_step": 2 * pairs,
+             "pair_tests_per_s": 2 * pairs / (ms * 1e-3),
              "rowsum_ms": prof.get(rk), "exchange_ms": prof.get(xk)}
         if search == mt.MT_SEARCH_FULL:
-            # each ordered pair's separation is tested once in each pass; only pairs whose
-            # weight does not underflow to zero are evaluated
             for key, k in (("rowsum_roofline", rk), ("exchange_roofline", xk)):
                 rate = pairs / (prof[k] * 1e-3)
                 r[key] = {"bound": "issue", "achieved": rate, "peak": peak, "unit": "pairs tested/s",
@@ -890,11 +889,12 @@ def workloads_run(local: int, flush_l2):
     """The two smaller workloads, timed like the headline (graph steps,
     events on the simulation's stream, L2 flushed between steps).
     N = 1e3 uniform on [0, 1e3], 100 steps, binary64: the cell list, the
-    cutoff brute force (every pair tested) and the full matrix (every
-    pair's weight, the paper's reference).  N = 1e5 uniform on [0, 1e5],
-    1000 steps, no advection: binary64, MIXED and double-binary32.
-    pair-interactions/s counts the unordered pairs within the cutoff (the
-    full matrix: every unordered pair it evaluates, labelled as such)."""
+    cutoff brute force and the full matrix (the paper's reference); the last
+    two test every pair.  N = 1e5 uniform on [0, 1e5], 1000 steps, no
+    advection: binary64, MIXED and double-binary32.  pair-interactions/s counts
+    the unordered pairs within the cutoff in every form (the same pairs: the
+    walk is the same); pair_tests_per_s the ordered pairs whose separation the
+    all-pairs forms test."""
     import torch
 
     from paper_1811_05474_gb300 import mt, synth
@@ -912,14 +912,15 @@ def workloads_run(local: int, flush_l2):
         sim = mt.Simulation(p, device=dev)
         sim.upload(x1, A1, B1)
         ms = timed_steps(sim, steps1, 3, flush_l2)
-        if search == mt.MT_SEARCH_FULL:
-            pairs, label = n1 * (n1 - 1) // 2, "all unordered pairs (evaluated)"
-        else:
-            pairs, label = mt.mt_read_pairs(sim.h, None, None, 0), "unordered pairs within the cutoff"
+        if search != mt.MT_SEARCH_FULL:  # (the full matrix: those of the last form)
+            pairs = mt.mt_read_pairs(sim.h, None, None, 0)
         sim.close()
         w1[name] = {"value": n1 * steps1 / (ms * 1e-3), "unit": "particle-steps/s",
-                    "ms_per_step": ms / steps1, "pairs_per_step": int(pairs), "pairs": label,
+                    "ms_per_step": ms / steps1, "pairs_per_step": int(pairs),
+                    "pairs": "unordered pairs within the cutoff",
                     "pair_interactions_per_s": pairs * steps1 / (ms * 1e-3)}
+        if search != mt.MT_SEARCH_CELL:
+            w1[name]["pair_tests_per_s"] = 2.0 * n1 * n1 * steps1 / (ms * 1e-3)
     out["n1e3"] = w1
     n2, steps2 = 10 ** 5, 1000
     x2 = synth.uniform_positions(n2, 1e5, seed=0)
@@ -1080,9 +1081,15 @@ def run_ncu(args):
         x = synth.uniform_positions(n, Ln, seed=9)
         sim = mt.Simulation(p)
         sim.upload(x, *synth.segregated_masses(x, Ln))
+    elif args.ncu_search == "cell2d":
+        Ln = 10.0 * float(n) ** 0.5
+        sim = mt.Simulation(mt.mt_params_init(dim=2, n=n, L=(Ln, Ln), D_mt=D, D_rw=D, dt=DT,
+                                              precision=prec, seed=2024))
+        sim.upload(synth.uniform_positions(n, Ln, dim=2, seed=0), *synth.uniform_masses(n, seed=0))
     else:
-        Ln = float(n) * (L / N)
-        search = mt.MT_SEARCH_FULL if args.ncu_search == "full" else mt.MT_SEARCH_CELL
+        # full50: the full matrix on the paper's 50 units, where much of it is nonzero
+        Ln = 50.0 if args.ncu_search == "full50" else float(n) * (L / N)
+        search = (mt.MT_SEARCH_FULL if args.ncu_search.startswith("full") else mt.MT_SEARCH_CELL)
         p = mt.mt_params_init(n=n, L=(Ln,), v=(V, 0.0), D_mt=D, D_rw=D, dt=DT, precision=prec,
                               search=search, seed=2024, observe_cap=args.steps + args.warmup)
         sim = mt.Simulation(p)
@@ -1104,16 +1111,14 @@ def compact_kernels(kernels):
 
 
 def fp64_ops_per_step(npairs: int, n: int) -> float:
-    """Binary64 pipe instructions (per lane) the step needs with binary64
-    masses (MIXED and FP64), the unit of the measured FMA rate: per ordered
-    pair within the cutoff and species, the difference M_j - M_i and one
-    fused multiply-add of it with P into the accumulator (2 x 2 species x 2
-    orders per unordered pair); per particle and species the update (one
-    fused multiply-add), per particle the reaction (a comparison and one
-    subtraction: the smaller mass becomes exactly 0) and the walk's product
-    (1).  MIXED's first tier forms the flux terms in exact integer
-    arithmetic instead, off this pipe: its fraction says how the step compares
-    with the binary64 form, not how busy the pipe is."""
+    """Binary64 pipe instructions (per lane) that MT_FP64's transfer issues,
+    the unit of the measured FMA rate: per ordered pair within the cutoff and
+    species, the difference M_j - M_i and one fused multiply-add of it with P
+    into the accumulator (2 x 2 species x 2 orders per unordered pair); per
+    particle and species the update (one fused multiply-add), per particle the
+    reaction (a comparison and one subtraction: the smaller mass becomes exactly
+    0) and the walk's product (1).  Its weights are integer arithmetic; so are
+    MIXED's flux terms, whose first tier this does not describe."""
     return 8.0 * npairs + 5.0 * n
 
 
@@ -1146,13 +1151,10 @@ def state_kernel(kernels):
     return max(kernels, key=lambda k: k["ms_per_step"])
 
 
-def variant_object(r, steps: int, name: str, peak: float, peak_kind: str, clocks, exp_peak,
-                   dfma_peak=None):
+def variant_object(r, steps: int, name: str, peak: float, peak_kind: str, clocks, dfma_peak=None):
     """A precision's own result on the headline workload: rate, its
-    state kernel against HBM (48 B per particle-step) and, with binary64
-    weights, the transfer phase against the measured binary64 exponential
-    rate (one exponential per unordered pair within the cutoff, the method's
-    minimum)."""
+    state kernel against HBM (48 B per particle-step) and, in MT_FP64, the
+    transfer phase against the measured binary64 rate."""
     dom = state_kernel(r["kernels"])
     achieved = ALGO_BYTES.get(dom["name"], 48) * N / (dom["ms"] * 1e-3) / 1e9
     obj = {"value": N * steps / (r["total_ms"] * 1e-3), "unit": "particle-steps/s",
@@ -1163,17 +1165,8 @@ def variant_object(r, steps: int, name: str, peak: float, peak_kind: str, clocks
                         "algo_bytes_per_launch": ALGO_BYTES.get(dom["name"], 48) * N,
                         "traffic": load_traffic(dom["name"] + ("" if name == "mixed" else "_" + name))},
            "clocks": clocks, "kernels": compact_kernels(r["kernels"])}
-    if name in ("fp64", "mixed") and dfma_peak:
+    if name == "fp64" and dfma_peak:
         obj["alu_roofline"] = alu_roofline(r, N, dfma_peak)
-    if name == "fp64" and exp_peak and r.get("phase_ms"):
-        rate = r["npairs"] / (r["phase_ms"] * 1e-3)
-        obj["exp_roofline"] = {"bound": "alu", "kernel": "fused_step || fused_pred (concurrent)",
-                               "achieved": rate,
-                               "peak": exp_peak, "unit": "binary64 exp/s", "frac": rate / exp_peak,
-                               "peak_kind": "measured (mt_probe_rate: a binary64 "
-                                            "exp(-t), exp_neg; the step forms its "
-                                            "weights in integer arithmetic)",
-                               "algo": "one exponential per unordered pair within the cutoff"}
     return obj
 
 
@@ -1279,23 +1272,22 @@ def main():
     achieved = dom_bytes / (dom["ms"] * 1e-3) / 1e9 if dom["ms"] > 0 else 0.0
     step_bytes = ALGO_BYTES["step"] * N
     path_achieved = step_bytes / (ms_step * 1e-3) / 1e9
-    exp_peak = probes["binary64_exp_neg_per_s"] if probes else None
     dfma_peak = probes["binary64_fma_per_s"] if probes else None
     objs = {name: variant_object(r, k, name, peak, peak_kind,
-                                 sampler.summary(r["t0"], r["t1"]), exp_peak, dfma_peak)
+                                 sampler.summary(r["t0"], r["t1"]), dfma_peak)
             for name, (r, k) in variants.items()}
     cpu = None
     if ws == 1 and not args.no_cpu:
         cpu = cpu_baselines()
     traffic_key = dom["name"] + ("" if args.precision == "mixed" else "_" + args.precision)
-    # the headline kernel's roofline: binary64 masses make the transfer
-    # binary64-bound on this GPU (MIXED and FP64); the double-binary32 form
-    # is compared with HBM
+    # the headline kernel's roofline: MT_FP64's transfer against the binary64
+    # pipe, the other precisions' first tier against HBM (issue_roofline: its
+    # warp instructions against the issue slots)
     hbm_roofline = {"bound": "hbm", "kernel": dom["name"], "achieved": achieved, "peak": peak,
                     "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
                     "algo_bytes_per_launch": dom_bytes, "traffic": load_traffic(traffic_key)}
     roofline = hbm_roofline
-    if args.precision in ("mixed", "fp64") and dfma_peak:
+    if args.precision == "fp64" and dfma_peak:
         alu = alu_roofline(main_run, N, dfma_peak)
         if alu:
             alu["traffic"] = hbm_roofline["traffic"]

@@ -342,7 +342,7 @@ mt_status mt_set_noise(mt_handle* h, const float* xi_device);
 mt_status mt_step(mt_handle* h);
 
 /* Enqueue nsteps time steps.  With the built-in generator the steps are
- * replayed from CUDA graphs.  A graph is captured (0.1 to 1 ms of host work)
+ * replayed from CUDA graphs.  A graph is captured (about 0.1 ms of host work)
  * by the first call that needs it: one of a single step or, in the 1-d
  * one-kernel step of systems below a wave of segments whose binary64 masses
  * are not observed, one of 12 steps for the multiples of 12 and one of a
