@@ -727,6 +727,13 @@ __device__ __forceinline__ long long gap(const Ring& g, const long long* Xs, lon
                                          long long p) {
   return ring_gap(g, q, Xs[q], p, Xs[p]);
 }
+// The same where it is rare (weights past the band): a call, so that the
+// exchange's own loops keep their registers (MT_MIXED_DF32, 1.9 10^5 particles at 116
+// per unit length: 581 -> 491 us per step, five species 1394 -> 982).
+__device__ __noinline__ long long gap_past(long long Lq, const long long* Xs, long long q,
+                                           long long p) {
+  return Xs[p] - Xs[q] + (p < q ? Lq : 0);
+}
 
 template <int PR>
 __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
@@ -826,13 +833,13 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
     }
     for (int k = bl + 1; k <= kl; ++k) {
       const long long q = ring(d, g, p, -k);
-      pair(q, W::near(d, gap(g, Xs, q, p), s_tab));
+      pair(q, W::near(d, gap_past(g.Lq, Xs, q, p), s_tab));
     }
 #pragma unroll 2
     for (int k = 1; k <= br; ++k) pair(ring(d, g, p, k), band[band_at(d, p, k)]);
     for (int k = br + 1; k <= kr; ++k) {
       const long long q = ring(d, g, p, k);
-      pair(q, W::near(d, gap(g, Xs, p, q), s_tab));
+      pair(q, W::near(d, gap_past(g.Lq, Xs, p, q), s_tab));
     }
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
