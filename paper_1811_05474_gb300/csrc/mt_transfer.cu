@@ -871,8 +871,9 @@ constexpr int kNone = -1, kMany = -2;
 // is tested, since a warp with many candidates (a pile) waits for them: 10^4
 // particles, most in a few cells, MT_MIXED 1057 -> 873 us per step (with the three
 // runs' loops before: 931), and 30000 at one per unit of area 58 -> 54;
-// MT_MIXED_DF32's exchange, which has no registers left for it, does without (10^6
-// at one per unit of area: 293 against 282 us).
+// MT_MIXED_DF32's exchange and MT_MIXED's of further species, which have no
+// registers left for it, do without (DF32, 10^6 at one per unit of area: 293 against
+// 282 us).
 template <bool PER, bool AHEAD, class F, class G>
 __device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, int p, long long x,
                                             long long y, F&& f, G&& self) {
@@ -915,24 +916,23 @@ __device__ __forceinline__ void cell2_visit(const Dev& d, const long long* Xs, i
   const unsigned int S2 = 2u * (unsigned int)d.S;
   const long long* Ys = Xs + d.n;
   auto slot = [&](int t) { return t + (t < n0 ? a[0] : t < n1 ? o1 : o2); };
-  int next = n2 > 0 ? slot(0) : 0;
-  long long xn = n2 > 0 ? Xs[next] : 0, yn = n2 > 0 ? Ys[next] : 0;
+  int next = AHEAD && n2 > 0 ? slot(0) : 0;
+  long long xn = AHEAD && n2 > 0 ? Xs[next] : 0, yn = AHEAD && n2 > 0 ? Ys[next] : 0;
 #pragma unroll 2
   for (int t = 0; t < n2; ++t) {
-    if (!AHEAD) {
-      next = slot(t);
-      xn = Xs[next];
-      yn = Ys[next];
+    const int q = AHEAD ? next : slot(t);
+    if (!AHEAD && q == p) {
+      self();
+      continue;
     }
-    const int q = next;
-    const unsigned long long ux = (unsigned long long)xn - x0;
-    const unsigned long long uy = (unsigned long long)yn - y0;
+    const unsigned long long ux = (unsigned long long)(AHEAD ? xn : Xs[q]) - x0;
+    const unsigned long long uy = (unsigned long long)(AHEAD ? yn : Ys[q]) - y0;
     if (AHEAD && t + 1 < n2) {
       next = slot(t + 1);
       xn = Xs[next];
       yn = Ys[next];
     }
-    if (q == p) {
+    if (AHEAD && q == p) {
       self();
       continue;
     }
@@ -1041,7 +1041,7 @@ __global__ void __launch_bounds__(kThreads) k_exchange_cell2(Dev d, int sp) {
     }
     pair(nb, dx, dy);
   } else {
-    cell2_visit<PER, PR != MT_MIXED_DF32>(d, Xs, (int)p, x, y, pair, [] {});
+    cell2_visit<PER, !mixw(PR) || (PR == MT_MIXED && !TR)>(d, Xs, (int)p, x, y, pair, [] {});
   }
   MS::update(A, B, dA, dB, TR ? 0 : d.react);
   store(p, A, B);
