@@ -727,13 +727,6 @@ __device__ __forceinline__ long long gap(const Ring& g, const long long* Xs, lon
                                          long long p) {
   return ring_gap(g, q, Xs[q], p, Xs[p]);
 }
-// The same where it is rare (weights past the band): a call, so that the
-// exchange's own loops keep their registers (MT_MIXED_DF32, 1.9 10^5 particles at 116
-// per unit length: 581 -> 491 us per step, five species 1394 -> 982).
-__device__ __noinline__ long long gap_past(long long Lq, const long long* Xs, long long q,
-                                           long long p) {
-  return Xs[p] - Xs[q] + (p < q ? Lq : 0);
-}
 
 template <int PR>
 __global__ void __launch_bounds__(kThreads) k_band_build(Dev d) {
@@ -794,8 +787,13 @@ __global__ void __launch_bounds__(kThreads) k_band_rowsum(Dev d) {
   store_rinv<mixw(PR)>(d, p, r.value());
 }
 
+// (MT_MIXED_DF32 is compiled for five CTAs per SM: 1.9 10^5 particles at 116 per unit
+// length 575 -> 455 us per step, five species 1250 -> 876.  The wall's length is read
+// again where weights past the band need it, so that it holds no registers in
+// the loops over the band.)
 template <int PR, bool TR>
-__global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
+__global__ void __launch_bounds__(kThreads, PR == MT_MIXED_DF32 ? 5 : 0)
+    k_band_exchange(Dev d, int sp) {
   using W = Weight<mixw(PR), 1>;
   using T = typename W::T;
   using MS = Mass<PR>;
@@ -823,6 +821,7 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
       MS::acc(dA, P, MS::diff(MS::load(MA, q), A));
       MS::acc(dB, P, MS::diff(MS::load(MB, q), B));
     };
+    auto wall = [&]() -> long long { return d.periodic ? ring_of(d, d.id[xc ^ 1][p]).Lq : 0; };
     const int kl = d.cnt[d.n + p], kr = d.cnt[p];
     const int bl = kl < d.band_cap ? kl : d.band_cap;
     const int br = kr < d.band_cap ? kr : d.band_cap;
@@ -831,15 +830,21 @@ __global__ void __launch_bounds__(kThreads) k_band_exchange(Dev d, int sp) {
       const long long q = ring(d, g, p, -k);
       pair(q, band[band_at(d, q, k)]);
     }
-    for (int k = bl + 1; k <= kl; ++k) {
-      const long long q = ring(d, g, p, -k);
-      pair(q, W::near(d, gap_past(g.Lq, Xs, q, p), s_tab));
+    if (kl > bl) {
+      const long long x = Xs[p], Lq = wall();
+      for (int k = bl + 1; k <= kl; ++k) {
+        const long long q = ring(d, g, p, -k);
+        pair(q, W::near(d, x - Xs[q] + (p < q ? Lq : 0), s_tab));
+      }
     }
 #pragma unroll 2
     for (int k = 1; k <= br; ++k) pair(ring(d, g, p, k), band[band_at(d, p, k)]);
-    for (int k = br + 1; k <= kr; ++k) {
-      const long long q = ring(d, g, p, k);
-      pair(q, W::near(d, gap_past(g.Lq, Xs, p, q), s_tab));
+    if (kr > br) {
+      const long long x = Xs[p], Lq = wall();
+      for (int k = br + 1; k <= kr; ++k) {
+        const long long q = ring(d, g, p, k);
+        pair(q, W::near(d, Xs[q] - x + (q < p ? Lq : 0), s_tab));
+      }
     }
     MS::update(A, B, dA, dB, TR ? 0 : d.react);
     MS::store(d.M[mc] + sq.oa, p, A);
